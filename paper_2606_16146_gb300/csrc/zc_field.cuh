@@ -1,11 +1,11 @@
 // zc_field.cuh -- arithmetic in the BLS12-381 scalar field r on sm_103a.
 //
 // Elements are 8 x 32-bit little-endian limbs (32 bytes).  The device
-// multiplier is a CIOS Montgomery product (Koc, Acar, Kaliski 1996) written
-// as PTX carry chains (mad.lo.cc / madc.hi.cc) on the integer pipe; r's low
-// limb is 1, so -r^{-1} mod 2^32 = 0xffffffff and the per-row quotient digit
-// is just the negated low word.  r < 2^255 keeps every intermediate of a row
-// inside nine words.
+// multiplier is a CIOS Montgomery product (Koc, Acar, Kaliski 1996) whose
+// 64-bit partial products are accumulated in place by carry chains of wide
+// multiply-adds (see zc_mul_row); r's low limb is 1, so -r^{-1} mod 2^32 =
+// 0xffffffff and the per-row quotient digit is just the negated low word.
+// r < 2^255 keeps every intermediate of a row inside nine words.
 //
 // "Level" bookkeeping: a Montgomery product of values x (stored as x R^i)
 // and y (stored as y R^j) returns x y R^(i+j-1).  Canonical storage is level
@@ -309,58 +309,7 @@ ZC_D fr fr_sub(const fr& a, const fr& b) {
   return s;
 }
 
-// One CIOS row: t += a * b; then t += m r with m = -t0, and shift one word.
-// t holds nine words; t8 is zero on entry and becomes the new top word.
-#define ZC_ROW(B)                                                                        \
-  asm("mad.lo.cc.u32 %0, %9, %17, %0;\n\t"                                               \
-      "madc.lo.cc.u32 %1, %10, %17, %1;\n\t"                                             \
-      "madc.lo.cc.u32 %2, %11, %17, %2;\n\t"                                             \
-      "madc.lo.cc.u32 %3, %12, %17, %3;\n\t"                                             \
-      "madc.lo.cc.u32 %4, %13, %17, %4;\n\t"                                             \
-      "madc.lo.cc.u32 %5, %14, %17, %5;\n\t"                                             \
-      "madc.lo.cc.u32 %6, %15, %17, %6;\n\t"                                             \
-      "madc.lo.cc.u32 %7, %16, %17, %7;\n\t"                                             \
-      "addc.u32 %8, 0, 0;\n\t"                                                           \
-      "mad.hi.cc.u32 %1, %9, %17, %1;\n\t"                                               \
-      "madc.hi.cc.u32 %2, %10, %17, %2;\n\t"                                             \
-      "madc.hi.cc.u32 %3, %11, %17, %3;\n\t"                                             \
-      "madc.hi.cc.u32 %4, %12, %17, %4;\n\t"                                             \
-      "madc.hi.cc.u32 %5, %13, %17, %5;\n\t"                                             \
-      "madc.hi.cc.u32 %6, %14, %17, %6;\n\t"                                             \
-      "madc.hi.cc.u32 %7, %15, %17, %7;\n\t"                                             \
-      "madc.hi.u32 %8, %16, %17, %8;"                                                    \
-      : "+r"(t0), "+r"(t1), "+r"(t2), "+r"(t3), "+r"(t4), "+r"(t5), "+r"(t6), "+r"(t7), \
-        "+r"(t8)                                                                         \
-      : "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]),    \
-        "r"(a.v[6]), "r"(a.v[7]), "r"(B));                                               \
-  {                                                                                      \
-    uint32_t m = 0u - t0;                                                                \
-    asm("add.cc.u32 %0, %0, %9;\n\t"                                                     \
-        "madc.lo.cc.u32 %1, %9, %10, %1;\n\t"                                            \
-        "madc.lo.cc.u32 %2, %9, %11, %2;\n\t"                                            \
-        "madc.lo.cc.u32 %3, %9, %12, %3;\n\t"                                            \
-        "madc.lo.cc.u32 %4, %9, %13, %4;\n\t"                                            \
-        "madc.lo.cc.u32 %5, %9, %14, %5;\n\t"                                            \
-        "madc.lo.cc.u32 %6, %9, %15, %6;\n\t"                                            \
-        "madc.lo.cc.u32 %7, %9, %16, %7;\n\t"                                            \
-        "addc.u32 %8, %8, 0;\n\t"                                                        \
-        "mad.hi.cc.u32 %2, %9, %10, %2;\n\t"                                             \
-        "madc.hi.cc.u32 %3, %9, %11, %3;\n\t"                                            \
-        "madc.hi.cc.u32 %4, %9, %12, %4;\n\t"                                            \
-        "madc.hi.cc.u32 %5, %9, %13, %5;\n\t"                                            \
-        "madc.hi.cc.u32 %6, %9, %14, %6;\n\t"                                            \
-        "madc.hi.cc.u32 %7, %9, %15, %7;\n\t"                                            \
-        "madc.hi.u32 %8, %9, %16, %8;"                                                   \
-        : "+r"(t0), "+r"(t1), "+r"(t2), "+r"(t3), "+r"(t4), "+r"(t5), "+r"(t6), "+r"(t7), \
-          "+r"(t8)                                                                       \
-        : "r"(m), "n"(ZC_P1), "n"(ZC_P2), "n"(ZC_P3), "n"(ZC_P4), "n"(ZC_P5), "n"(ZC_P6), \
-          "n"(ZC_P7));                                                                   \
-  }                                                                                      \
-  t0 = t1; t1 = t2; t2 = t3; t3 = t4; t4 = t5; t5 = t6; t6 = t7; t7 = t8; t8 = 0;
-
-// In the reduction asm, %9 is m and %10..%16 are r1..r7; r0 = 1 turns its
-// low product into a plain add and its high product into zero.
-
+// t - r when t >= r, for t < 2r given as words
 ZC_D fr fr_reduce_final(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3, uint32_t t4,
                         uint32_t t5, uint32_t t6, uint32_t t7) {
   fr s, r;
@@ -389,90 +338,113 @@ ZC_D fr fr_reduce_final(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3, uint
   return r;
 }
 
-// Carry-chain variant (mad.lo.cc / madc.hi.cc), kept for comparison.
-ZC_D fr fr_mul_cc(const fr& a, const fr& b) {
-  uint32_t t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0, t5 = 0, t6 = 0, t7 = 0, t8 = 0;
-  ZC_ROW(b.v[0])
-  ZC_ROW(b.v[1])
-  ZC_ROW(b.v[2])
-  ZC_ROW(b.v[3])
-  ZC_ROW(b.v[4])
-  ZC_ROW(b.v[5])
-  ZC_ROW(b.v[6])
-  ZC_ROW(b.v[7])
-  return fr_reduce_final(t0, t1, t2, t3, t4, t5, t6, t7);
+// Montgomery rows (CIOS) with the even/odd split of the partial products
+// (Emmart, Luitjens, Weems, Woolley, "Optimizing Modular Multiplication for
+// NVIDIA's Maxwell GPUs", ARITH 2016).  The accumulator is E + 2^32 O: a_j b
+// is 64 bits wide, so the products with even j fill E's word pairs and those
+// with odd j O's, and each half is one carry chain of mad.lo.cc / madc.hi.cc
+// pairs that the integer multiplier accumulates in place (one wide
+// multiply-add per product, the carry in a predicate): no separate additions.
+// Dropping the zero low word after a reduction swaps the halves: the new E is
+// O, the new O is E from word 2 on, and E's word 1 (X) enters the next row at
+// word 0, its carry flowing into the O chain, which starts at word 1.
+//
+// The reduction adds m r, m = -t0 (r0 = 1).  r1 = 2^32 - 1 needs no product:
+// m (2^32 - 1) = (m - [m != 0]) 2^32 + t0.
+//
+// Bound: a wide multiply-add holds the multiplier pipe four cycles per warp
+// and SM quarter, so 64 + 48 products take 448 cycles: at most 9.0e10
+// products/s at 2070 MHz.  Measured (chains of dependent products, 16 warps
+// per SM, one GB300): 7.59e10 inlined, 85 % of that, against 5.08e10 for rows
+// of plain 64-bit products joined by add-with-carry chains (426 instructions
+// a product, the ALU pipe's additions the bound); with m r1 as a ninth wide
+// product 6.4e10, with m r0 too 6.1e10.
+
+// E[0..8], O[0..7] = a b (E[8] = 0)
+ZC_D void zc_mul_first(const fr& a, uint32_t b, uint32_t (&E)[9], uint32_t (&O)[8]) {
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    asm("mul.lo.u32 %0, %2, %3;\n\tmul.hi.u32 %1, %2, %3;" : "=r"(E[j]), "=r"(E[j + 1]) : "r"(a.v[j]), "r"(b));
+    asm("mul.lo.u32 %0, %2, %3;\n\tmul.hi.u32 %1, %2, %3;" : "=r"(O[j]), "=r"(O[j + 1]) : "r"(a.v[j + 1]), "r"(b));
+  }
+  E[8] = 0;
 }
 
-// CIOS with 64-bit partial products (mul.wide.u32, IMAD.WIDE on the integer
-// pipe).  Each row forms the eight products q_j = a_j b_i as 64-bit values
-// with no addend (an addend pair costs extra register moves on the same
-// pipe), joins lo(q_j) with hi(q_{j-1}) in one add-with-carry chain and adds
-// that to t in a second chain on the ALU pipe.  The reduction row does the
-// same with m r_j; r_0 = 1 and r_1 = 2^32 - 1 need no multiplication
-// (m (2^32 - 1) has low word -m = t_0 and high word m - [m != 0]).
-#define ZC_LO(x) ((uint32_t)(x))
-#define ZC_HI(x) ((uint32_t)((x) >> 32))
+// E[0..7] + 2^32 O[0..6] + X + a b -> E[0..8], O[0..7]
+ZC_D void zc_mul_row(const fr& a, uint32_t b, uint32_t X, uint32_t (&E)[9], uint32_t (&O)[8]) {
+  asm("add.cc.u32 %0, %0, %17;\n\t"
+      "madc.lo.cc.u32 %9, %19, %26, %9;\n\t"
+      "madc.hi.cc.u32 %10, %19, %26, %10;\n\t"
+      "madc.lo.cc.u32 %11, %21, %26, %11;\n\t"
+      "madc.hi.cc.u32 %12, %21, %26, %12;\n\t"
+      "madc.lo.cc.u32 %13, %23, %26, %13;\n\t"
+      "madc.hi.cc.u32 %14, %23, %26, %14;\n\t"
+      "madc.lo.cc.u32 %15, %25, %26, %15;\n\t"
+      "madc.hi.u32 %16, %25, %26, 0;\n\t"
+      "mad.lo.cc.u32 %0, %18, %26, %0;\n\t"
+      "madc.hi.cc.u32 %1, %18, %26, %1;\n\t"
+      "madc.lo.cc.u32 %2, %20, %26, %2;\n\t"
+      "madc.hi.cc.u32 %3, %20, %26, %3;\n\t"
+      "madc.lo.cc.u32 %4, %22, %26, %4;\n\t"
+      "madc.hi.cc.u32 %5, %22, %26, %5;\n\t"
+      "madc.lo.cc.u32 %6, %24, %26, %6;\n\t"
+      "madc.hi.cc.u32 %7, %24, %26, %7;\n\t"
+      "addc.u32 %8, 0, 0;"
+      : "+r"(E[0]), "+r"(E[1]), "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]), "=r"(E[8]),
+        "+r"(O[0]), "+r"(O[1]), "+r"(O[2]), "+r"(O[3]), "+r"(O[4]), "+r"(O[5]), "+r"(O[6]), "=r"(O[7])
+      : "r"(X), "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]), "r"(a.v[6]),
+        "r"(a.v[7]), "r"(b));
+}
 
-ZC_D void zc_row_wide(const fr& a, uint32_t bi, uint32_t& t0, uint32_t& t1, uint32_t& t2,
-                      uint32_t& t3, uint32_t& t4, uint32_t& t5, uint32_t& t6, uint32_t& t7) {
-  uint64_t q0, q1, q2, q3, q4, q5, q6, q7;
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q0) : "r"(a.v[0]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q1) : "r"(a.v[1]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q2) : "r"(a.v[2]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q3) : "r"(a.v[3]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q4) : "r"(a.v[4]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q5) : "r"(a.v[5]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q6) : "r"(a.v[6]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q7) : "r"(a.v[7]), "r"(bi));
-  uint32_t s1, s2, s3, s4, s5, s6, s7, s8;
-  asm("add.cc.u32 %0, %8, %9;\n\t"
-      "addc.cc.u32 %1, %10, %11;\n\t"
-      "addc.cc.u32 %2, %12, %13;\n\t"
-      "addc.cc.u32 %3, %14, %15;\n\t"
-      "addc.cc.u32 %4, %16, %17;\n\t"
-      "addc.cc.u32 %5, %18, %19;\n\t"
-      "addc.cc.u32 %6, %20, %21;\n\t"
-      "addc.u32 %7, %22, 0;"
-      : "=r"(s1), "=r"(s2), "=r"(s3), "=r"(s4), "=r"(s5), "=r"(s6), "=r"(s7), "=r"(s8)
-      : "r"(ZC_LO(q1)), "r"(ZC_HI(q0)), "r"(ZC_LO(q2)), "r"(ZC_HI(q1)), "r"(ZC_LO(q3)),
-        "r"(ZC_HI(q2)), "r"(ZC_LO(q4)), "r"(ZC_HI(q3)), "r"(ZC_LO(q5)), "r"(ZC_HI(q4)),
-        "r"(ZC_LO(q6)), "r"(ZC_HI(q5)), "r"(ZC_LO(q7)), "r"(ZC_HI(q6)), "r"(ZC_HI(q7)));
-  uint32_t u0, u1, u2, u3, u4, u5, u6, u7, u8;
-  asm("add.cc.u32 %0, %9, %17;\n\t"
-      "addc.cc.u32 %1, %10, %18;\n\t"
-      "addc.cc.u32 %2, %11, %19;\n\t"
-      "addc.cc.u32 %3, %12, %20;\n\t"
-      "addc.cc.u32 %4, %13, %21;\n\t"
-      "addc.cc.u32 %5, %14, %22;\n\t"
-      "addc.cc.u32 %6, %15, %23;\n\t"
-      "addc.cc.u32 %7, %16, %24;\n\t"
-      "addc.u32 %8, %25, 0;"
-      : "=r"(u0), "=r"(u1), "=r"(u2), "=r"(u3), "=r"(u4), "=r"(u5), "=r"(u6), "=r"(u7), "=r"(u8)
-      : "r"(t0), "r"(t1), "r"(t2), "r"(t3), "r"(t4), "r"(t5), "r"(t6), "r"(t7), "r"(ZC_LO(q0)),
-        "r"(s1), "r"(s2), "r"(s3), "r"(s4), "r"(s5), "r"(s6), "r"(s7), "r"(s8));
-  // reduction: m = -u0 (r0 = 1), add m r, drop the zero low word
-  const uint32_t m = 0u - u0, c0 = u0 != 0 ? 1u : 0u;
-  const uint32_t r1lo = u0, r1hi = m - c0;  // m (2^32 - 1)
-  uint64_t r2, r3, r4, r5, r6, r7;
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r2) : "r"(m), "n"(ZC_P2));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r3) : "r"(m), "n"(ZC_P3));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r4) : "r"(m), "n"(ZC_P4));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r5) : "r"(m), "n"(ZC_P5));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r6) : "r"(m), "n"(ZC_P6));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r7) : "r"(m), "n"(ZC_P7));
-  uint32_t v1, v2, v3, v4, v5, v6, v7, v8;
-  asm("add.cc.u32 %0, %8, %9;\n\t"
-      "addc.cc.u32 %1, %10, %11;\n\t"
-      "addc.cc.u32 %2, %12, %13;\n\t"
-      "addc.cc.u32 %3, %14, %15;\n\t"
-      "addc.cc.u32 %4, %16, %17;\n\t"
-      "addc.cc.u32 %5, %18, %19;\n\t"
-      "addc.cc.u32 %6, %20, %21;\n\t"
-      "addc.u32 %7, %22, 0;"
-      : "=r"(v1), "=r"(v2), "=r"(v3), "=r"(v4), "=r"(v5), "=r"(v6), "=r"(v7), "=r"(v8)
-      : "r"(r1lo), "r"(c0), "r"(ZC_LO(r2)), "r"(r1hi), "r"(ZC_LO(r3)), "r"(ZC_HI(r2)),
-        "r"(ZC_LO(r4)), "r"(ZC_HI(r3)), "r"(ZC_LO(r5)), "r"(ZC_HI(r4)), "r"(ZC_LO(r6)),
-        "r"(ZC_HI(r5)), "r"(ZC_LO(r7)), "r"(ZC_HI(r6)), "r"(ZC_HI(r7)));
+// E + 2^32 O += m r, m = -E[0]; E[0] becomes 0
+ZC_D void zc_mul_reduce(uint32_t (&E)[9], uint32_t (&O)[8]) {
+  uint32_t m, h;
+  asm("sub.cc.u32 %0, 0, %2;\n\tsubc.u32 %1, %0, 0;" : "=&r"(m), "=&r"(h) : "r"(E[0]));
+  asm("add.cc.u32 %0, %0, %9;\n\t"
+      "addc.cc.u32 %1, %1, %10;\n\t"
+      "madc.lo.cc.u32 %2, %8, %11, %2;\n\t"
+      "madc.hi.cc.u32 %3, %8, %11, %3;\n\t"
+      "madc.lo.cc.u32 %4, %8, %12, %4;\n\t"
+      "madc.hi.cc.u32 %5, %8, %12, %5;\n\t"
+      "madc.lo.cc.u32 %6, %8, %13, %6;\n\t"
+      "madc.hi.u32 %7, %8, %13, %7;"
+      : "+r"(O[0]), "+r"(O[1]), "+r"(O[2]), "+r"(O[3]), "+r"(O[4]), "+r"(O[5]), "+r"(O[6]), "+r"(O[7])
+      : "r"(m), "r"(E[0]), "r"(h), "n"(ZC_P3), "n"(ZC_P5), "n"(ZC_P7));
+  asm("add.cc.u32 %0, %0, %9;\n\t"
+      "addc.cc.u32 %1, %1, 0;\n\t"
+      "madc.lo.cc.u32 %2, %9, %10, %2;\n\t"
+      "madc.hi.cc.u32 %3, %9, %10, %3;\n\t"
+      "madc.lo.cc.u32 %4, %9, %11, %4;\n\t"
+      "madc.hi.cc.u32 %5, %9, %11, %5;\n\t"
+      "madc.lo.cc.u32 %6, %9, %12, %6;\n\t"
+      "madc.hi.cc.u32 %7, %9, %12, %7;\n\t"
+      "addc.u32 %8, %8, 0;"
+      : "+r"(E[0]), "+r"(E[1]), "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]), "+r"(E[8])
+      : "r"(m), "n"(ZC_P2), "n"(ZC_P4), "n"(ZC_P6));
+}
+
+// a b R^-1 in [0, 2r) for a < r and any b < 2^256.  Between rows the
+// accumulator is below 2r (b's digits come one a row), within one below
+// 2^288: E needs nine words and O, at most the whole shifted by a word, eight.
+ZC_D fr fr_mul_lazy_inl(const fr& a, const fr& b) {
+  uint32_t E[9], O[8];
+  zc_mul_first(a, b.v[0], E, O);
+  zc_mul_reduce(E, O);
+#pragma unroll
+  for (int i = 1; i < 8; i++) {
+    uint32_t nE[9], nO[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) nE[j] = O[j];
+#pragma unroll
+    for (int j = 0; j < 7; j++) nO[j] = E[j + 2];
+    zc_mul_row(a, b.v[i], E[1], nE, nO);
+    zc_mul_reduce(nE, nO);
+#pragma unroll
+    for (int j = 0; j < 9; j++) E[j] = nE[j];
+#pragma unroll
+    for (int j = 0; j < 8; j++) O[j] = nO[j];
+  }
+  fr t;
   asm("add.cc.u32 %0, %8, %16;\n\t"
       "addc.cc.u32 %1, %9, %17;\n\t"
       "addc.cc.u32 %2, %10, %18;\n\t"
@@ -481,115 +453,84 @@ ZC_D void zc_row_wide(const fr& a, uint32_t bi, uint32_t& t0, uint32_t& t1, uint
       "addc.cc.u32 %5, %13, %21;\n\t"
       "addc.cc.u32 %6, %14, %22;\n\t"
       "addc.u32 %7, %15, %23;"
-      : "=r"(t0), "=r"(t1), "=r"(t2), "=r"(t3), "=r"(t4), "=r"(t5), "=r"(t6), "=r"(t7)
-      : "r"(u1), "r"(u2), "r"(u3), "r"(u4), "r"(u5), "r"(u6), "r"(u7), "r"(u8), "r"(v1),
-        "r"(v2), "r"(v3), "r"(v4), "r"(v5), "r"(v6), "r"(v7), "r"(v8));
+      : "=r"(t.v[0]), "=r"(t.v[1]), "=r"(t.v[2]), "=r"(t.v[3]), "=r"(t.v[4]), "=r"(t.v[5]), "=r"(t.v[6]),
+        "=r"(t.v[7])
+      : "r"(O[0]), "r"(O[1]), "r"(O[2]), "r"(O[3]), "r"(O[4]), "r"(O[5]), "r"(O[6]), "r"(O[7]), "r"(E[1]), "r"(E[2]),
+        "r"(E[3]), "r"(E[4]), "r"(E[5]), "r"(E[6]), "r"(E[7]), "r"(E[8]));
+  return t;
 }
 
 ZC_D fr fr_mul_inl(const fr& a, const fr& b) {
-  uint32_t t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0, t5 = 0, t6 = 0, t7 = 0;
-  zc_row_wide(a, b.v[0], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[1], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[2], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[3], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[4], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[5], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[6], t0, t1, t2, t3, t4, t5, t6, t7);
-  zc_row_wide(a, b.v[7], t0, t1, t2, t3, t4, t5, t6, t7);
-  return fr_reduce_final(t0, t1, t2, t3, t4, t5, t6, t7);
+  const fr t = fr_mul_lazy_inl(a, b);
+  return fr_reduce_final(t.v[0], t.v[1], t.v[2], t.v[3], t.v[4], t.v[5], t.v[6], t.v[7]);
 }
 
 // Sums of products with one reduction: (a0 b0 + ... + a_{K-1} b_{K-1}) R^-1
-// mod r, for inputs below r, K = 2 or 3.  Each CIOS row adds a_p b_p[i] for
-// every p into a 10-word accumulator, then one reduction step m r (m = -t0)
-// and a one-word shift.  Between rows the accumulator stays below (K+1) r
-// < 2^257 (nine words), before the shift below 2^289 (ten); at the end it is
-// (sum a_p b_p + M r) / 2^256 < r (K r / 2^256 + 1) < 2.36 r for K = 3, so
-// at most two subtractions of r give the canonical result.  Against K
-// separate products and K - 1 additions this saves K - 1 reductions and the
-// final corrections (~30 % fewer instructions for K = 3).
+// mod r, for inputs below r, K = 2 or 3.  Each row adds a_p b_p[i] for every
+// p, then one reduction and the one-word shift.  Between rows the accumulator
+// stays below (K+1) r < 2^257, before the shift below 2^289, so E takes ten
+// words and O nine; at the end it is (sum a_p b_p + M r) / 2^256
+// < r (K r / 2^256 + 1) < 2.36 r for K = 3: at most two subtractions of r
+// give the canonical result.  Against K separate products and K - 1 additions
+// this saves K - 1 reductions (48 of 112 wide products each).
 
-// t[0..9] += a * bi
-ZC_D void zc_acc_row(const fr& a, uint32_t bi, uint32_t& t0, uint32_t& t1, uint32_t& t2, uint32_t& t3,
-                     uint32_t& t4, uint32_t& t5, uint32_t& t6, uint32_t& t7, uint32_t& t8, uint32_t& t9) {
-  uint64_t q0, q1, q2, q3, q4, q5, q6, q7;
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q0) : "r"(a.v[0]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q1) : "r"(a.v[1]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q2) : "r"(a.v[2]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q3) : "r"(a.v[3]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q4) : "r"(a.v[4]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q5) : "r"(a.v[5]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q6) : "r"(a.v[6]), "r"(bi));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(q7) : "r"(a.v[7]), "r"(bi));
-  uint32_t s1, s2, s3, s4, s5, s6, s7, s8;
-  asm("add.cc.u32 %0, %8, %9;\n\t"
-      "addc.cc.u32 %1, %10, %11;\n\t"
-      "addc.cc.u32 %2, %12, %13;\n\t"
-      "addc.cc.u32 %3, %14, %15;\n\t"
-      "addc.cc.u32 %4, %16, %17;\n\t"
-      "addc.cc.u32 %5, %18, %19;\n\t"
-      "addc.cc.u32 %6, %20, %21;\n\t"
-      "addc.u32 %7, %22, 0;"
-      : "=r"(s1), "=r"(s2), "=r"(s3), "=r"(s4), "=r"(s5), "=r"(s6), "=r"(s7), "=r"(s8)
-      : "r"(ZC_LO(q1)), "r"(ZC_HI(q0)), "r"(ZC_LO(q2)), "r"(ZC_HI(q1)), "r"(ZC_LO(q3)),
-        "r"(ZC_HI(q2)), "r"(ZC_LO(q4)), "r"(ZC_HI(q3)), "r"(ZC_LO(q5)), "r"(ZC_HI(q4)),
-        "r"(ZC_LO(q6)), "r"(ZC_HI(q5)), "r"(ZC_LO(q7)), "r"(ZC_HI(q6)), "r"(ZC_HI(q7)));
-  asm("add.cc.u32 %0, %0, %10;\n\t"
-      "addc.cc.u32 %1, %1, %11;\n\t"
-      "addc.cc.u32 %2, %2, %12;\n\t"
-      "addc.cc.u32 %3, %3, %13;\n\t"
-      "addc.cc.u32 %4, %4, %14;\n\t"
-      "addc.cc.u32 %5, %5, %15;\n\t"
-      "addc.cc.u32 %6, %6, %16;\n\t"
-      "addc.cc.u32 %7, %7, %17;\n\t"
-      "addc.cc.u32 %8, %8, %18;\n\t"
+// E[0..9] + 2^32 O[0..8] + X += a b
+ZC_D void zc_acc_row(const fr& a, uint32_t b, uint32_t X, uint32_t (&E)[10], uint32_t (&O)[9]) {
+  asm("add.cc.u32 %0, %0, %19;\n\t"
+      "madc.lo.cc.u32 %10, %21, %28, %10;\n\t"
+      "madc.hi.cc.u32 %11, %21, %28, %11;\n\t"
+      "madc.lo.cc.u32 %12, %23, %28, %12;\n\t"
+      "madc.hi.cc.u32 %13, %23, %28, %13;\n\t"
+      "madc.lo.cc.u32 %14, %25, %28, %14;\n\t"
+      "madc.hi.cc.u32 %15, %25, %28, %15;\n\t"
+      "madc.lo.cc.u32 %16, %27, %28, %16;\n\t"
+      "madc.hi.cc.u32 %17, %27, %28, %17;\n\t"
+      "addc.u32 %18, %18, 0;\n\t"
+      "mad.lo.cc.u32 %0, %20, %28, %0;\n\t"
+      "madc.hi.cc.u32 %1, %20, %28, %1;\n\t"
+      "madc.lo.cc.u32 %2, %22, %28, %2;\n\t"
+      "madc.hi.cc.u32 %3, %22, %28, %3;\n\t"
+      "madc.lo.cc.u32 %4, %24, %28, %4;\n\t"
+      "madc.hi.cc.u32 %5, %24, %28, %5;\n\t"
+      "madc.lo.cc.u32 %6, %26, %28, %6;\n\t"
+      "madc.hi.cc.u32 %7, %26, %28, %7;\n\t"
+      "addc.cc.u32 %8, %8, 0;\n\t"
       "addc.u32 %9, %9, 0;"
-      : "+r"(t0), "+r"(t1), "+r"(t2), "+r"(t3), "+r"(t4), "+r"(t5), "+r"(t6), "+r"(t7), "+r"(t8), "+r"(t9)
-      : "r"(ZC_LO(q0)), "r"(s1), "r"(s2), "r"(s3), "r"(s4), "r"(s5), "r"(s6), "r"(s7), "r"(s8));
+      : "+r"(E[0]), "+r"(E[1]), "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]), "+r"(E[8]),
+        "+r"(E[9]), "+r"(O[0]), "+r"(O[1]), "+r"(O[2]), "+r"(O[3]), "+r"(O[4]), "+r"(O[5]), "+r"(O[6]), "+r"(O[7]),
+        "+r"(O[8])
+      : "r"(X), "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]), "r"(a.v[6]),
+        "r"(a.v[7]), "r"(b));
 }
 
-// t <- (t + m r) / 2^32 with m = -t0 (r0 = 1, r1 = 2^32 - 1); t9 becomes 0
-ZC_D void zc_reduce_row(uint32_t& t0, uint32_t& t1, uint32_t& t2, uint32_t& t3, uint32_t& t4, uint32_t& t5,
-                        uint32_t& t6, uint32_t& t7, uint32_t& t8, uint32_t& t9) {
-  const uint32_t m = 0u - t0, c0 = t0 != 0 ? 1u : 0u;
-  const uint32_t r1lo = t0, r1hi = m - c0;  // m (2^32 - 1)
-  uint64_t r2, r3, r4, r5, r6, r7;
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r2) : "r"(m), "n"(ZC_P2));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r3) : "r"(m), "n"(ZC_P3));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r4) : "r"(m), "n"(ZC_P4));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r5) : "r"(m), "n"(ZC_P5));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r6) : "r"(m), "n"(ZC_P6));
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r7) : "r"(m), "n"(ZC_P7));
-  uint32_t v1, v2, v3, v4, v5, v6, v7, v8;
-  asm("add.cc.u32 %0, %8, %9;\n\t"
-      "addc.cc.u32 %1, %10, %11;\n\t"
-      "addc.cc.u32 %2, %12, %13;\n\t"
-      "addc.cc.u32 %3, %14, %15;\n\t"
-      "addc.cc.u32 %4, %16, %17;\n\t"
-      "addc.cc.u32 %5, %18, %19;\n\t"
-      "addc.cc.u32 %6, %20, %21;\n\t"
-      "addc.u32 %7, %22, 0;"
-      : "=r"(v1), "=r"(v2), "=r"(v3), "=r"(v4), "=r"(v5), "=r"(v6), "=r"(v7), "=r"(v8)
-      : "r"(r1lo), "r"(c0), "r"(ZC_LO(r2)), "r"(r1hi), "r"(ZC_LO(r3)), "r"(ZC_HI(r2)),
-        "r"(ZC_LO(r4)), "r"(ZC_HI(r3)), "r"(ZC_LO(r5)), "r"(ZC_HI(r4)), "r"(ZC_LO(r6)),
-        "r"(ZC_HI(r5)), "r"(ZC_LO(r7)), "r"(ZC_HI(r6)), "r"(ZC_HI(r7)));
-  // t0 + (m r mod 2^32) = 0 with a carry exactly when t0 != 0 (c0 above);
-  // the shifted sum goes to fresh registers
-  uint32_t n0, n1, n2, n3, n4, n5, n6, n7, n8;
-  asm("add.cc.u32 %0, %9, %18;\n\t"
-      "addc.cc.u32 %1, %10, %19;\n\t"
-      "addc.cc.u32 %2, %11, %20;\n\t"
-      "addc.cc.u32 %3, %12, %21;\n\t"
-      "addc.cc.u32 %4, %13, %22;\n\t"
-      "addc.cc.u32 %5, %14, %23;\n\t"
-      "addc.cc.u32 %6, %15, %24;\n\t"
-      "addc.cc.u32 %7, %16, %25;\n\t"
-      "addc.u32 %8, %17, 0;"
-      : "=r"(n0), "=r"(n1), "=r"(n2), "=r"(n3), "=r"(n4), "=r"(n5), "=r"(n6), "=r"(n7), "=r"(n8)
-      : "r"(t1), "r"(t2), "r"(t3), "r"(t4), "r"(t5), "r"(t6), "r"(t7), "r"(t8), "r"(t9), "r"(v1),
-        "r"(v2), "r"(v3), "r"(v4), "r"(v5), "r"(v6), "r"(v7), "r"(v8));
-  t0 = n0; t1 = n1; t2 = n2; t3 = n3; t4 = n4; t5 = n5; t6 = n6; t7 = n7; t8 = n8;
-  t9 = 0;
+// E + 2^32 O += m r, m = -E[0] (as zc_mul_reduce, on the wider accumulator)
+ZC_D void zc_acc_reduce(uint32_t (&E)[10], uint32_t (&O)[9]) {
+  uint32_t m, h;
+  asm("sub.cc.u32 %0, 0, %2;\n\tsubc.u32 %1, %0, 0;" : "=&r"(m), "=&r"(h) : "r"(E[0]));
+  asm("add.cc.u32 %0, %0, %10;\n\t"
+      "addc.cc.u32 %1, %1, %11;\n\t"
+      "madc.lo.cc.u32 %2, %9, %12, %2;\n\t"
+      "madc.hi.cc.u32 %3, %9, %12, %3;\n\t"
+      "madc.lo.cc.u32 %4, %9, %13, %4;\n\t"
+      "madc.hi.cc.u32 %5, %9, %13, %5;\n\t"
+      "madc.lo.cc.u32 %6, %9, %14, %6;\n\t"
+      "madc.hi.cc.u32 %7, %9, %14, %7;\n\t"
+      "addc.u32 %8, %8, 0;"
+      : "+r"(O[0]), "+r"(O[1]), "+r"(O[2]), "+r"(O[3]), "+r"(O[4]), "+r"(O[5]), "+r"(O[6]), "+r"(O[7]), "+r"(O[8])
+      : "r"(m), "r"(E[0]), "r"(h), "n"(ZC_P3), "n"(ZC_P5), "n"(ZC_P7));
+  asm("add.cc.u32 %0, %0, %10;\n\t"
+      "addc.cc.u32 %1, %1, 0;\n\t"
+      "madc.lo.cc.u32 %2, %10, %11, %2;\n\t"
+      "madc.hi.cc.u32 %3, %10, %11, %3;\n\t"
+      "madc.lo.cc.u32 %4, %10, %12, %4;\n\t"
+      "madc.hi.cc.u32 %5, %10, %12, %5;\n\t"
+      "madc.lo.cc.u32 %6, %10, %13, %6;\n\t"
+      "madc.hi.cc.u32 %7, %10, %13, %7;\n\t"
+      "addc.cc.u32 %8, %8, 0;\n\t"
+      "addc.u32 %9, %9, 0;"
+      : "+r"(E[0]), "+r"(E[1]), "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]), "+r"(E[8]),
+        "+r"(E[9])
+      : "r"(m), "n"(ZC_P2), "n"(ZC_P4), "n"(ZC_P6));
 }
 
 // t (nine words, below 3r) minus r when it is at least r
@@ -616,13 +557,38 @@ ZC_D void zc_sub_r_if(uint32_t& t0, uint32_t& t1, uint32_t& t2, uint32_t& t3, ui
 
 template <int K>
 ZC_D fr fr_mul_sum_inl(const fr (&a)[K], const fr (&b)[K]) {
-  uint32_t t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0, t5 = 0, t6 = 0, t7 = 0, t8 = 0, t9 = 0;
+  uint32_t E[10] = {}, O[9] = {}, X = 0;
 #pragma unroll
   for (int i = 0; i < 8; i++) {
 #pragma unroll
-    for (int p = 0; p < K; p++) zc_acc_row(a[p], b[p].v[i], t0, t1, t2, t3, t4, t5, t6, t7, t8, t9);
-    zc_reduce_row(t0, t1, t2, t3, t4, t5, t6, t7, t8, t9);
+    for (int p = 0; p < K; p++) zc_acc_row(a[p], b[p].v[i], p == 0 ? X : 0u, E, O);
+    zc_acc_reduce(E, O);
+    uint32_t nE[10], nO[9];
+#pragma unroll
+    for (int j = 0; j < 9; j++) nE[j] = O[j];
+    nE[9] = 0;
+#pragma unroll
+    for (int j = 0; j < 8; j++) nO[j] = E[j + 2];
+    nO[8] = 0;
+    X = E[1];
+#pragma unroll
+    for (int j = 0; j < 10; j++) E[j] = nE[j];
+#pragma unroll
+    for (int j = 0; j < 9; j++) O[j] = nO[j];
   }
+  uint32_t t0, t1, t2, t3, t4, t5, t6, t7, t8;
+  asm("add.cc.u32 %0, %9, %18;\n\t"
+      "addc.cc.u32 %1, %10, %19;\n\t"
+      "addc.cc.u32 %2, %11, %20;\n\t"
+      "addc.cc.u32 %3, %12, %21;\n\t"
+      "addc.cc.u32 %4, %13, %22;\n\t"
+      "addc.cc.u32 %5, %14, %23;\n\t"
+      "addc.cc.u32 %6, %15, %24;\n\t"
+      "addc.cc.u32 %7, %16, %25;\n\t"
+      "addc.u32 %8, %17, %26;"
+      : "=r"(t0), "=r"(t1), "=r"(t2), "=r"(t3), "=r"(t4), "=r"(t5), "=r"(t6), "=r"(t7), "=r"(t8)
+      : "r"(E[0]), "r"(E[1]), "r"(E[2]), "r"(E[3]), "r"(E[4]), "r"(E[5]), "r"(E[6]), "r"(E[7]), "r"(E[8]), "r"(X),
+        "r"(O[0]), "r"(O[1]), "r"(O[2]), "r"(O[3]), "r"(O[4]), "r"(O[5]), "r"(O[6]), "r"(O[7]));
   zc_sub_r_if(t0, t1, t2, t3, t4, t5, t6, t7, t8);
   if (K > 2) zc_sub_r_if(t0, t1, t2, t3, t4, t5, t6, t7, t8);
   fr x;
@@ -640,9 +606,9 @@ ZC_D fr fr_mul_sum3(const fr& a0, const fr& b0, const fr& a1, const fr& b1, cons
   return fr_mul_sum3_call(a0, b0, a1, b1, a2, b2);
 }
 
-// The multiplier is ~400 instructions; kernels call one out-of-line copy so
-// that their code fits the instruction cache (inlined at every call site, a
-// round body of ~30 products missed the cache on almost every instruction).
+// Kernels call one out-of-line copy of the multiplier so that their code fits
+// the instruction cache (inlined at every call site, a round body of ~30
+// products missed the cache on almost every instruction).
 static __device__ __noinline__ fr fr_mul_call(fr a, fr b) { return fr_mul_inl(a, b); }
 ZC_D fr fr_mul(const fr& a, const fr& b) { return fr_mul_call(a, b); }
 
