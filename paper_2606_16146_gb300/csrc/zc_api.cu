@@ -114,6 +114,13 @@ fr h_canon_mul(const fr& a, const fr& b, const DevConst& C) {
   return fr_mul_g(fr_mul_g(a, b), C.r2);
 }
 
+frc h_frc(const fr& a, const DevConst& C) {
+  frc c;
+  c.w = a;
+  c.q = fr_quot(h_canon_mul(a, C.one, C));
+  return c;
+}
+
 static fr h_pow_limbs(const fr& a, const uint32_t e[8], const DevConst& C) {
   fr acc = h_from_u64(1);
   for (int i = 7; i >= 0; i--)

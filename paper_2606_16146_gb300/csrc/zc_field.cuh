@@ -160,6 +160,42 @@ ZC_HD fr fr_mul_g(const fr& a, const fr& b) {
   return r;
 }
 
+// ---- multiplication by a known constant
+// y w mod r for a multiplier w whose quotient q = floor(2^256 w / r) is kept
+// beside it (Shoup's method): qh = floor(y q / 2^256), y w - qh r, whose low
+// 256 bits are all that is needed.  Only the word sums 6 and up of y q are
+// formed (43 of 64 products): what is left out is below 6 2^224, so qh is
+// short of y w / r by less than 1 + y / 2^256 + 6 / 2^32 and the result is
+// below 2r for every y < 2r.  The low halves of y w and of qh r take 28 + 15
+// wide products and 14 low ones (-r = 2^32 - 1 + 2^64 N, N = ~r / 2^64: the
+// two lowest words of r need none); every carry chain of theirs ends at word
+// 7, so they need no additions besides the chains.  86 wide and 14 low
+// products against 112 wide: 372 cycles of the multiplier pipe a product
+// against 448, and 35 other instructions against 90.  Measured (dependent
+// products, 16 warps per SM, one GB300): 9.1e10 products/s, 9.3e10 with the
+// constant in the kernel parameters, against 7.1e10 for fr_mul_inl in the
+// same run.
+struct frc {
+  fr w, q;  // canonical w, floor(2^256 w / r)
+};
+
+// floor(2^256 w / r) from w R mod r: 2^256 w = q r + (w R mod r), so
+// q = (w R mod r) (-r^-1) mod 2^256
+ZC_HD fr fr_quot(const fr& w1) {
+  const uint32_t ninv[8] = {0xffffffffu, 0xfffffffeu, 0xfffe5bfdu, 0x53ba5bffu,
+                            0x0004ec06u, 0x181b2c17u, 0xd7bf2839u, 0x3d443ab0u};
+  fr t = fr_zero();
+  for (int i = 0; i < 8; i++) {
+    uint64_t k = 0;
+    for (int j = 0; i + j < 8; j++) {
+      k += (uint64_t)w1.v[i] * ninv[j] + t.v[i + j];
+      t.v[i + j] = (uint32_t)k;
+      k >>= 32;
+    }
+  }
+  return t;
+}
+
 // ---------------------------------------------------------------- device --
 #if defined(__CUDACC__)
 
@@ -465,6 +501,151 @@ ZC_D fr fr_mul_inl(const fr& a, const fr& b) {
   return fr_reduce_final(t.v[0], t.v[1], t.v[2], t.v[3], t.v[4], t.v[5], t.v[6], t.v[7]);
 }
 
+// Product by a constant (see frc): y w mod r in [0, 2r), for y < 2r.
+// c[0..2NP) += b (a0, a1, ...) as one carry chain of 64-bit products.  TAIL 0:
+// the chain ends there (no carry out), 1: the carry is added to c[2NP], 2: the
+// low word of al b (with the carry) is added to c[2NP].
+template <int NP, int TAIL>
+ZC_D void zc_chain(uint32_t* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b, uint32_t al = 0) {
+  if constexpr (NP == 0) {
+    if constexpr (TAIL == 2) asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(c[0]) : "r"(al), "r"(b));
+  } else if constexpr (NP == 1) {
+    if constexpr (TAIL == 0)
+      asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, %1;" : "+r"(c[0]), "+r"(c[1]) : "r"(a0), "r"(b));
+    else if constexpr (TAIL == 1)
+      asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\tmadc.hi.cc.u32 %1, %3, %4, %1;\n\taddc.u32 %2, %2, 0;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]) : "r"(a0), "r"(b));
+    else
+      asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\tmadc.hi.cc.u32 %1, %3, %4, %1;\n\tmadc.lo.u32 %2, %5, %4, %2;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]) : "r"(a0), "r"(b), "r"(al));
+  } else if constexpr (NP == 2) {
+#define ZC_C2 "mad.lo.cc.u32 %0, %5, %7, %0;\n\tmadc.hi.cc.u32 %1, %5, %7, %1;\n\tmadc.lo.cc.u32 %2, %6, %7, %2;\n\t"
+    if constexpr (TAIL == 0)
+      asm(ZC_C2 "madc.hi.u32 %3, %6, %7, %3;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(al) : "r"(a0), "r"(a1), "r"(b));
+    else if constexpr (TAIL == 1)
+      asm(ZC_C2 "madc.hi.cc.u32 %3, %6, %7, %3;\n\taddc.u32 %4, %4, 0;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]) : "r"(a0), "r"(a1), "r"(b));
+    else
+      asm(ZC_C2 "madc.hi.cc.u32 %3, %6, %7, %3;\n\tmadc.lo.u32 %4, %8, %7, %4;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]) : "r"(a0), "r"(a1), "r"(b), "r"(al));
+  } else if constexpr (NP == 3) {
+#define ZC_C3                                                                                                     \
+  "mad.lo.cc.u32 %0, %7, %10, %0;\n\tmadc.hi.cc.u32 %1, %7, %10, %1;\n\tmadc.lo.cc.u32 %2, %8, %10, %2;\n\t"       \
+  "madc.hi.cc.u32 %3, %8, %10, %3;\n\tmadc.lo.cc.u32 %4, %9, %10, %4;\n\t"
+    if constexpr (TAIL == 0)
+      asm(ZC_C3 "madc.hi.u32 %5, %9, %10, %5;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(al)
+          : "r"(a0), "r"(a1), "r"(a2), "r"(b));
+    else if constexpr (TAIL == 1)
+      asm(ZC_C3 "madc.hi.cc.u32 %5, %9, %10, %5;\n\taddc.u32 %6, %6, 0;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6])
+          : "r"(a0), "r"(a1), "r"(a2), "r"(b));
+    else
+      asm(ZC_C3 "madc.hi.cc.u32 %5, %9, %10, %5;\n\tmadc.lo.u32 %6, %11, %10, %6;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6])
+          : "r"(a0), "r"(a1), "r"(a2), "r"(b), "r"(al));
+  } else {
+#define ZC_C4                                                                                                     \
+  "mad.lo.cc.u32 %0, %9, %13, %0;\n\tmadc.hi.cc.u32 %1, %9, %13, %1;\n\tmadc.lo.cc.u32 %2, %10, %13, %2;\n\t"      \
+  "madc.hi.cc.u32 %3, %10, %13, %3;\n\tmadc.lo.cc.u32 %4, %11, %13, %4;\n\tmadc.hi.cc.u32 %5, %11, %13, %5;\n\t"   \
+  "madc.lo.cc.u32 %6, %12, %13, %6;\n\t"
+    if constexpr (TAIL == 0)
+      asm(ZC_C4 "madc.hi.u32 %7, %12, %13, %7;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7]), "+r"(al)
+          : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b));
+    else
+      asm(ZC_C4 "madc.hi.cc.u32 %7, %12, %13, %7;\n\taddc.u32 %8, %8, 0;"
+          : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7]), "+r"(c[8])
+          : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b));
+  }
+}
+
+ZC_D fr fr_mulc_lazy(const frc& W, const fr& y) {
+  const uint32_t* p = W.q.v;
+  uint32_t E[10] = {}, O[9] = {};  // words 6..15 (products of even word sums) and 7..15 (odd) of y q
+  zc_chain<1, 0>(E, p[6], 0, 0, 0, y.v[0]);
+  zc_chain<1, 0>(O, p[7], 0, 0, 0, y.v[0]);
+  zc_chain<2, 0>(E, p[5], p[7], 0, 0, y.v[1]);
+  zc_chain<1, 1>(O, p[6], 0, 0, 0, y.v[1]);
+  zc_chain<2, 1>(E, p[4], p[6], 0, 0, y.v[2]);
+  zc_chain<2, 0>(O, p[5], p[7], 0, 0, y.v[2]);
+  zc_chain<3, 0>(E, p[3], p[5], p[7], 0, y.v[3]);
+  zc_chain<2, 1>(O, p[4], p[6], 0, 0, y.v[3]);
+  zc_chain<3, 1>(E, p[2], p[4], p[6], 0, y.v[4]);
+  zc_chain<3, 0>(O, p[3], p[5], p[7], 0, y.v[4]);
+  zc_chain<4, 0>(E, p[1], p[3], p[5], p[7], y.v[5]);
+  zc_chain<3, 1>(O, p[2], p[4], p[6], 0, y.v[5]);
+  zc_chain<4, 1>(E, p[0], p[2], p[4], p[6], y.v[6]);
+  zc_chain<4, 0>(O, p[1], p[3], p[5], p[7], y.v[6]);
+  zc_chain<4, 0>(E + 2, p[1], p[3], p[5], p[7], y.v[7]);
+  zc_chain<4, 1>(O, p[0], p[2], p[4], p[6], y.v[7]);
+  fr q;
+  asm("add.cc.u32 %0, %9, %18;\n\t"
+      "addc.cc.u32 %1, %10, %19;\n\t"
+      "addc.cc.u32 %2, %11, %20;\n\t"
+      "addc.cc.u32 %3, %12, %21;\n\t"
+      "addc.cc.u32 %4, %13, %22;\n\t"
+      "addc.cc.u32 %5, %14, %23;\n\t"
+      "addc.cc.u32 %6, %15, %24;\n\t"
+      "addc.cc.u32 %7, %16, %25;\n\t"
+      "addc.u32 %8, %17, %26;"
+      : "+r"(E[0]), "=r"(q.v[0]), "=r"(q.v[1]), "=r"(q.v[2]), "=r"(q.v[3]), "=r"(q.v[4]), "=r"(q.v[5]), "=r"(q.v[6]),
+        "=r"(q.v[7])
+      : "r"(E[1]), "r"(E[2]), "r"(E[3]), "r"(E[4]), "r"(E[5]), "r"(E[6]), "r"(E[7]), "r"(E[8]), "r"(E[9]), "r"(O[0]),
+        "r"(O[1]), "r"(O[2]), "r"(O[3]), "r"(O[4]), "r"(O[5]), "r"(O[6]), "r"(O[7]), "r"(O[8]));
+  // y w - q r mod 2^256, -r = -1 + 2^32 + 2^64 N: A = -q - 1 (words 0..7), B = q (words 1..7)
+  constexpr uint32_t N0 = ~ZC_P2, N1 = ~ZC_P3, N2 = ~ZC_P4, N3 = ~ZC_P5, N4 = ~ZC_P6, N5 = ~ZC_P7;
+  uint32_t A[8], B[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) A[i] = ~q.v[i];
+#pragma unroll
+  for (int i = 0; i < 7; i++) B[i] = q.v[i];
+  const uint32_t* w = W.w.v;
+  zc_chain<4, 0>(A, w[0], w[2], w[4], w[6], y.v[0]);
+  zc_chain<3, 2>(B, w[1], w[3], w[5], 0, y.v[0], w[7]);
+  zc_chain<3, 0>(A + 2, w[1], w[3], w[5], 0, y.v[1]);
+  zc_chain<3, 2>(B, w[0], w[2], w[4], 0, y.v[1], w[6]);
+  zc_chain<3, 0>(A + 2, w[0], w[2], w[4], 0, y.v[2]);
+  zc_chain<2, 2>(B + 2, w[1], w[3], 0, 0, y.v[2], w[5]);
+  zc_chain<2, 0>(A + 4, w[1], w[3], 0, 0, y.v[3]);
+  zc_chain<2, 2>(B + 2, w[0], w[2], 0, 0, y.v[3], w[4]);
+  zc_chain<2, 0>(A + 4, w[0], w[2], 0, 0, y.v[4]);
+  zc_chain<1, 2>(B + 4, w[1], 0, 0, 0, y.v[4], w[3]);
+  zc_chain<1, 0>(A + 6, w[1], 0, 0, 0, y.v[5]);
+  zc_chain<1, 2>(B + 4, w[0], 0, 0, 0, y.v[5], w[2]);
+  zc_chain<1, 0>(A + 6, w[0], 0, 0, 0, y.v[6]);
+  zc_chain<0, 2>(B + 6, 0, 0, 0, 0, y.v[6], w[1]);
+  zc_chain<0, 2>(B + 6, 0, 0, 0, 0, y.v[7], w[0]);
+  // q N at word 2
+  zc_chain<3, 0>(A + 2, N0, N2, N4, 0, q.v[0]);
+  zc_chain<2, 2>(B + 2, N1, N3, 0, 0, q.v[0], N5);
+  zc_chain<2, 0>(A + 4, N1, N3, 0, 0, q.v[1]);
+  zc_chain<2, 2>(B + 2, N0, N2, 0, 0, q.v[1], N4);
+  zc_chain<2, 0>(A + 4, N0, N2, 0, 0, q.v[2]);
+  zc_chain<1, 2>(B + 4, N1, 0, 0, 0, q.v[2], N3);
+  zc_chain<1, 0>(A + 6, N1, 0, 0, 0, q.v[3]);
+  zc_chain<1, 2>(B + 4, N0, 0, 0, 0, q.v[3], N2);
+  zc_chain<1, 0>(A + 6, N0, 0, 0, 0, q.v[4]);
+  zc_chain<0, 2>(B + 6, 0, 0, 0, 0, q.v[4], N1);
+  zc_chain<0, 2>(B + 6, 0, 0, 0, 0, q.v[5], N0);
+  fr t;
+  asm("add.cc.u32 %0, %8, 1;\n\t"
+      "addc.cc.u32 %1, %9, %16;\n\t"
+      "addc.cc.u32 %2, %10, %17;\n\t"
+      "addc.cc.u32 %3, %11, %18;\n\t"
+      "addc.cc.u32 %4, %12, %19;\n\t"
+      "addc.cc.u32 %5, %13, %20;\n\t"
+      "addc.cc.u32 %6, %14, %21;\n\t"
+      "addc.u32 %7, %15, %22;"
+      : "=r"(t.v[0]), "=r"(t.v[1]), "=r"(t.v[2]), "=r"(t.v[3]), "=r"(t.v[4]), "=r"(t.v[5]), "=r"(t.v[6]), "=r"(t.v[7])
+      : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(B[0]), "r"(B[1]),
+        "r"(B[2]), "r"(B[3]), "r"(B[4]), "r"(B[5]), "r"(B[6]));
+  return t;
+}
+
+ZC_D fr fr_mulc(const frc& W, const fr& y) { return fr_reduce1(fr_mulc_lazy(W, y)); }
+
 // Sums of products with one reduction: (a0 b0 + ... + a_{K-1} b_{K-1}) R^-1
 // mod r, for inputs below r, K = 2 or 3.  Each row adds a_p b_p[i] for every
 // p, then one reduction and the one-word shift.  Between rows the accumulator
@@ -611,6 +792,16 @@ ZC_D fr fr_mul_sum3(const fr& a0, const fr& b0, const fr& a1, const fr& b1, cons
 // products missed the cache on almost every instruction).
 static __device__ __noinline__ fr fr_mul_call(fr a, fr b) { return fr_mul_inl(a, b); }
 ZC_D fr fr_mul(const fr& a, const fr& b) { return fr_mul_call(a, b); }
+
+// the constant c from its level-1 form c R mod r
+ZC_D frc frc_of(const fr& c1) {
+  frc c;
+  fr one = fr_zero();
+  one.v[0] = 1;
+  c.w = fr_mul(one, c1);
+  c.q = fr_quot(c1);
+  return c;
+}
 
 #else
 inline fr fr_add(const fr& a, const fr& b) { return fr_add_g(a, b); }

@@ -117,20 +117,23 @@ struct zc_ctx {
     void* mem = nullptr;
     size_t bytes = 0;
     uint64_t stamp = 0;
-    zc::fr *tw_fwd = nullptr, *tw_inv = nullptr, *coset = nullptr, *outer = nullptr, *fin = nullptr;
-    zc::fr* zinv = nullptr;  // per slice: (7^N w_s^j - 1)^-1 M^-1, level 1
+    zc::frc *tw_fwd = nullptr, *tw_inv = nullptr, *coset = nullptr, *outer = nullptr;
+    zc::frc* fin = nullptr;   // 7^-(N t), t < s
+    zc::frc* zinv = nullptr;  // per slice: (7^N w_s^j - 1)^-1 M^-1
     // step-radix domain 2^lb N + N (built on first use): the small part's
-    // coset factors sigma^k / N (level 2) and sigma^-k 7^k (level 1),
-    // k < N, sigma = 7 w_{2M}; constants: [0] the small part's z_H inverse
-    // times kappa^-1 N^-1, [1] 7^M (level 1), [8 + m] sigma^(mN) kappa^-1,
+    // coset factors sigma^k / N and sigma^-k 7^k (level 1), k < N,
+    // sigma = 7 w_{2M}; constants: [0], [1] the small part's z_H inverse
+    // times kappa^-1 N^-1 (frc), [2] 7^M (level 1), [8 + m] sigma^(mN) kappa^-1,
     // m < 2^lb (level 1), kappa = sigma^M - 7^M.
     void* step_mem = nullptr;
     size_t step_bytes = 0;
-    zc::fr *step_coset = nullptr, *step_unscale = nullptr, *step_const = nullptr;
+    zc::frc* step_coset = nullptr;
+    zc::fr *step_unscale = nullptr, *step_const = nullptr;
   };
   std::vector<NttSizeTables> ntt_cache;
   uint64_t ntt_cache_clock = 0;
-  size_t ntt_cache_budget = 16ull << 30;
+  // 24 GiB holds every size that 16 GiB of 32-byte entries did
+  size_t ntt_cache_budget = 24ull << 30;
   // While a prepared batch is being enqueued (possibly under graph capture)
   // the cache neither allocates nor evicts; a missing size falls back to the
   // two-level power tables.
@@ -173,6 +176,7 @@ fr h_canon_mul(const fr& a, const fr& b, const DevConst& C);  // a*b mod r, cano
 fr h_pow(const fr& a, uint64_t e, const DevConst& C);          // canonical
 fr h_inv(const fr& a, const DevConst& C);                      // canonical, a != 0
 fr h_from_u64(uint64_t x);
+frc h_frc(const fr& a, const DevConst& C);                     // the constant multiplier of canonical a
 fr h_root_of_unity(uint32_t logn, const DevConst& C);        // canonical generator of the 2^logn subgroup
 const DevConst& host_constants();                            // the field constants, built once
 void h_to_bytes(const fr& a, uint8_t* out);
@@ -205,7 +209,7 @@ size_t root_scratch_bytes(int c, uint64_t L);
 // column digests, leaves and tree levels (2W - 1 nodes of 8 words, leaves
 // first) of the encoded columns
 zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uint32_t nc, fr* const* enc,
-                     fr* tab, cudaStream_t st);
+                     frc* tab, cudaStream_t st);
 zc_status pcs_hash_tree(zc_ctx* ctx, const fr* const* enc, int c, uint64_t m, uint64_t W, uint32_t* dig,
                         uint32_t* tree, cudaStream_t st);
 void static_constants(DevConst* C, std::vector<fr>* tabs);
@@ -240,6 +244,12 @@ __device__ __forceinline__ fr ld_fr(const fr* p) {
   x.v[4] = b.x; x.v[5] = b.y; x.v[6] = b.z; x.v[7] = b.w;
   return x;
 }
+__device__ __forceinline__ frc ld_frc(const frc* p) {
+  frc c;
+  c.w = ld_fr(&p->w);
+  c.q = ld_fr(&p->q);
+  return c;
+}
 // plain (coherent) load for data written earlier by the same kernel family
 __device__ __forceinline__ fr ld_fr_cg(const fr* p) {
   const uint4* q = reinterpret_cast<const uint4*>(p);
@@ -253,6 +263,10 @@ __device__ __forceinline__ void st_fr(fr* p, const fr& x) {
   uint4* q = reinterpret_cast<uint4*>(p);
   q[0] = make_uint4(x.v[0], x.v[1], x.v[2], x.v[3]);
   q[1] = make_uint4(x.v[4], x.v[5], x.v[6], x.v[7]);
+}
+__device__ __forceinline__ void st_frc(frc* p, const frc& c) {
+  st_fr(&p->w, c.w);
+  st_fr(&p->q, c.q);
 }
 __device__ __forceinline__ fr shfl_down_fr(const fr& x, int delta) {
   fr y;

@@ -39,8 +39,9 @@ constexpr int kMaxNttN = 24;
 struct NttTables {
   bool ready = false;
   fr w32h;                 // 7^((r-1)/2^32), canonical, host copy
-  fr* dft_fwd = nullptr;   // w_4096^m, m < 4096 (level 1)
-  fr* dft_inv = nullptr;
+  frc* dft_fwd = nullptr;  // w_4096^m, m < 4096
+  frc* dft_inv = nullptr;
+  frc c_fwd[3], c_inv[3];  // w_8, w_4, w_8^3 of each direction (host copies, passed to the kernels by value)
   fr* wf_lo = nullptr;     // w_2^30^b, b < 2^15 (level 1)
   fr* wf_hi = nullptr;     // w_2^30^(a 2^15)
   fr* wi_lo = nullptr;     // inverse root
@@ -56,7 +57,7 @@ static NttTables g_tabs_by_dev[64];
 static std::mutex g_tabs_mu;
 
 struct NttTabArgs {
-  fr* dft_fwd; fr* dft_inv; fr* wf_lo; fr* wf_hi; fr* wi_lo; fr* wi_hi; fr* s7_lo; fr* s7_hi;
+  frc* dft_fwd; frc* dft_inv; fr* wf_lo; fr* wf_hi; fr* wi_lo; fr* wi_hi; fr* s7_lo; fr* s7_hi;
   fr* p7_lo; fr* p7_hi;
   fr w30;        // 2^30-th root (level 1)
   fr w30i;       // its inverse (level 1)
@@ -79,8 +80,8 @@ __global__ void k_ntt_tables(NttTabArgs A) {
   const DevConst* C = A.C;
   if (i < 4096) {
     // w_4096 = w30^(2^18)
-    A.dft_fwd[i] = fr_pow_dev(A.w30, (uint64_t)i << 18, C);
-    A.dft_inv[i] = fr_pow_dev(A.w30i, (uint64_t)i << 18, C);
+    A.dft_fwd[i] = frc_of(fr_pow_dev(A.w30, (uint64_t)i << 18, C));
+    A.dft_inv[i] = frc_of(fr_pow_dev(A.w30i, (uint64_t)i << 18, C));
   }
   if (i < (1u << kLoBits)) {
     A.wf_lo[i] = fr_pow_dev(A.w30, i, C);
@@ -114,7 +115,8 @@ struct NttPassArgs {
   uint32_t in_lbdiv, out_lbdiv;
   uint64_t in_bs_hi, in_bs_lo, in_ts;
   uint64_t out_bs_hi, out_bs_lo, out_ts;
-  const fr* dft;          // 4096-th roots, forward or inverse
+  const frc* dft;         // 4096-th roots, forward or inverse
+  frc w8, w4, w83;        // their powers 512, 1024, 1536
   int pre;
   const fr* pre_lo;       // per-item coset tables (item stride pre_stride)
   const fr* pre_hi;
@@ -129,24 +131,27 @@ struct NttPassArgs {
   uint64_t fin_N;         // POST_FINAL: k = fin_N * t + b
   // table modes: PRE_TAB factor = pre_tab[b * pre_kb + t * pre_kt];
   // POST_TAB factor = post_tab[(b >> p_lbdiv) * p_hs + (b & (2^p_lbdiv - 1)) * p_ls + t * p_ts]
-  const fr* pre_tab;
-  const fr* post_tab;
+  const frc* pre_tab;
+  const frc* post_tab;
   uint32_t p_lbdiv;
   uint64_t p_hs, p_ls, p_ts;
   uint32_t* err;          // if set: the pass reads the proof's input columns, and a value >= r sets bit 0
 };
 
 // radix-2/4/8 butterflies on x[0..R) in registers, X[k] = sum_r x[r] w_R^(rk).
-// Inputs are canonical.  A value that only feeds a multiplication (as
-// fr_mul's second operand, which may be any value below 2r) is left lazily
-// reduced in [0, 2r): the stage outputs (the next stage multiplies all but
-// one of them by its twiddle and reduces that one, the pass's store reduces
-// or multiplies every one), and the terms multiplied by w_4, w_8, w_8^3.
+// Inputs are canonical.  A value that only feeds a multiplication (fr_mulc
+// takes any value below 2r) is left lazily reduced in [0, 2r): the stage
+// outputs (the next stage multiplies all but one of them by its twiddle and
+// reduces that one, the pass's store reduces or multiplies every one), and
+// the terms multiplied by w_4, w_8, w_8^3.  Every factor of a transform is a
+// constant, so all of them are fr_mulc products, inlined; w_4, w_8 and w_8^3
+// are kernel parameters, which the multiplier reads as operands without a
+// load.
 // OUT: 0 every output canonical, 1 a0 canonical and a1..a3 lazy, 2 all lazy.
 template <int OUT>
-__device__ __forceinline__ void dft4(fr& a0, fr& a1, fr& a2, fr& a3, const fr& w4) {
+__device__ __forceinline__ void dft4(fr& a0, fr& a1, fr& a2, fr& a3, const frc& w4) {
   const fr u0 = fr_add(a0, a2), u1 = fr_sub(a0, a2);
-  const fr v0 = fr_add(a1, a3), v1 = fr_mul(w4, fr_sub_lazy(a1, a3));
+  const fr v0 = fr_add(a1, a3), v1 = fr_mulc(w4, fr_sub_lazy(a1, a3));
   a0 = OUT == 2 ? fr_add_lazy(u0, v0) : fr_add(u0, v0);
   a2 = OUT >= 1 ? fr_sub_lazy(u0, v0) : fr_sub(u0, v0);
   a1 = OUT >= 1 ? fr_add_lazy(u1, v1) : fr_add(u1, v1);
@@ -154,14 +159,14 @@ __device__ __forceinline__ void dft4(fr& a0, fr& a1, fr& a2, fr& a3, const fr& w
 }
 
 // outputs lazy
-__device__ __forceinline__ void dft8(fr (&x)[8], const fr* tab) {
+__device__ __forceinline__ void dft8(fr (&x)[8], const NttPassArgs& A) {
   fr e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
   fr o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
-  dft4<0>(e0, e1, e2, e3, ld_fr(tab + 1024));
-  dft4<1>(o0, o1, o2, o3, ld_fr(tab + 1024));
-  o1 = fr_mul(ld_fr(tab + 512), o1);    // w_8
-  o2 = fr_mul(ld_fr(tab + 1024), o2);   // w_4
-  o3 = fr_mul(ld_fr(tab + 1536), o3);   // w_8^3
+  dft4<0>(e0, e1, e2, e3, A.w4);
+  dft4<1>(o0, o1, o2, o3, A.w4);
+  o1 = fr_mulc(A.w8, o1);
+  o2 = fr_mulc(A.w4, o2);
+  o3 = fr_mulc(A.w83, o3);
   x[0] = fr_add_lazy(e0, o0);
   x[4] = fr_sub_lazy(e0, o0);
   x[1] = fr_add_lazy(e1, o1);
@@ -199,7 +204,7 @@ struct SmTile {
 // thread owns 8 elements (8 / R independent groups).
 template <int LR>
 __device__ __forceinline__ void stockham_stage(const SmTile& sm, uint32_t logL, uint32_t logW,
-                                               uint32_t logNs, const fr* tab) {
+                                               uint32_t logNs, const NttPassArgs& A) {
   constexpr int R = 1 << LR;
   constexpr int GROUPS = 8 / R;
   const uint32_t L = 1u << logL, W = 1u << logW;
@@ -226,25 +231,21 @@ __device__ __forceinline__ void stockham_stage(const SmTile& sm, uint32_t logL, 
     const uint32_t k = j & ((1u << logNs) - 1);
     if (logNs > 0) {
       // the previous stage left its outputs lazy: x[0] is reduced, the
-      // others are reduced by their twiddle w_{Ns R}^{r k} = tab[r k 4096 / (Ns R)].
-      // These products, and the pass's load and store factors, use the
-      // inlined multiplier (fewer instructions than the shared call); the
-      // DFT-8's own products stay calls (inlined they spilled registers and
-      // measured slower).
+      // others are reduced by their twiddle w_{Ns R}^{r k} = dft[r k 4096 / (Ns R)]
       const uint32_t sh = 12 - (logNs + LR);
       x[g * R] = fr_reduce1(x[g * R]);
 #pragma unroll
-      for (int r = 1; r < R; r++) x[g * R + r] = fr_mul_inl(ld_fr(tab + ((r * k) << sh)), x[g * R + r]);
+      for (int r = 1; r < R; r++) x[g * R + r] = fr_mulc(ld_frc(A.dft + ((r * k) << sh)), x[g * R + r]);
     }
     if (R == 8) {
       fr y[8];
 #pragma unroll
       for (int r = 0; r < 8; r++) y[r] = x[r];
-      dft8(y, tab);
+      dft8(y, A);
 #pragma unroll
       for (int r = 0; r < 8; r++) x[r] = y[r];
     } else if (R == 4) {
-      dft4<2>(x[g * 4], x[g * 4 + 1], x[g * 4 + 2], x[g * 4 + 3], ld_fr(tab + 1024));
+      dft4<2>(x[g * 4], x[g * 4 + 1], x[g * 4 + 2], x[g * 4 + 3], A.w4);
     } else {
       fr a = x[g * 2], b = x[g * 2 + 1];
       x[g * 2] = fr_add_lazy(a, b);
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(TILE / 8, MINB) k_ntt_pass(NttPassArgs A) {
     fr x = ld_fr(in + a);
     if (A.err && !fr_is_canonical(x)) atomicOr(A.err, 1u);
     if (A.pre == PRE_TAB) {
-      x = fr_mul_inl(ld_fr(A.pre_tab + b * A.pre_kb + t * A.pre_kt), x);
+      x = fr_mulc(ld_frc(A.pre_tab + b * A.pre_kb + t * A.pre_kt), x);
     } else if (A.pre == PRE_COSET) {
       const uint64_t k = b * A.pre_kb + t * A.pre_kt;
       // one slice per launch: every column uses the same tables
@@ -338,11 +339,11 @@ __global__ void __launch_bounds__(TILE / 8, MINB) k_ntt_pass(NttPassArgs A) {
   // ---- Stockham stages: radix 8 while >= 3 bits remain, then 4 or 2
   uint32_t logNs = 0;
   while (logL - logNs >= 3) {
-    stockham_stage<3>(sm, logL, logW, logNs, A.dft);
+    stockham_stage<3>(sm, logL, logW, logNs, A);
     logNs += 3;
   }
-  if (logL - logNs == 2) stockham_stage<2>(sm, logL, logW, logNs, A.dft);
-  else if (logL - logNs == 1) stockham_stage<1>(sm, logL, logW, logNs, A.dft);
+  if (logL - logNs == 2) stockham_stage<2>(sm, logL, logW, logNs, A);
+  else if (logL - logNs == 1) stockham_stage<1>(sm, logL, logW, logNs, A);
 
   // ---- store (with the twiddle / final scale)
   for (uint32_t idx = threadIdx.x; idx < n_el; idx += blockDim.x) {
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(TILE / 8, MINB) k_ntt_pass(NttPassArgs A) {
     fr y = sm.get(t * W + w);  // lazily reduced: multiplied (as the second operand) or reduced here
     if (A.post == POST_TAB) {
       const uint64_t ti = (b >> A.p_lbdiv) * A.p_hs + (b & ((1ull << A.p_lbdiv) - 1)) * A.p_ls + t * A.p_ts;
-      y = fr_mul_inl(ld_fr(A.post_tab + ti), y);
+      y = fr_mulc(ld_frc(A.post_tab + ti), y);
     } else if (A.post == POST_TW) {
       const uint64_t e = (b & ((1ull << A.tw_lbmod) - 1)) * t;
       const uint32_t ex = (uint32_t)((e << A.tw_shift) & ((1ull << kLog30) - 1));
@@ -380,14 +381,15 @@ __global__ void __launch_bounds__(TILE / 8, MINB) k_ntt_pass(NttPassArgs A) {
 // For one (n, log2 s): the four-step twiddles of size N in both directions,
 // the coset factors (7 w_M^j)^k / N of every slice (level 2, which also
 // converts canonical coefficients to Montgomery form), the outer twiddles of
-// the quotient INTT and its final scale 7^-k (level 0).  They depend only on
-// the sizes, so a context builds them on first use and reuses them.
+// the quotient INTT with its scale 7^-k, all as constant multipliers (frc).
+// The scale's other part, 7^-(N t) of the cross-slice stage's output t, is a
+// table of s constants on the host.  They depend only on the sizes, so a
+// context builds them on first use and reuses them.
 struct NttSizeArgs {
-  fr* tw_fwd;   // [b * L1 + t] = w_N^(b t), b < L2, t < L1
-  fr* tw_inv;   // [b * L2 + t] = w_N^-(b t), b < L1, t < L2
-  fr* coset;    // [j * N + k] = (7 w_M^j)^k / N   (level 2)
-  fr* outer;    // [j * N + k] = w_M^-(j k)
-  fr* fin;      // [k] = 7^-k                       (level 0)
+  frc* tw_fwd;   // [b * L1 + t] = w_N^(b t), b < L2, t < L1
+  frc* tw_inv;   // [b * L2 + t] = w_N^-(b t), b < L1, t < L2
+  frc* coset;    // [j * N + k] = (7 w_M^j)^k / N, and to level 1
+  frc* outer;    // [j * N + k] = w_M^-(j k) 7^-k, and from level 1
   uint32_t n, lb, l1, l2;
   fr ninv_l2;
   const NttTables* T;
@@ -398,30 +400,28 @@ __global__ void k_ntt_size_tables(NttSizeArgs A, NttTables T) {
   const uint64_t N = 1ull << A.n, M = N << A.lb;
   const uint32_t logm = A.n + A.lb;
   const uint64_t L1 = 1ull << A.l1, L2 = 1ull << A.l2;
-  const uint64_t total = 2 * N + 3 * M;
+  const uint64_t total = 2 * N + 2 * M;
   for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (uint64_t)gridDim.x * blockDim.x) {
     if (e < N) {
       const uint64_t b = e / L1, t = e % L1;
       const uint32_t ex = (uint32_t)((((b * t) & (N - 1)) << (kLog30 - A.n)) & ((1ull << kLog30) - 1));
-      st_fr(A.tw_fwd + e, root_pow(T.wf_lo, T.wf_hi, ex));
+      st_frc(A.tw_fwd + e, frc_of(root_pow(T.wf_lo, T.wf_hi, ex)));
     } else if (e < 2 * N) {
       const uint64_t i = e - N, b = i / L2, t = i % L2;
       const uint32_t ex = (uint32_t)((((b * t) & (N - 1)) << (kLog30 - A.n)) & ((1ull << kLog30) - 1));
-      st_fr(A.tw_inv + i, root_pow(T.wi_lo, T.wi_hi, ex));
+      st_frc(A.tw_inv + i, frc_of(root_pow(T.wi_lo, T.wi_hi, ex)));
     } else if (e < 2 * N + M) {
       const uint64_t i = e - 2 * N, j = i >> A.n, k = i & (N - 1);
       const uint32_t ex = (uint32_t)(((j * k) & (M - 1)) << (kLog30 - logm));
       fr f = fr_mul(fr_mul(ld_fr(T.p7_hi + (k >> kLoBits)), ld_fr(T.p7_lo + (k & kLoMask))),
                     root_pow(T.wf_lo, T.wf_hi, ex));
-      st_fr(A.coset + i, fr_mul(f, A.ninv_l2));
-    } else if (e < 2 * N + 2 * M) {
+      st_frc(A.coset + i, frc_of(fr_mul(f, A.ninv_l2)));
+    } else {
       const uint64_t i = e - 2 * N - M, j = i >> A.n, k = i & (N - 1);
       const uint32_t ex = (uint32_t)(((j * k) & (M - 1)) << (kLog30 - logm));
-      st_fr(A.outer + i, root_pow(T.wi_lo, T.wi_hi, ex));
-    } else {
-      const uint64_t k = e - 2 * N - 2 * M;
-      st_fr(A.fin + k, fr_mul(ld_fr(T.s7_hi + (k >> kLoBits)), ld_fr(T.s7_lo + (k & kLoMask))));
+      const fr s7 = fr_mul(ld_fr(T.s7_hi + (k >> kLoBits)), ld_fr(T.s7_lo + (k & kLoMask)));  // 7^-k, level 0
+      st_frc(A.outer + i, frc_of(fr_mul(root_pow(T.wi_lo, T.wi_hi, ex), s7)));
     }
   }
 }
@@ -431,7 +431,7 @@ __global__ void k_ntt_size_tables(NttSizeArgs A, NttTables T) {
 struct NttSliceTabArgs {
   fr* lo;            // [s][2^hbits] c_j^b (level 1)
   fr* hi;            // [s][2^(n-hbits)] c_j^(a 2^hbits) / N (level 2)
-  fr* zinv;          // [s] (7^N w_s^j - 1)^-1 M^-1 (level 1)
+  frc* zinv;         // [s] (7^N w_s^j - 1)^-1 M^-1
   uint32_t s, n, hbits, logm;
   fr ninv_l2;        // N^-1 at level 2
   fr minv_l1;        // M^-1 at level 1
@@ -464,14 +464,14 @@ __global__ void k_ntt_slice_tables(NttSliceTabArgs A) {
     const uint32_t ex = (j << (kLog30 - (A.logm - A.n))) & ((1u << kLog30) - 1);
     fr zj = fr_sub(fr_mul(s7n, root_pow(A.wf_lo, A.wf_hi, ex)), C->one);
     fr inv = fr_inv_binary(from_mont(zj));        // canonical
-    A.zinv[j] = fr_mul(fr_mul(inv, C->r2), A.minv_l1);
+    A.zinv[j] = frc_of(fr_mul(fr_mul(inv, C->r2), A.minv_l1));
   }
 }
 
 struct NttGateArgs {
   const fr* col[kMaxCols];  // slice evaluations, level 1
   fr* qhat;                 // slice output
-  const fr* zinv;           // constant of this slice
+  const frc* zinv;          // constant of this slice
   const fr* sub;            // nullptr, or values subtracted after the scaling (level 1)
   uint64_t N;
   uint32_t gate, d, c;       // gate word, degree, columns
@@ -480,7 +480,7 @@ struct NttGateArgs {
 // f at the slice points, times the slice constant 1 / (z_H M): Plonk; product
 // q w1 .. w_{d-1} - o; sum g_1 .. g_d + g_{d+1} + .. + g_c (all at level 1).
 __global__ void __launch_bounds__(256) k_ntt_gate(NttGateArgs A) {
-  const fr zi = ld_fr(A.zinv);
+  const frc zi = ld_frc(A.zinv);
   for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < A.N;
        p += (uint64_t)gridDim.x * blockDim.x) {
     fr f;
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(256) k_ntt_gate(NttGateArgs A) {
       else
         for (uint32_t j = A.d; j < A.c; j++) f = fr_add(f, ld_fr(A.col[j] + p));
     }
-    f = fr_mul_inl(zi, f);
+    f = fr_mulc(zi, f);
     if (A.sub) f = fr_sub(f, ld_fr(A.sub + p));
     st_fr(A.qhat + p, f);
   }
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(256) k_ntt_gate(NttGateArgs A) {
 // (qhat - q_big) / kappa, kappa = sigma^M - 7^M.
 
 struct NttStepTabArgs {
-  fr* coset;      // [k] sigma^k / N, level 2
+  frc* coset;     // [k] sigma^k / N, and to level 1
   fr* unscale;    // [k] w_{2M}^-k, level 1
   uint32_t n, shift2m;  // exponent shift of w_{2M} in the 2^30 tables: 30 - log2(2M)
   fr ninv_l2;
@@ -524,7 +524,7 @@ __global__ void k_ntt_step_tables(NttStepTabArgs A) {
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t ex = (uint32_t)((k << A.shift2m) & ((1ull << kLog30) - 1));
     const fr p7 = fr_mul(ld_fr(A.T.p7_hi + (k >> kLoBits)), ld_fr(A.T.p7_lo + (k & kLoMask)));  // 7^k
-    st_fr(A.coset + k, fr_mul(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex)), A.ninv_l2));
+    st_frc(A.coset + k, frc_of(fr_mul(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex)), A.ninv_l2)));
     st_fr(A.unscale + k, root_pow(A.T.wi_lo, A.T.wi_hi, ex));
   }
 }
@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(256) k_ntt_open(NttOpenArgs A, const DevConst*
   const fr* x = A.x[item];
   const uint64_t len = A.len[item];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const fr z32 = ld_fr(A.zpow + 5);
+  const frc z32 = frc_of(ld_fr(A.zpow + 5));
   fr tot = fr_zero();
   const uint64_t nseg = (len + A.seg - 1) / A.seg;
   for (uint64_t sgi = (uint64_t)blockIdx.x * 8 + warp; sgi < nseg; sgi += (uint64_t)gridDim.x * 8) {
@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(256) k_ntt_open(NttOpenArgs A, const DevConst*
       // while the warp's accumulators and values are all zero (the zero top
       // of an honest quotient) the step would multiply zeros: skip it
       if (__all_sync(0xffffffffu, fr_is_zero(acc) && fr_is_zero(xk))) continue;
-      acc = fr_add(fr_mul_inl(z32, acc), xk);
+      acc = fr_add(fr_mulc(z32, acc), xk);
     }
     if (__all_sync(0xffffffffu, fr_is_zero(acc))) continue;
     acc = fr_mul(acc, zpow_of(A.zpow, base + lane, C->one));
@@ -704,15 +704,15 @@ static zc_status ensure_tables(zc_ctx* ctx, cudaStream_t st, NttTables** out) {
   NttTables& T = g_tabs_by_dev[ctx->device];
   if (!T.ready) {
     const size_t n4 = 4096, n15 = 1u << kLoBits;
-    size_t bytes = sizeof(fr) * (2 * n4 + 8 * n15);
+    size_t bytes = sizeof(frc) * 2 * n4 + sizeof(fr) * 8 * n15;
     if (cudaMalloc(&T.mem, bytes) != cudaSuccess) {
       cudaGetLastError();
       ctx->err = "cudaMalloc NTT tables";
       return ZC_ERR_OOM;
     }
-    fr* p = static_cast<fr*>(T.mem);
-    T.dft_fwd = p; p += n4;
-    T.dft_inv = p; p += n4;
+    T.dft_fwd = static_cast<frc*>(T.mem);
+    T.dft_inv = T.dft_fwd + n4;
+    fr* p = reinterpret_cast<fr*>(T.dft_inv + n4);
     T.wf_lo = p; p += n15;
     T.wf_hi = p; p += n15;
     T.wi_lo = p; p += n15;
@@ -743,6 +743,13 @@ static zc_status ensure_tables(zc_ctx* ctx, cudaStream_t st, NttTables** out) {
     a.p7_lo = T.p7_lo; a.p7_hi = T.p7_hi;
     a.w30 = fr_mul_g(w30, C.r2);
     a.w30i = fr_mul_g(h_inv(w30, C), C.r2);
+    {
+      const fr w8 = h_pow(w30, 1ull << 27, C), w8i = h_inv(w8, C);
+      for (int q = 0; q < 3; q++) {
+        T.c_fwd[q] = h_frc(h_pow(w8, q + 1, C), C);
+        T.c_inv[q] = h_frc(h_pow(w8i, q + 1, C), C);
+      }
+    }
     a.seveninv = fr_mul_g(h_inv(seven, C), C.r2);
     a.C = ctx->dconst;
     k_ntt_tables<<<(n15 + 255) / 256, 256, 0, st>>>(a);
@@ -778,6 +785,14 @@ static void ensure_pass_attributes(int dev) {
     set_pass_attributes();
     g_attr_done[dev] = 1;
   }
+}
+
+static void set_dft(NttPassArgs& a, const NttTables* T, bool inverse) {
+  const frc* c = inverse ? T->c_inv : T->c_fwd;
+  a.dft = inverse ? T->dft_inv : T->dft_fwd;
+  a.w8 = c[0];
+  a.w4 = c[1];
+  a.w83 = c[2];
 }
 
 // launch one batched pass over `items` columns
@@ -819,7 +834,7 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
       return &e;
     }
   const uint64_t s = 1ull << lb;
-  const size_t bytes = sizeof(fr) * (2 * N + 3 * M + s);
+  const size_t bytes = sizeof(frc) * (2 * N + 2 * M + 2 * s);
   if (ctx->ntt_cache_frozen || bytes > ctx->ntt_cache_budget) return nullptr;
   size_t used = 0;
   for (auto& e : ctx->ntt_cache) used += e.bytes + e.step_bytes;
@@ -842,26 +857,29 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
   e.lb = lb;
   e.l1 = l1;
   e.bytes = bytes;
-  fr* q = static_cast<fr*>(e.mem);
+  frc* q = static_cast<frc*>(e.mem);
   e.tw_fwd = q; q += N;
   e.tw_inv = q; q += N;
   e.coset = q; q += M;
   e.outer = q; q += M;
-  e.fin = q; q += M;
+  e.fin = q; q += s;
   e.zinv = q;
   {
-    // (z_H on slice j)^-1 M^-1 = (7^N w_s^j - 1)^-1 M^-1, level 1, on the host
+    // on the host: 7^-(N t), t < s; (z_H on slice j)^-1 M^-1 = (7^N w_s^j - 1)^-1 M^-1
     const DevConst& C = ctx->hconst;
     const fr ws = h_pow(T->w32h, (1ull << 32) >> lb, C);
     const fr s7n = h_pow(h_from_u64(7), N, C), minv = h_inv(h_from_u64(M), C);
-    std::vector<fr> zi(s);
-    fr wj = h_from_u64(1);
+    const fr s7i = h_inv(s7n, C);
+    std::vector<frc> hc(2 * s);
+    fr wj = h_from_u64(1), fj = h_from_u64(1);
     for (uint64_t j = 0; j < s; j++) {
       const fr v = fr_sub_g(h_canon_mul(s7n, wj, C), h_from_u64(1));
-      zi[j] = h_canon_mul(h_canon_mul(h_inv(v, C), minv, C), C.one, C);
+      hc[j] = h_frc(fj, C);
+      hc[s + j] = h_frc(h_canon_mul(h_inv(v, C), minv, C), C);
+      fj = h_canon_mul(fj, s7i, C);
       wj = h_canon_mul(wj, ws, C);
     }
-    if (cudaMemcpyAsync(e.zinv, zi.data(), sizeof(fr) * s, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(e.fin, hc.data(), sizeof(frc) * 2 * s, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(e.mem);
@@ -873,7 +891,6 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
   a.tw_inv = e.tw_inv;
   a.coset = e.coset;
   a.outer = e.outer;
-  a.fin = e.fin;
   a.n = n;
   a.lb = lb;
   a.l1 = l1;
@@ -881,7 +898,7 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
   const DevConst& C = ctx->hconst;
   a.ninv_l2 = fr_mul_g(fr_mul_g(h_inv(h_from_u64(N), C), C.r2), C.r2);
   a.C = ctx->dconst;
-  const uint64_t total = 2 * N + 3 * M;
+  const uint64_t total = 2 * N + 2 * M;
   k_ntt_size_tables<<<(unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)ctx->sm_count * 16), 256, 0,
                       st>>>(a, *T);
   ctx->launches++;
@@ -915,7 +932,7 @@ size_t ntt_scratch_bytes(const zc_params* p, int sm_count, bool q_direct) {
   need += align_up(sizeof(fr) * M, 256);                  // qhat (both parts)
   if (!q_direct) need += align_up(sizeof(fr) * M, 256);   // q
   if (D.step) need += 2 * align_up(sizeof(fr) * N, 256);  // q_big reduced, and its LDE
-  need += align_up(sizeof(fr) * s * (nlo + nhi), 256) + align_up(sizeof(fr) * s, 256);
+  need += align_up(sizeof(fr) * s * (nlo + nhi), 256) + align_up(sizeof(frc) * s, 256);
   need += align_up(sizeof(fr) * (c + 1) * nblk_open, 256) + align_up(sizeof(fr) * 32, 256);
   need += align_up(sizeof(NttState), 256) + align_up(psize, 256) + align_up(32 * (size_t)(c + 1), 256);
   need += root_scratch_bytes(c, N) + root_scratch_bytes(1, M) + 8192;
@@ -966,16 +983,15 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
   const uint64_t N = 1ull << n, M = N << lb, parts = 1ull << lb;
   if (n + lb + 1 > (uint32_t)kLog30 || parts > 64) return false;
   const size_t nconst = 8 + parts;
-  const size_t bytes = sizeof(fr) * (2 * N + nconst);
+  const size_t bytes = sizeof(fr) * (3 * N + nconst);
   void* mem = nullptr;
   if (cudaMalloc(&mem, bytes) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  fr* q = static_cast<fr*>(mem);
-  fr* coset = q;
-  fr* unscale = q + N;
-  fr* cst = q + 2 * N;
+  frc* coset = static_cast<frc*>(mem);
+  fr* unscale = reinterpret_cast<fr*>(coset + N);
+  fr* cst = unscale + N;
   const DevConst& C = ctx->hconst;
   // sigma = 7 w_{2M}; kappa = sigma^M - 7^M; z_H on D_small = sigma^N - 1
   const fr w2m = h_pow(T->w32h, (1ull << 32) >> (n + lb + 1), C);
@@ -986,8 +1002,10 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
   const fr ninv = h_inv(h_from_u64(N), C);
   const fr sn = h_pow(sigma, N, C);
   std::vector<fr> hc(nconst, fr_zero());
-  hc[0] = h_canon_mul(h_canon_mul(h_canon_mul(h_inv(fr_sub_g(sn, one), C), kinv, C), ninv, C), C.one, C);
-  hc[1] = h_canon_mul(s7m, C.one, C);
+  const frc zi = h_frc(h_canon_mul(h_canon_mul(h_inv(fr_sub_g(sn, one), C), kinv, C), ninv, C), C);
+  hc[0] = zi.w;
+  hc[1] = zi.q;
+  hc[2] = h_canon_mul(s7m, C.one, C);
   fr pm = one;
   for (uint64_t m = 0; m < parts; m++) {
     hc[8 + m] = h_canon_mul(h_canon_mul(pm, kinv, C), C.one, C);  // level 1
@@ -1027,7 +1045,7 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
 // on load; canonical columns in, canonical codewords out.
 
 struct PcsTabArgs {
-  fr* tab;            // [s w + l] = (7 w_W^s)^l, level 1
+  frc* tab;           // [s w + l] = (7 w_W^s)^l
   uint32_t nc;        // w = 2^nc
   uint32_t shiftW;    // 30 - log2 W
   NttTables T;
@@ -1039,12 +1057,12 @@ __global__ void k_pcs_tables(PcsTabArgs A) {
     const uint32_t s = e >> A.nc, l = e & (w - 1);
     const fr p7 = fr_mul(ld_fr(A.T.p7_hi + (l >> kLoBits)), ld_fr(A.T.p7_lo + (l & kLoMask)));  // 7^l
     const uint32_t ex = (uint32_t)((((uint64_t)s * l) << A.shiftW) & ((1ull << kLog30) - 1));
-    st_fr(A.tab + e, fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex)));
+    st_frc(A.tab + e, frc_of(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex))));
   }
 }
 
 zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uint32_t nc, fr* const* enc,
-                     fr* tab, cudaStream_t st) {
+                     frc* tab, cudaStream_t st) {
   if (nc < 1 || nc > 12 || c < 1 || c > kMaxCols) {
     ctx->err = "pcs: rows of 2 .. 2^12 elements";
     return ZC_ERR_UNSUPPORTED;
@@ -1072,7 +1090,7 @@ zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uin
     a.logL = nc;
     a.in_bs_lo = w; a.in_ts = 1;      // row b, coefficient t
     a.out_bs_lo = 1; a.out_ts = 4 * m;
-    a.dft = T->dft_fwd;
+    set_dft(a, T, false);
     a.pre = PRE_TAB; a.pre_tab = tab + sl * w;
     a.pre_kb = 0; a.pre_kt = 1;
     zc_status rs = run_pass(ctx, st, a, c, m);
@@ -1144,7 +1162,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   fr* vsm = D.step ? ar.take<fr>(N) : nullptr;   // its values on D_small
   fr* tlo = ar.take<fr>(s * nlo);
   fr* thi = ar.take<fr>(s * nhi);
-  fr* zinv = ar.take<fr>(s);
+  frc* zinv = ar.take<frc>(s);
   fr* opart = ar.take<fr>((size_t)(c + 1) * nblk_open);
   fr* zpow = ar.take<fr>(32);
   NttState* dstate = ar.take<NttState>(1);
@@ -1179,7 +1197,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     a.logL = l2;                       // rows of length L2 over i2
     a.in_bs_lo = 1; a.in_ts = L1;      // element (i1, i2) read from e[i1 + L1 i2]
     a.out_bs_lo = L2; a.out_ts = 1;
-    a.dft = T->dft_inv;
+    set_dft(a, T, true);
     a.err = &dstate->err;              // every input element passes through here once
     a.post = POST_TW; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
     a.tw_lbmod = l1; a.tw_shift = kLog30 - n;
@@ -1200,7 +1218,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     a.logL = l1;
     a.in_bs_lo = 1; a.in_ts = L2;
     a.out_bs_lo = 1; a.out_ts = L2;
-    a.dft = T->dft_inv;
+    set_dft(a, T, true);
     return run_pass(ctx, st, a, j1 - j0, L2);
   };
 
@@ -1280,7 +1298,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     a.logL = n;
     a.in_bs_lo = 0; a.in_ts = 1;
     a.out_bs_lo = 0; a.out_ts = 1;
-    a.dft = T->dft_inv;
+    set_dft(a, T, true);
     a.err = &dstate->err;
     if ((rs = run_pass(ctx, st, a, c, 1)) != ZC_OK) return rs;
   }
@@ -1290,7 +1308,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   // slice_lde: the coset NTT of the `items` coefficient vectors in[] into
   // out[] on one slice, with the coset factor table pre (per-size tables)
   // or slice j's two-level tables (without them).
-  auto slice_lde = [&](const fr* const* in, fr* const* out, int items, const fr* pre, uint64_t j,
+  auto slice_lde = [&](const fr* const* in, fr* const* out, int items, const frc* pre, uint64_t j,
                        bool mark) -> zc_status {
     NttPassArgs a;
     pass_defaults(a);
@@ -1302,7 +1320,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     a.pre_lo = tlo + j * nlo;
     a.pre_hi = thi + j * nhi;
     a.pre_shift = hbits;
-    a.dft = T->dft_fwd;
+    set_dft(a, T, false);
     if (two) {
       a.logL = l1;                     // columns over k1: k = L2 k1 + k2
       a.in_bs_lo = 1; a.in_ts = L2;
@@ -1325,7 +1343,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.logL = l2;                     // rows over k2
       a.in_bs_lo = L2; a.in_ts = 1;
       a.out_bs_lo = L2; a.out_ts = 1;
-      a.dft = T->dft_fwd;
+      set_dft(a, T, false);
       if ((rs = run_pass(ctx, st, a, items, L1)) != ZC_OK) return rs;
     } else {
       a.logL = n;
@@ -1341,7 +1359,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     return ZC_OK;
   };
   // gate and division by z_H (constant zi on the slice), minus sub if given
-  auto slice_gate = [&](fr* out, const fr* zi, const fr* sub) {
+  auto slice_gate = [&](fr* out, const frc* zi, const fr* sub) {
     NttGateArgs ga{};
     for (int i = 0; i < c; i++) ga.col[i] = slb[i];
     ga.qhat = out;
@@ -1373,7 +1391,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.logL = l2;                     // rows (j, i2) over i3
       a.in_bs_lo = L2; a.in_ts = 1;
       a.out_bs_lo = L2; a.out_ts = 1;
-      a.dft = T->dft_inv;
+      set_dft(a, T, true);
       a.post = POST_TW; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.tw_lbmod = l1; a.tw_shift = kLog30 - n;
       if (ST) {  // w_N^-(i2 k3) = tw_inv[(b mod L1) L2 + k3]
@@ -1386,10 +1404,11 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.logL = l1;                     // columns (j, k3) over i2 within a slice
       a.in_lbdiv = l2; a.in_bs_hi = N; a.in_bs_lo = 1; a.in_ts = L2;
       a.out_lbdiv = l2; a.out_bs_hi = N; a.out_bs_lo = 1; a.out_ts = L2;
-      a.dft = T->dft_inv;
+      set_dft(a, T, true);
       a.post = POST_OUTER; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.outer_lbdiv = l2; a.tw_shift = kLog30 - logm;
-      if (ST) {  // w_M^-(j k'), k' = L2 k2 + k3: outer[j N + k']
+      if (ST) {  // w_M^-(j k') 7^-k', k' = L2 k2 + k3: outer[j N + k']
+        if (s == 1) a.out[0] = qout;  // no cross-slice stage
         a.post = POST_TAB; a.post_tab = ST->outer;
         a.p_lbdiv = l2; a.p_hs = N; a.p_ls = 1; a.p_ts = L2;
       }
@@ -1400,26 +1419,28 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.logL = n;                      // one row per slice
       a.in_bs_lo = N; a.in_ts = 1;
       a.out_bs_lo = N; a.out_ts = 1;
-      a.dft = T->dft_inv;
+      set_dft(a, T, true);
       a.post = POST_OUTER; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.outer_lbdiv = 0; a.tw_shift = kLog30 - logm;
       if (ST) {
+        if (s == 1) a.out[0] = qout;
         a.post = POST_TAB; a.post_tab = ST->outer;
         a.p_lbdiv = 63; a.p_ls = N; a.p_ts = 1;
       }
       if ((rs = run_pass(ctx, st, a, 1, s)) != ZC_OK) return rs;
     }
+    if (ST && s == 1) return ZC_OK;
     pass_defaults(a);
     a.in[0] = qin; a.out[0] = qout;
     a.logL = lb;                       // across slices
     a.in_bs_lo = 1; a.in_ts = N;
     a.out_bs_lo = 1; a.out_ts = N;
-    a.dft = T->dft_inv;
+    set_dft(a, T, true);
     a.post = POST_FINAL; a.tw_lo = T->s7_lo; a.tw_hi = T->s7_hi;
     a.fin_N = N;
-    if (ST) {  // 7^-k, k = N t + b
+    if (ST) {  // 7^-(N t)
       a.post = POST_TAB; a.post_tab = ST->fin;
-      a.p_lbdiv = 63; a.p_ls = 1; a.p_ts = N;
+      a.p_lbdiv = 63; a.p_ls = 0; a.p_ts = 1;
     }
     if ((rs = run_pass(ctx, st, a, 1, N)) != ZC_OK) return rs;
   }
@@ -1443,12 +1464,12 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     fr* rout[1] = {vsm};
     if ((rs = slice_lde(rin, rout, 1, ST->step_coset, 0, false)) != ZC_OK) return rs;
     if ((rs = slice_lde(coef, slb, c, ST->step_coset, 0, false)) != ZC_OK) return rs;
-    slice_gate(qhat + Mb, ST->step_const, vsm);
+    slice_gate(qhat + Mb, reinterpret_cast<const frc*>(ST->step_const), vsm);
     if ((rs = inverse(qhat + Mb, qv + Mb, 1, 0, n)) != ZC_OK) return rs;
     NttStepCombineArgs ca{};
     ca.q = qv;
     ca.unscale = ST->step_unscale;
-    ca.s7m = ST->step_const + 1;
+    ca.s7m = ST->step_const + 2;
     ca.N = N;
     ca.M = Mb;
     k_ntt_step_combine<<<eg, 256, 0, st>>>(ca);

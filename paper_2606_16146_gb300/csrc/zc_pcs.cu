@@ -272,7 +272,7 @@ zc_status zc_pcs_commit(zc_ctx* ctx, const zc_pcs_params* params, const void* co
   P->S = S;
   // device memory: host-column copies, encodings, coset table, digests, tree
   const size_t bcol = align_up(N * sizeof(fr), 256), benc = align_up(4 * N * sizeof(fr), 256);
-  const size_t btab = align_up(S.W * sizeof(fr), 256), bdig = align_up(S.W * S.c * 32, 256);
+  const size_t btab = align_up(S.W * sizeof(frc), 256), bdig = align_up(S.W * S.c * 32, 256);
   const size_t btree = align_up(2 * S.W * 32, 256);
   const size_t bytes = (cols_on_device ? 0 : bcol * S.c) + benc * S.c + btab + bdig + btree;
   if (cudaMalloc(&P->mem, bytes) != cudaSuccess) {
@@ -300,7 +300,7 @@ zc_status zc_pcs_commit(zc_ctx* ctx, const zc_pcs_params* params, const void* co
     P->enc[j] = reinterpret_cast<fr*>(q);
     q += benc;
   }
-  fr* tab = reinterpret_cast<fr*>(q);
+  frc* tab = reinterpret_cast<frc*>(q);
   q += btab;
   uint32_t* dig = reinterpret_cast<uint32_t*>(q);
   q += bdig;
