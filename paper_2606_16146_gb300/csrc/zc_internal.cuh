@@ -61,6 +61,34 @@ struct NttState {       // NTT per-proof device state
   uint32_t pad[7];
 };
 
+// A table of constant multipliers (frc) in four planes of 16 bytes per entry,
+// so that consecutive lanes read consecutive 16-byte words.
+struct FrcTab {
+  uint4* p = nullptr;
+  size_t n = 0;          // entries per plane
+#if defined(__CUDACC__)
+  __device__ __forceinline__ frc ld(ptrdiff_t i) const {
+    frc c;
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+      const uint4 v = __ldg(p + (i + (ptrdiff_t)(h * n)));
+      uint32_t* d = h < 2 ? c.w.v + 4 * h : c.q.v + 4 * (h - 2);
+      d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+    }
+    return c;
+  }
+  __device__ __forceinline__ void st(size_t i, const frc& c) const {
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+      const uint32_t* d = h < 2 ? c.w.v + 4 * h : c.q.v + 4 * (h - 2);
+      p[i + h * n] = make_uint4(d[0], d[1], d[2], d[3]);
+    }
+  }
+#endif
+  ZC_HD FrcTab at(ptrdiff_t i) const { FrcTab t = *this; t.p += i; return t; }
+  static FrcTab make(void* mem, size_t n) { FrcTab t; t.p = static_cast<uint4*>(mem); t.n = n; return t; }
+};
+
 struct Arena {
   char* base = nullptr;
   size_t cap = 0;
@@ -117,8 +145,8 @@ struct zc_ctx {
     void* mem = nullptr;
     size_t bytes = 0;
     uint64_t stamp = 0;
-    zc::frc *tw_fwd = nullptr, *tw_inv = nullptr, *coset = nullptr, *outer = nullptr;
-    zc::frc* fin = nullptr;   // 7^-(N t), t < s
+    zc::FrcTab tw_fwd, tw_inv, coset, outer;
+    zc::FrcTab fin;           // 7^-(N t), t < s
     zc::frc* zinv = nullptr;  // per slice: (7^N w_s^j - 1)^-1 M^-1
     // step-radix domain 2^lb N + N (built on first use): the small part's
     // coset factors sigma^k / N and sigma^-k 7^k (level 1), k < N,
@@ -127,7 +155,7 @@ struct zc_ctx {
     // m < 2^lb (level 1), kappa = sigma^M - 7^M.
     void* step_mem = nullptr;
     size_t step_bytes = 0;
-    zc::frc* step_coset = nullptr;
+    zc::FrcTab step_coset;
     zc::fr *step_unscale = nullptr, *step_const = nullptr;
   };
   std::vector<NttSizeTables> ntt_cache;
@@ -209,7 +237,7 @@ size_t root_scratch_bytes(int c, uint64_t L);
 // column digests, leaves and tree levels (2W - 1 nodes of 8 words, leaves
 // first) of the encoded columns
 zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uint32_t nc, fr* const* enc,
-                     frc* tab, cudaStream_t st);
+                     FrcTab tab, cudaStream_t st);
 zc_status pcs_hash_tree(zc_ctx* ctx, const fr* const* enc, int c, uint64_t m, uint64_t W, uint32_t* dig,
                         uint32_t* tree, cudaStream_t st);
 void static_constants(DevConst* C, std::vector<fr>* tabs);
@@ -263,10 +291,6 @@ __device__ __forceinline__ void st_fr(fr* p, const fr& x) {
   uint4* q = reinterpret_cast<uint4*>(p);
   q[0] = make_uint4(x.v[0], x.v[1], x.v[2], x.v[3]);
   q[1] = make_uint4(x.v[4], x.v[5], x.v[6], x.v[7]);
-}
-__device__ __forceinline__ void st_frc(frc* p, const frc& c) {
-  st_fr(&p->w, c.w);
-  st_fr(&p->q, c.q);
 }
 __device__ __forceinline__ fr shfl_down_fr(const fr& x, int delta) {
   fr y;

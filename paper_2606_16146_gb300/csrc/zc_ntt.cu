@@ -39,8 +39,7 @@ constexpr int kMaxNttN = 24;
 struct NttTables {
   bool ready = false;
   fr w32h;                 // 7^((r-1)/2^32), canonical, host copy
-  frc* dft_fwd = nullptr;  // w_4096^m, m < 4096
-  frc* dft_inv = nullptr;
+  FrcTab dft_fwd, dft_inv; // the stages' twiddles, see stage_tab
   frc c_fwd[3], c_inv[3];  // w_8, w_4, w_8^3 of each direction (host copies, passed to the kernels by value)
   fr* wf_lo = nullptr;     // w_2^30^b, b < 2^15 (level 1)
   fr* wf_hi = nullptr;     // w_2^30^(a 2^15)
@@ -56,8 +55,17 @@ struct NttTables {
 static NttTables g_tabs_by_dev[64];
 static std::mutex g_tabs_mu;
 
+// Twiddles of the radix-R stage at stride Ns = 8, 64 or 512: w_{Ns R}^{r k},
+// 1 <= r < R, k < Ns, at stage_tab + (r - 1) Ns + k, so that consecutive k are
+// consecutive entries.
+constexpr uint32_t kStageTab = 11 * (8 + 64 + 512);
+__host__ __device__ __forceinline__ uint32_t stage_tab(uint32_t logNs, uint32_t lr) {
+  const uint32_t Ns = 1u << logNs;
+  return 11 * ((Ns - 8) / 7) + (lr == 3 ? 0 : lr == 2 ? 7 * Ns : 10 * Ns);
+}
+
 struct NttTabArgs {
-  frc* dft_fwd; frc* dft_inv; fr* wf_lo; fr* wf_hi; fr* wi_lo; fr* wi_hi; fr* s7_lo; fr* s7_hi;
+  FrcTab dft_fwd, dft_inv; fr* wf_lo; fr* wf_hi; fr* wi_lo; fr* wi_hi; fr* s7_lo; fr* s7_hi;
   fr* p7_lo; fr* p7_hi;
   fr w30;        // 2^30-th root (level 1)
   fr w30i;       // its inverse (level 1)
@@ -78,10 +86,12 @@ __device__ fr fr_pow_dev(fr base, uint64_t e, const DevConst* C) {  // level 1 i
 __global__ void k_ntt_tables(NttTabArgs A) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const DevConst* C = A.C;
-  if (i < 4096) {
-    // w_4096 = w30^(2^18)
-    A.dft_fwd[i] = frc_of(fr_pow_dev(A.w30, (uint64_t)i << 18, C));
-    A.dft_inv[i] = frc_of(fr_pow_dev(A.w30i, (uint64_t)i << 18, C));
+  if (i < kStageTab) {
+    const uint32_t logNs = i < 88 ? 3 : i < 792 ? 6 : 9, e = i - stage_tab(logNs, 3), Ns = 1u << logNs;
+    const uint32_t lr = e < 7 * Ns ? 3 : e < 10 * Ns ? 2 : 1, g = i - stage_tab(logNs, lr);
+    const uint64_t ex = (uint64_t)((g / Ns + 1) * (g % Ns)) << (30 - logNs - lr);  // r k
+    A.dft_fwd.st(i, frc_of(fr_pow_dev(A.w30, ex, C)));
+    A.dft_inv.st(i, frc_of(fr_pow_dev(A.w30i, ex, C)));
   }
   if (i < (1u << kLoBits)) {
     A.wf_lo[i] = fr_pow_dev(A.w30, i, C);
@@ -105,36 +115,51 @@ __device__ __forceinline__ fr root_pow(const fr* lo, const fr* hi, uint32_t e) {
 enum { PRE_NONE = 0, PRE_COSET = 1, PRE_TAB = 2 };
 enum { POST_NONE = 0, POST_TW = 1, POST_OUTER = 2, POST_FINAL = 3, POST_TAB = 4 };
 
+// Index of element t of sub-DFT b in a column or a factor table; every stride
+// is a power of two: ((b >> div) << hs) + ((b & mask) << ls) + (t << ts).
+struct NttMap {
+  uint32_t div, hs, mask, ls, ts;
+  __device__ __forceinline__ uint32_t at(uint32_t b, uint32_t t) const {
+    return ((b >> div) << hs) + ((b & mask) << ls) + (t << ts);
+  }
+};
+constexpr uint32_t kNone = 31;  // a shift that leaves nothing of b < 2^31
+// b << ls, t << ts
+static NttMap map_flat(uint32_t ls, uint32_t ts) { return NttMap{kNone, 0, 0xffffffffu, ls, ts}; }
+// (b >> div) << hs, (b mod 2^div) << ls, t << ts
+static NttMap map_split(uint32_t div, uint32_t hs, uint32_t ls, uint32_t ts) {
+  return NttMap{div, hs, (1u << div) - 1, ls, ts};
+}
+// the low div bits of b only
+static NttMap map_low(uint32_t div, uint32_t ls, uint32_t ts) {
+  return NttMap{kNone, 0, (1u << div) - 1, ls, ts};
+}
+
 struct NttPassArgs {
   const fr* in[kMaxCols];
   fr* out[kMaxCols];
   uint32_t items;         // columns in this launch
   uint32_t logL;          // sub-DFT length
   uint32_t logW;          // sub-DFTs per CTA
-  // element (b, t) address: ((b >> lbdiv) * bs_hi) + (b & (bdiv-1)) * bs_lo + t * ts
-  uint32_t in_lbdiv, out_lbdiv;
-  uint64_t in_bs_hi, in_bs_lo, in_ts;
-  uint64_t out_bs_hi, out_bs_lo, out_ts;
-  const frc* dft;         // 4096-th roots, forward or inverse
-  frc w8, w4, w83;        // their powers 512, 1024, 1536
+  uint32_t B;             // sub-DFTs (a CTA's surplus ones are neither read nor written)
+  NttMap im, om;          // element (b, t) of a column
+  FrcTab dft;             // stage twiddles, forward or inverse
+  frc w8, w4, w83;        // w_8, w_4, w_8^3
   int pre;
-  const fr* pre_lo;       // per-item coset tables (item stride pre_stride)
+  NttMap pm;              // PRE_TAB: factor pre_tab[pm]; PRE_COSET: k = pm, factor hi[k >> shift] lo[k & mask]
+  FrcTab pre_tab;
+  const fr* pre_lo;
   const fr* pre_hi;
-  uint32_t pre_shift;     // k = b * pre_kb + t * pre_kt; factor = hi[k >> shift] * lo[k & mask]
-  uint64_t pre_kb, pre_kt;
+  uint32_t pre_shift;
   int post;
+  NttMap qm;              // POST_TAB: factor post_tab[qm]
+  FrcTab post_tab;
   const fr* tw_lo;
   const fr* tw_hi;
   uint32_t tw_lbmod;      // POST_TW: e = (b mod 2^lbmod) * t
   uint32_t tw_shift;      // exponent in the 2^30 table: (e mod 2^(30-shift)) << shift
   uint32_t outer_lbdiv;   // POST_OUTER: e = (b >> lbdiv) * ((t << lbdiv) + (b mod 2^lbdiv))
-  uint64_t fin_N;         // POST_FINAL: k = fin_N * t + b
-  // table modes: PRE_TAB factor = pre_tab[b * pre_kb + t * pre_kt];
-  // POST_TAB factor = post_tab[(b >> p_lbdiv) * p_hs + (b & (2^p_lbdiv - 1)) * p_ls + t * p_ts]
-  const frc* pre_tab;
-  const frc* post_tab;
-  uint32_t p_lbdiv;
-  uint64_t p_hs, p_ls, p_ts;
+  uint32_t fin_logN;      // POST_FINAL: k = (t << fin_logN) + b
   uint32_t* err;          // if set: the pass reads the proof's input columns, and a value >= r sets bit 0
 };
 
@@ -185,8 +210,8 @@ struct SmTile {
   uint4* p;     // plane 0: p[0, T), plane 1: p[T, 2T)
   uint32_t T;
   __device__ __forceinline__ uint32_t sw(uint32_t i) const { return i ^ ((i >> 3) & 7); }
-  __device__ __forceinline__ fr get(uint32_t i) const {
-    const uint32_t s = sw(i);
+  __device__ __forceinline__ fr get(uint32_t i) const { return get_at(sw(i)); }
+  __device__ __forceinline__ fr get_at(uint32_t s) const {
     const uint4 a = p[s], b = p[T + s];
     fr x;
     x.v[0] = a.x; x.v[1] = a.y; x.v[2] = a.z; x.v[3] = a.w;
@@ -200,180 +225,195 @@ struct SmTile {
   }
 };
 
-// One Stockham stage of radix R = 2^lr on the CTA tile sm[t * W + w]; each
-// thread owns 8 elements (8 / R independent groups).
-template <int LR>
-__device__ __forceinline__ void stockham_stage(const SmTile& sm, uint32_t logL, uint32_t logW,
-                                               uint32_t logNs, const NttPassArgs& A) {
-  constexpr int R = 1 << LR;
-  constexpr int GROUPS = 8 / R;
-  const uint32_t L = 1u << logL, W = 1u << logW;
-  const uint32_t qL = L >> LR;   // L / R
-  const uint32_t ngroups = (L << logW) >> LR;
-  fr x[8];
-  uint32_t jj[GROUPS], ww[GROUPS];
-#pragma unroll
-  for (int g = 0; g < GROUPS; g++) {
-    uint32_t j_all = threadIdx.x * GROUPS + g;
-    uint32_t w = j_all & (W - 1), j = j_all >> logW;
-    jj[g] = j;
-    ww[g] = w;
-    if (j_all < ngroups) {
-#pragma unroll
-      for (int r = 0; r < R; r++) x[g * R + r] = sm.get((j + r * qL) * W + w);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int g = 0; g < GROUPS; g++) {
-    if (threadIdx.x * GROUPS + g >= ngroups) continue;
-    const uint32_t j = jj[g];
-    const uint32_t k = j & ((1u << logNs) - 1);
-    if (logNs > 0) {
-      // the previous stage left its outputs lazy: x[0] is reduced, the
-      // others are reduced by their twiddle w_{Ns R}^{r k} = dft[r k 4096 / (Ns R)]
-      const uint32_t sh = 12 - (logNs + LR);
-      x[g * R] = fr_reduce1(x[g * R]);
-#pragma unroll
-      for (int r = 1; r < R; r++) x[g * R + r] = fr_mulc(ld_frc(A.dft + ((r * k) << sh)), x[g * R + r]);
-    }
-    if (R == 8) {
-      fr y[8];
-#pragma unroll
-      for (int r = 0; r < 8; r++) y[r] = x[r];
-      dft8(y, A);
-#pragma unroll
-      for (int r = 0; r < 8; r++) x[r] = y[r];
-    } else if (R == 4) {
-      dft4<2>(x[g * 4], x[g * 4 + 1], x[g * 4 + 2], x[g * 4 + 3], A.w4);
-    } else {
-      fr a = x[g * 2], b = x[g * 2 + 1];
-      x[g * 2] = fr_add_lazy(a, b);
-      x[g * 2 + 1] = fr_sub_lazy(a, b);
-    }
-  }
-#pragma unroll
-  for (int g = 0; g < GROUPS; g++) {
-    if (threadIdx.x * GROUPS + g >= ngroups) continue;
-    const uint32_t j = jj[g], w = ww[g];
-    const uint32_t k = j & ((1u << logNs) - 1);
-    const uint32_t idxD = ((j >> logNs) << (logNs + LR)) + k;
-#pragma unroll
-    for (int r = 0; r < R; r++) sm.put((idxD + (r << logNs)) * W + w, x[g * R + r]);
-  }
-  __syncthreads();
-}
-
-template <int TILE, int MINB>
-__global__ void __launch_bounds__(TILE / 8, MINB) k_ntt_pass(NttPassArgs A) {
+// One pass: the sub-DFTs b of length L = 2^logL over strided elements, W of
+// them per CTA, blockDim.x = L W / 8 threads with 8 elements each.
+//
+// Every stage reads element tid + NT p of the tile into register p (NT =
+// blockDim.x, p < 8), so its radix-R groups are the registers p that agree
+// modulo 8 / R, whatever L, W and the stage.  The factors of a step (the pre
+// table before the first stage, the twiddles before the others, the post
+// table before the store) go through one copy of the code.
+//
+// What bounds it: the wide multiply-adds of the ~6 products per element (the
+// multiplier pipe is 77 % busy in the first N2 pass at n = 20, 699 us; reading
+// elements and factors one per lane it was 67 %, 769 us), then the latency of
+// 16 warps per SM.  Why the pass looks as it does: 32- and 64-byte elements
+// read one per lane made every request touch 16 to 32 lines (L1 75 % busy, now
+// 22 %), so columns move in 16-byte halves, two lanes to an element, and
+// factors lie in 16-byte planes in the order the lanes read them; products
+// inlined at each use were 75 KB of instructions, more than the instruction
+// cache keeps, hence the shared step; address arithmetic competes for the
+// multiplier pipe, hence the FAST form (8.21 -> 8.02 ms for the proof).
+// FAST: whole tiles of sub-DFTs of at least 8 points, 64 threads or more, all
+// factors from tables; slot p's addresses are slot 0's plus a uniform offset.
+// The general form also takes short sub-DFTs, a part-filled tile (sub-DFTs
+// past the last one repeat it and are not stored) and the two-level power
+// tables.
+template <int MAXT, int MINB, bool FAST>
+__global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   extern __shared__ __align__(16) uint4 sm_planes[];
-  const SmTile sm{sm_planes, (uint32_t)TILE};
+  const uint32_t NT = blockDim.x, tid = threadIdx.x;
+  const SmTile sm{sm_planes, NT * 8};
   // items (columns) vary fastest across consecutive CTAs, so the per-element
   // factor tables, shared by every column, are reused from L2
-  const uint32_t items = A.items;
-  const int item = (int)(blockIdx.x % items);
-  const uint64_t blk = blockIdx.x / items;
-  const fr* __restrict__ in = A.in[item];
-  fr* out = A.out[item];
-  const uint32_t logL = A.logL, logW = A.logW;
-  const uint32_t L = 1u << logL, W = 1u << logW;
-  const uint64_t b0 = blk << logW;
-  const uint32_t n_el = L << logW;  // <= TILE (smaller only for tiny transforms)
-  const bool in_t_fast = A.in_ts == 1, out_t_fast = A.out_ts == 1;
-  const uint64_t in_bdiv_mask = (1ull << A.in_lbdiv) - 1, out_bdiv_mask = (1ull << A.out_lbdiv) - 1;
-
-  // ---- load (with the coset factor when asked)
-  if (A.pre == PRE_NONE && n_el == (uint32_t)TILE) {
-    // no factor to apply: both 16-byte halves of every element go straight
-    // from global to their planes (cp.async, no register staging), all of
-    // this thread's copies in flight together
+  const uint32_t item = blockIdx.x % A.items;
+  const uint32_t logL = A.logL, logW = A.logW, Wm = (1u << logW) - 1, tq = (1u << logL) >> 3;
+  const uint32_t b0 = (blockIdx.x / A.items) << logW;
+  // the sub-DFT and the element of tile element i
+  auto sub = [&](uint32_t i) { return FAST ? b0 + (i & Wm) : min(b0 + (i & Wm), A.B - 1); };
+  auto elt = [&](uint32_t i) { return i >> logW; };
+  // index of tile element i, and from i0 to i0 + NT p (FAST: p tq elements
+  // further on; otherwise it may go back)
+  auto index = [&](const NttMap& m, uint32_t i) { return m.at(sub(i), elt(i)); };
+  auto step = [&](const NttMap& m, uint32_t i0, int p) -> ptrdiff_t {
+    return FAST ? (ptrdiff_t)(p * (tq << m.ts)) : (ptrdiff_t)index(m, i0 + NT * p) - (ptrdiff_t)index(m, i0);
+  };
+  // The column's elements come through shared memory in 16-byte halves, two
+  // lanes to an element; a warp copies its own slots only.
+  {
+    const uint32_t half = tid & 1;
+    const char* in = reinterpret_cast<const char*>(A.in[item]) + 16 * half;
 #pragma unroll
-    for (int u = 0; u < 8; u++) {
-      const uint32_t idx = threadIdx.x + (uint32_t)u * (TILE / 8);
-      uint32_t w, t;
-      if (in_t_fast) { t = idx & (L - 1); w = idx >> logL; }
-      else { w = idx & (W - 1); t = idx >> logW; }
-      const uint64_t b = b0 + w;
-      const uint64_t a = (b >> A.in_lbdiv) * A.in_bs_hi + (b & in_bdiv_mask) * A.in_bs_lo + t * A.in_ts;
-      const uint32_t s = sm.sw(t * W + w);
-      const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(sm.p + s);
-      const uint32_t d1 = (uint32_t)__cvta_generic_to_shared(sm.p + TILE + s);
-      const char* g = reinterpret_cast<const char*>(in + a);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0), "l"(g) : "memory");
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d1), "l"(g + 16) : "memory");
-    }
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-    if (A.err) {
-      // the input check reads back what this thread copied
+    for (int s = 0; s < 2; s++) {
+      const uint32_t i = (tid & ~31u) + ((tid & 31) >> 1) + 16 * s;
+      const char* g = in + sizeof(fr) * (size_t)index(A.im, i);
 #pragma unroll
-      for (int u = 0; u < 8; u++) {
-        const uint32_t idx = threadIdx.x + (uint32_t)u * (TILE / 8);
-        uint32_t w, t;
-        if (in_t_fast) { t = idx & (L - 1); w = idx >> logL; }
-        else { w = idx & (W - 1); t = idx >> logW; }
-        if (!fr_is_canonical(sm.get(t * W + w))) atomicOr(A.err, 1u);
+      for (int p = 0; p < 8; p++) {
+        const uint32_t sl = FAST ? sm.sw(i) + NT * p : sm.sw(i + NT * p);
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(sm.p + sm.T * half + sl);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(g + (ptrdiff_t)sizeof(fr) * step(A.im, i, p))
+                     : "memory");
       }
     }
-  } else
-  for (uint32_t idx = threadIdx.x; idx < n_el; idx += blockDim.x) {
-    uint32_t w, t;
-    if (in_t_fast) { t = idx & (L - 1); w = idx >> logL; }
-    else { w = idx & (W - 1); t = idx >> logW; }
-    const uint64_t b = b0 + w;
-    const uint64_t a = (b >> A.in_lbdiv) * A.in_bs_hi + (b & in_bdiv_mask) * A.in_bs_lo + t * A.in_ts;
-    fr x = ld_fr(in + a);
-    if (A.err && !fr_is_canonical(x)) atomicOr(A.err, 1u);
-    if (A.pre == PRE_TAB) {
-      x = fr_mulc(ld_frc(A.pre_tab + b * A.pre_kb + t * A.pre_kt), x);
-    } else if (A.pre == PRE_COSET) {
-      const uint64_t k = b * A.pre_kb + t * A.pre_kt;
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+  }
+  // slot p of this thread (NT is a multiple of 64 in the FAST form: the swizzle of slot 0 serves all)
+  auto get = [&](int p) { return FAST ? sm.get_at(sm.sw(tid) + NT * p) : sm.get(tid + NT * p); };
+  fr x[8];
+#pragma unroll
+  for (int p = 0; p < 8; p++) x[p] = get(p);
+  if (A.err) {
+    bool bad = false;
+#pragma unroll
+    for (int p = 0; p < 8; p++) bad |= !fr_is_canonical(x[p]);
+    if (bad) atomicOr(A.err, 1u);
+  }
+  if (!FAST && A.pre == PRE_COSET) {
+#pragma unroll
+    for (int p = 0; p < 8; p++) {
+      const uint32_t k = index(A.pm, tid + NT * p);
       // one slice per launch: every column uses the same tables
-      fr f = fr_mul(ld_fr(A.pre_hi + (k >> A.pre_shift)),
-                    ld_fr(A.pre_lo + (k & ((1ull << A.pre_shift) - 1))));
-      x = fr_mul(x, f);
+      x[p] = fr_mul(fr_mul(ld_fr(A.pre_hi + (k >> A.pre_shift)), ld_fr(A.pre_lo + (k & ((1u << A.pre_shift) - 1)))),
+                    x[p]);
     }
-    sm.put(t * W + w, x);
   }
-  __syncthreads();
-
-  // ---- Stockham stages: radix 8 while >= 3 bits remain, then 4 or 2
+  const bool post_tab = A.post == POST_TAB;
   uint32_t logNs = 0;
-  while (logL - logNs >= 3) {
-    stockham_stage<3>(sm, logL, logW, logNs, A);
-    logNs += 3;
-  }
-  if (logL - logNs == 2) stockham_stage<2>(sm, logL, logW, logNs, A);
-  else if (logL - logNs == 1) stockham_stage<1>(sm, logL, logW, logNs, A);
-
-  // ---- store (with the twiddle / final scale)
-  for (uint32_t idx = threadIdx.x; idx < n_el; idx += blockDim.x) {
-    uint32_t w, t;
-    if (out_t_fast) { t = idx & (L - 1); w = idx >> logL; }
-    else { w = idx & (W - 1); t = idx >> logW; }
-    const uint64_t b = b0 + w;
-    fr y = sm.get(t * W + w);  // lazily reduced: multiplied (as the second operand) or reduced here
-    if (A.post == POST_TAB) {
-      const uint64_t ti = (b >> A.p_lbdiv) * A.p_hs + (b & ((1ull << A.p_lbdiv) - 1)) * A.p_ls + t * A.p_ts;
-      y = fr_mulc(ld_frc(A.post_tab + ti), y);
-    } else if (A.post == POST_TW) {
-      const uint64_t e = (b & ((1ull << A.tw_lbmod) - 1)) * t;
-      const uint32_t ex = (uint32_t)((e << A.tw_shift) & ((1ull << kLog30) - 1));
-      y = ex ? fr_mul(root_pow(A.tw_lo, A.tw_hi, ex), y) : fr_reduce1(y);
-    } else if (A.post == POST_OUTER) {
-      const uint64_t jsl = b >> A.outer_lbdiv;
-      const uint64_t kp = ((uint64_t)t << A.outer_lbdiv) + (b & ((1ull << A.outer_lbdiv) - 1));
-      const uint64_t e = jsl * kp;
-      const uint32_t ex = (uint32_t)((e << A.tw_shift) & ((1ull << kLog30) - 1));
-      y = ex ? fr_mul(root_pow(A.tw_lo, A.tw_hi, ex), y) : fr_reduce1(y);
-    } else if (A.post == POST_FINAL) {
-      const uint64_t k = A.fin_N * t + b;
-      fr f = fr_mul(ld_fr(A.tw_hi + (k >> kLoBits)), ld_fr(A.tw_lo + (k & kLoMask)));  // level 0
-      y = fr_mul(f, y);
-    } else {
-      y = fr_reduce1(y);
+  bool fin = false;  // the step after the last stage: the post table
+#pragma unroll 1
+  while (true) {
+    const uint32_t lr = min(3u, logL - logNs), lg = 3 - lr;  // radix R, and the 8 / R groups, as logs
+    // factors: pre or post table, or the twiddles w_{Ns R}^{r k}, r = p >> lg
+    // (for r = 0 the previous stage's lazy output is only reduced)
+    const bool tw = !fin && logNs > 0, all = fin || (logNs == 0 && A.pre == PRE_TAB);
+    if (tw || all) {
+      const FrcTab base = tw ? A.dft : fin ? A.post_tab : A.pre_tab;
+      const NttMap m = fin ? A.qm : A.pm;
+      // group g's sub-DFT element is j + g tq; only a last stage has several
+      // groups, and there k = j
+      const uint32_t j = elt(tid), km = (1u << logNs) - 1;
+      const FrcTab first = base.at(tw ? (ptrdiff_t)(stage_tab(logNs, lr) + (FAST ? j & km : 0)) - (ptrdiff_t)(km + 1)
+                                     : (ptrdiff_t)index(m, tid));
+      auto fac = [&](int p) {
+        if (tw) {
+          const uint32_t g = p & ((1u << lg) - 1), r = (uint32_t)p >> lg;
+          return first.ld((r << logNs) + (FAST ? g * tq : elt(tid + NT * g) & km));
+        }
+        return first.ld(step(m, tid, p));
+      };
+#pragma unroll
+      for (int p = 7; p >= 4; p--) x[p] = fr_mulc(fac(p), x[p]);
+      if (all || lr >= 2) {
+        x[3] = fr_mulc(fac(3), x[3]);
+        x[2] = fr_mulc(fac(2), x[2]);
+      } else {
+        x[3] = fr_reduce1(x[3]);
+        x[2] = fr_reduce1(x[2]);
+      }
+      if (all || lr == 3) x[1] = fr_mulc(fac(1), x[1]);
+      else x[1] = fr_reduce1(x[1]);
+      if (all) x[0] = fr_mulc(fac(0), x[0]);
+      else x[0] = fr_reduce1(x[0]);
     }
-    const uint64_t a = (b >> A.out_lbdiv) * A.out_bs_hi + (b & out_bdiv_mask) * A.out_bs_lo + t * A.out_ts;
-    st_fr(out + a, y);
+    if (fin) break;
+    if (lr == 3) {
+      dft8(x, A);
+    } else if (lr == 2) {
+      dft4<2>(x[0], x[2], x[4], x[6], A.w4);
+      dft4<2>(x[1], x[3], x[5], x[7], A.w4);
+    } else if (lr == 1) {
+#pragma unroll
+      for (int g = 0; g < 4; g++) {
+        const fr u = x[g], v = x[g + 4];
+        x[g] = fr_add_lazy(u, v);
+        x[g + 4] = fr_sub_lazy(u, v);
+      }
+    }
+    if (logNs + lr == logL) {
+      if (!post_tab) break;
+      fin = true;
+      continue;
+    }
+    // element (j, r) of the stage goes to (j / Ns) Ns R + j mod Ns + r Ns
+    const uint32_t ls = logNs + logW;
+    __syncthreads();  // every slot has been read
+#pragma unroll
+    for (int p = 0; p < 8; p++) {
+      const uint32_t ja = tid + NT * (p & ((1u << lg) - 1)), r = (uint32_t)p >> lg;
+      sm.put(((ja >> ls) << (ls + lr)) + (ja & ((1u << ls) - 1)) + (r << ls), x[p]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < 8; p++) x[p] = get(p);
+    logNs += lr;
+  }
+
+  // ---- store, two lanes to an element as in the load: a lane keeps one half
+  // of its own element and swaps the other for that half of its neighbour's.
+  // Without a post table the values are lazy: reduced, or multiplied here.
+  const bool odd = tid & 1;
+  char* const out = reinterpret_cast<char*>(A.out[item]) + 16 * odd;
+  char* const oe = out + sizeof(fr) * (size_t)index(A.om, tid & ~1u);  // the even lane's element
+  char* const oo = out + sizeof(fr) * (size_t)index(A.om, tid | 1u);
+#pragma unroll
+  for (int p = 0; p < 8; p++) {
+    fr y = x[p];
+    if (!post_tab) {
+      const uint32_t b = sub(tid + NT * p), t = elt(tid + NT * p);
+      if (FAST || A.post == POST_NONE) {
+        y = fr_reduce1(y);
+      } else if (A.post == POST_FINAL) {
+        const uint32_t k = (t << A.fin_logN) + b;
+        y = fr_mul(fr_mul(ld_fr(A.tw_hi + (k >> kLoBits)), ld_fr(A.tw_lo + (k & kLoMask))), y);  // level 0
+      } else {
+        const uint32_t dm = (1u << A.outer_lbdiv) - 1;
+        const uint64_t e = A.post == POST_TW ? (uint64_t)(b & ((1u << A.tw_lbmod) - 1)) * t
+                                             : (uint64_t)(b >> A.outer_lbdiv) * ((t << A.outer_lbdiv) + (b & dm));
+        const uint32_t ex = (uint32_t)((e << A.tw_shift) & ((1ull << kLog30) - 1));
+        y = ex ? fr_mul(root_pow(A.tw_lo, A.tw_hi, ex), y) : fr_reduce1(y);
+      }
+    }
+    uint32_t r[4];
+#pragma unroll
+    for (int h = 0; h < 4; h++) r[h] = __shfl_xor_sync(0xffffffffu, odd ? y.v[h] : y.v[4 + h], 1);
+    const bool le = FAST || b0 + (((tid & ~1u) + NT * p) & Wm) < A.B, lo = FAST || b0 + (((tid | 1u) + NT * p) & Wm) < A.B;
+    if (le)
+      *reinterpret_cast<uint4*>(oe + (ptrdiff_t)sizeof(fr) * step(A.om, tid & ~1u, p)) =
+          odd ? make_uint4(r[0], r[1], r[2], r[3]) : make_uint4(y.v[0], y.v[1], y.v[2], y.v[3]);
+    if (lo)
+      *reinterpret_cast<uint4*>(oo + (ptrdiff_t)sizeof(fr) * step(A.om, tid | 1u, p)) =
+          odd ? make_uint4(y.v[4], y.v[5], y.v[6], y.v[7]) : make_uint4(r[0], r[1], r[2], r[3]);
   }
 }
 
@@ -386,15 +426,20 @@ __global__ void __launch_bounds__(TILE / 8, MINB) k_ntt_pass(NttPassArgs A) {
 // table of s constants on the host.  They depend only on the sizes, so a
 // context builds them on first use and reuses them.
 struct NttSizeArgs {
-  frc* tw_fwd;   // [b * L1 + t] = w_N^(b t), b < L2, t < L1
-  frc* tw_inv;   // [b * L2 + t] = w_N^-(b t), b < L1, t < L2
-  frc* coset;    // [j * N + k] = (7 w_M^j)^k / N, and to level 1
-  frc* outer;    // [j * N + k] = w_M^-(j k) 7^-k, and from level 1
+  FrcTab tw_fwd;   // [b * L1 + t] = w_N^(b t), b < L2, t < L1
+  FrcTab tw_inv;   // [b * L2 + t] = w_N^-(b t), b < L1, t < L2
+  FrcTab coset;    // [j * N + pos(k)] = (7 w_M^j)^k / N, and to level 1
+  FrcTab outer;    // [j * N + pos(k)] = w_M^-(j k) 7^-k, and from level 1
   uint32_t n, lb, l1, l2;
   fr ninv_l2;
   const NttTables* T;
   const DevConst* C;
 };
+
+// coefficient k = L2 t + b at entry L1 b + t: the passes over t read consecutive entries
+__host__ __device__ __forceinline__ uint64_t tab_pos(uint64_t k, uint32_t l1, uint32_t l2) {
+  return ((k & ((1ull << l2) - 1)) << l1) + (k >> l2);
+}
 
 __global__ void k_ntt_size_tables(NttSizeArgs A, NttTables T) {
   const uint64_t N = 1ull << A.n, M = N << A.lb;
@@ -406,22 +451,22 @@ __global__ void k_ntt_size_tables(NttSizeArgs A, NttTables T) {
     if (e < N) {
       const uint64_t b = e / L1, t = e % L1;
       const uint32_t ex = (uint32_t)((((b * t) & (N - 1)) << (kLog30 - A.n)) & ((1ull << kLog30) - 1));
-      st_frc(A.tw_fwd + e, frc_of(root_pow(T.wf_lo, T.wf_hi, ex)));
+      A.tw_fwd.st(e, frc_of(root_pow(T.wf_lo, T.wf_hi, ex)));
     } else if (e < 2 * N) {
       const uint64_t i = e - N, b = i / L2, t = i % L2;
       const uint32_t ex = (uint32_t)((((b * t) & (N - 1)) << (kLog30 - A.n)) & ((1ull << kLog30) - 1));
-      st_frc(A.tw_inv + i, frc_of(root_pow(T.wi_lo, T.wi_hi, ex)));
+      A.tw_inv.st(i, frc_of(root_pow(T.wi_lo, T.wi_hi, ex)));
     } else if (e < 2 * N + M) {
       const uint64_t i = e - 2 * N, j = i >> A.n, k = i & (N - 1);
       const uint32_t ex = (uint32_t)(((j * k) & (M - 1)) << (kLog30 - logm));
       fr f = fr_mul(fr_mul(ld_fr(T.p7_hi + (k >> kLoBits)), ld_fr(T.p7_lo + (k & kLoMask))),
                     root_pow(T.wf_lo, T.wf_hi, ex));
-      st_frc(A.coset + i, frc_of(fr_mul(f, A.ninv_l2)));
+      A.coset.st((j << A.n) + tab_pos(k, A.l1, A.l2), frc_of(fr_mul(f, A.ninv_l2)));
     } else {
       const uint64_t i = e - 2 * N - M, j = i >> A.n, k = i & (N - 1);
       const uint32_t ex = (uint32_t)(((j * k) & (M - 1)) << (kLog30 - logm));
       const fr s7 = fr_mul(ld_fr(T.s7_hi + (k >> kLoBits)), ld_fr(T.s7_lo + (k & kLoMask)));  // 7^-k, level 0
-      st_frc(A.outer + i, frc_of(fr_mul(root_pow(T.wi_lo, T.wi_hi, ex), s7)));
+      A.outer.st((j << A.n) + tab_pos(k, A.l1, A.l2), frc_of(fr_mul(root_pow(T.wi_lo, T.wi_hi, ex), s7)));
     }
   }
 }
@@ -512,9 +557,9 @@ __global__ void __launch_bounds__(256) k_ntt_gate(NttGateArgs A) {
 // (qhat - q_big) / kappa, kappa = sigma^M - 7^M.
 
 struct NttStepTabArgs {
-  frc* coset;     // [k] sigma^k / N, and to level 1
+  FrcTab coset;   // [pos(k)] sigma^k / N, and to level 1
   fr* unscale;    // [k] w_{2M}^-k, level 1
-  uint32_t n, shift2m;  // exponent shift of w_{2M} in the 2^30 tables: 30 - log2(2M)
+  uint32_t n, l1, l2, shift2m;  // exponent shift of w_{2M} in the 2^30 tables: 30 - log2(2M)
   fr ninv_l2;
   NttTables T;
 };
@@ -524,7 +569,7 @@ __global__ void k_ntt_step_tables(NttStepTabArgs A) {
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t ex = (uint32_t)((k << A.shift2m) & ((1ull << kLog30) - 1));
     const fr p7 = fr_mul(ld_fr(A.T.p7_hi + (k >> kLoBits)), ld_fr(A.T.p7_lo + (k & kLoMask)));  // 7^k
-    st_frc(A.coset + k, frc_of(fr_mul(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex)), A.ninv_l2)));
+    A.coset.st(tab_pos(k, A.l1, A.l2), frc_of(fr_mul(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex)), A.ninv_l2)));
     st_fr(A.unscale + k, root_pow(A.T.wi_lo, A.T.wi_hi, ex));
   }
 }
@@ -703,16 +748,16 @@ static zc_status ensure_tables(zc_ctx* ctx, cudaStream_t st, NttTables** out) {
   std::lock_guard<std::mutex> lk(g_tabs_mu);
   NttTables& T = g_tabs_by_dev[ctx->device];
   if (!T.ready) {
-    const size_t n4 = 4096, n15 = 1u << kLoBits;
+    const size_t n4 = kStageTab, n15 = 1u << kLoBits;
     size_t bytes = sizeof(frc) * 2 * n4 + sizeof(fr) * 8 * n15;
     if (cudaMalloc(&T.mem, bytes) != cudaSuccess) {
       cudaGetLastError();
       ctx->err = "cudaMalloc NTT tables";
       return ZC_ERR_OOM;
     }
-    T.dft_fwd = static_cast<frc*>(T.mem);
-    T.dft_inv = T.dft_fwd + n4;
-    fr* p = reinterpret_cast<fr*>(T.dft_inv + n4);
+    T.dft_fwd = FrcTab::make(T.mem, n4);
+    T.dft_inv = FrcTab::make(static_cast<frc*>(T.mem) + n4, n4);
+    fr* p = reinterpret_cast<fr*>(static_cast<frc*>(T.mem) + 2 * n4);
     T.wf_lo = p; p += n15;
     T.wf_hi = p; p += n15;
     T.wi_lo = p; p += n15;
@@ -763,19 +808,27 @@ static zc_status ensure_tables(zc_ctx* ctx, cudaStream_t st, NttTables** out) {
   return ZC_OK;
 }
 
-// Pass kernel variants: tile of 2^logTile elements (TILE / 8 threads, each
-// owning 8 elements per stage) and a minimum number of resident CTAs per SM
-// (caps registers).  The context's tuning picks the tile and residency.
-template <int TILE, int MINB>
-static void launch_pass_variant(const NttPassArgs& a, dim3 grid, cudaStream_t st) {
-  k_ntt_pass<TILE, MINB><<<grid, TILE / 8, TILE * sizeof(fr), st>>>(a);
+// Pass variants: 8 elements per thread, up to 512 threads, a minimum number of
+// resident CTAs per SM (caps registers).  The context's tuning picks the tile
+// and residency.
+template <int MAXT, int MINB>
+static void launch_pass_variant(const NttPassArgs& a, uint32_t grid, uint32_t tile, cudaStream_t st) {
+  if (a.logL >= 3 && tile >= 512 && !(a.B & ((1u << a.logW) - 1)) && a.pre != PRE_COSET &&
+      (a.post == POST_NONE || a.post == POST_TAB))
+    k_ntt_pass<MAXT, MINB, true><<<grid, tile / 8, tile * sizeof(fr), st>>>(a);
+  else
+    k_ntt_pass<MAXT, MINB, false><<<grid, tile / 8, tile * sizeof(fr), st>>>(a);
 }
 
 static void set_pass_attributes() {
-  cudaFuncSetAttribute(k_ntt_pass<1024, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 * 32);
-  cudaFuncSetAttribute(k_ntt_pass<2048, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
-  cudaFuncSetAttribute(k_ntt_pass<2048, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
-  cudaFuncSetAttribute(k_ntt_pass<4096, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<128, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<128, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<256, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<256, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<256, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<256, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<512, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * 32);
+  cudaFuncSetAttribute(k_ntt_pass<512, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * 32);
 }
 
 static int g_attr_done[64] = {0};
@@ -803,20 +856,19 @@ static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int item
   if (logTile < logL) logTile = logL < 10 ? 10 : logL;
   if (logTile > 12) logTile = 12;
   if (logTile < 10) logTile = 10;
+  // a tile holds at least one warp's elements, sub-DFTs past the last included
   a.logW = logTile - logL;
-  while (a.logW > 0 && (1ull << a.logW) > B) a.logW--;
+  while (a.logW > 0 && a.logW + logL > 8 && (1ull << a.logW) > B) a.logW--;
   const uint64_t W = 1ull << a.logW;
   const uint64_t blocks = (B + W - 1) / W;
-  if (B % W) {
-    ctx->err = "NTT pass: batch not a multiple of the tile";
-    return ZC_ERR_ARG;
-  }
+  const uint32_t tile = 1u << (a.logW + logL);
   a.items = (uint32_t)items;
-  dim3 grid((unsigned)(blocks * (uint64_t)items));
-  if (logTile == 12) launch_pass_variant<4096, 1>(a, grid, st);
-  else if (logTile == 11 && minb != 1) launch_pass_variant<2048, 2>(a, grid, st);
-  else if (logTile == 11) launch_pass_variant<2048, 1>(a, grid, st);
-  else launch_pass_variant<1024, 4>(a, grid, st);
+  a.B = (uint32_t)B;
+  const uint32_t grid = (uint32_t)(blocks * (uint64_t)items);
+  if (logTile == 12) launch_pass_variant<512, 1>(a, grid, tile, st);
+  else if (logTile == 11 && minb != 1) launch_pass_variant<256, 2>(a, grid, tile, st);
+  else if (logTile == 11) launch_pass_variant<256, 1>(a, grid, tile, st);
+  else launch_pass_variant<128, 4>(a, grid, tile, st);
   ctx->launches++;
   return ZC_OK;
 }
@@ -858,11 +910,11 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
   e.l1 = l1;
   e.bytes = bytes;
   frc* q = static_cast<frc*>(e.mem);
-  e.tw_fwd = q; q += N;
-  e.tw_inv = q; q += N;
-  e.coset = q; q += M;
-  e.outer = q; q += M;
-  e.fin = q; q += s;
+  e.tw_fwd = FrcTab::make(q, N); q += N;
+  e.tw_inv = FrcTab::make(q, N); q += N;
+  e.coset = FrcTab::make(q, M); q += M;
+  e.outer = FrcTab::make(q, M); q += M;
+  e.fin = FrcTab::make(q, s); q += s;
   e.zinv = q;
   {
     // on the host: 7^-(N t), t < s; (z_H on slice j)^-1 M^-1 = (7^N w_s^j - 1)^-1 M^-1
@@ -874,12 +926,14 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
     fr wj = h_from_u64(1), fj = h_from_u64(1);
     for (uint64_t j = 0; j < s; j++) {
       const fr v = fr_sub_g(h_canon_mul(s7n, wj, C), h_from_u64(1));
-      hc[j] = h_frc(fj, C);
+      const frc fc = h_frc(fj, C);
+      for (int h = 0; h < 4; h++)  // planes, as FrcTab
+        std::memcpy(reinterpret_cast<char*>(hc.data()) + 16 * (h * s + j), reinterpret_cast<const char*>(&fc) + 16 * h, 16);
       hc[s + j] = h_frc(h_canon_mul(h_inv(v, C), minv, C), C);
       fj = h_canon_mul(fj, s7i, C);
       wj = h_canon_mul(wj, ws, C);
     }
-    if (cudaMemcpyAsync(e.fin, hc.data(), sizeof(frc) * 2 * s, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(e.fin.p, hc.data(), sizeof(frc) * 2 * s, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(e.mem);
@@ -909,8 +963,6 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
 
 static void pass_defaults(NttPassArgs& a) {
   std::memset(&a, 0, sizeof a);
-  a.in_lbdiv = 63;
-  a.out_lbdiv = 63;
 }
 
 static NttDomain domain_of(const zc_params* p) {
@@ -989,8 +1041,8 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
     cudaGetLastError();
     return false;
   }
-  frc* coset = static_cast<frc*>(mem);
-  fr* unscale = reinterpret_cast<fr*>(coset + N);
+  const FrcTab coset = FrcTab::make(mem, N);
+  fr* unscale = reinterpret_cast<fr*>(static_cast<frc*>(mem) + N);
   fr* cst = unscale + N;
   const DevConst& C = ctx->hconst;
   // sigma = 7 w_{2M}; kappa = sigma^M - 7^M; z_H on D_small = sigma^N - 1
@@ -1021,6 +1073,8 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
   a.coset = coset;
   a.unscale = unscale;
   a.n = n;
+  a.l1 = e->l1;
+  a.l2 = n - e->l1;
   a.shift2m = kLog30 - (n + lb + 1);
   a.ninv_l2 = fr_mul_g(fr_mul_g(ninv, C.r2), C.r2);
   a.T = *T;
@@ -1045,7 +1099,7 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
 // on load; canonical columns in, canonical codewords out.
 
 struct PcsTabArgs {
-  frc* tab;           // [s w + l] = (7 w_W^s)^l
+  FrcTab tab;         // [s w + l] = (7 w_W^s)^l
   uint32_t nc;        // w = 2^nc
   uint32_t shiftW;    // 30 - log2 W
   NttTables T;
@@ -1057,12 +1111,12 @@ __global__ void k_pcs_tables(PcsTabArgs A) {
     const uint32_t s = e >> A.nc, l = e & (w - 1);
     const fr p7 = fr_mul(ld_fr(A.T.p7_hi + (l >> kLoBits)), ld_fr(A.T.p7_lo + (l & kLoMask)));  // 7^l
     const uint32_t ex = (uint32_t)((((uint64_t)s * l) << A.shiftW) & ((1ull << kLog30) - 1));
-    st_frc(A.tab + e, frc_of(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex))));
+    A.tab.st(e, frc_of(fr_mul(p7, root_pow(A.T.wf_lo, A.T.wf_hi, ex))));
   }
 }
 
 zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uint32_t nc, fr* const* enc,
-                     frc* tab, cudaStream_t st) {
+                     FrcTab tab, cudaStream_t st) {
   if (nc < 1 || nc > 12 || c < 1 || c > kMaxCols) {
     ctx->err = "pcs: rows of 2 .. 2^12 elements";
     return ZC_ERR_UNSUPPORTED;
@@ -1088,11 +1142,11 @@ zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uin
       a.out[j] = enc[j] + sl * m;     // position k = sl + 4 k'
     }
     a.logL = nc;
-    a.in_bs_lo = w; a.in_ts = 1;      // row b, coefficient t
-    a.out_bs_lo = 1; a.out_ts = 4 * m;
+    a.im = map_flat(nc, 0);           // row b, coefficient t
+    a.om = map_flat(0, nr + 2);       // position 4 t
     set_dft(a, T, false);
-    a.pre = PRE_TAB; a.pre_tab = tab + sl * w;
-    a.pre_kb = 0; a.pre_kt = 1;
+    a.pre = PRE_TAB; a.pre_tab = tab.at(sl * w);
+    a.pm = map_low(0, 0, 0);
     zc_status rs = run_pass(ctx, st, a, c, m);
     if (rs != ZC_OK) return rs;
   }
@@ -1195,15 +1249,15 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.out[j - j0] = coef[j];
     }
     a.logL = l2;                       // rows of length L2 over i2
-    a.in_bs_lo = 1; a.in_ts = L1;      // element (i1, i2) read from e[i1 + L1 i2]
-    a.out_bs_lo = L2; a.out_ts = 1;
+    a.im = map_flat(0, l1);            // element (i1, i2) read from e[i1 + L1 i2]
+    a.om = map_flat(l2, 0);
     set_dft(a, T, true);
     a.err = &dstate->err;              // every input element passes through here once
     a.post = POST_TW; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
     a.tw_lbmod = l1; a.tw_shift = kLog30 - n;
     if (ST) {  // w_N^-(i1 k2) = tw_inv[i1 L2 + k2]
       a.post = POST_TAB; a.post_tab = ST->tw_inv;
-      a.p_lbdiv = 63; a.p_ls = L2; a.p_ts = 1;
+      a.qm = map_flat(l2, 0);
     }
     return run_pass(ctx, st, a, j1 - j0, L1);
   };
@@ -1216,8 +1270,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.out[j - j0] = coef[j];
     }
     a.logL = l1;
-    a.in_bs_lo = 1; a.in_ts = L2;
-    a.out_bs_lo = 1; a.out_ts = L2;
+    a.im = a.om = map_flat(0, l2);
     set_dft(a, T, true);
     return run_pass(ctx, st, a, j1 - j0, L2);
   };
@@ -1296,8 +1349,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.out[j] = coef[j];
     }
     a.logL = n;
-    a.in_bs_lo = 0; a.in_ts = 1;
-    a.out_bs_lo = 0; a.out_ts = 1;
+    a.im = a.om = map_flat(0, 0);
     set_dft(a, T, true);
     a.err = &dstate->err;
     if ((rs = run_pass(ctx, st, a, c, 1)) != ZC_OK) return rs;
@@ -1308,7 +1360,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   // slice_lde: the coset NTT of the `items` coefficient vectors in[] into
   // out[] on one slice, with the coset factor table pre (per-size tables)
   // or slice j's two-level tables (without them).
-  auto slice_lde = [&](const fr* const* in, fr* const* out, int items, const frc* pre, uint64_t j,
+  auto slice_lde = [&](const fr* const* in, fr* const* out, int items, const FrcTab* pre, uint64_t j,
                        bool mark) -> zc_status {
     NttPassArgs a;
     pass_defaults(a);
@@ -1323,15 +1375,13 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     set_dft(a, T, false);
     if (two) {
       a.logL = l1;                     // columns over k1: k = L2 k1 + k2
-      a.in_bs_lo = 1; a.in_ts = L2;
-      a.out_bs_lo = 1; a.out_ts = L2;
-      a.pre_kb = 1; a.pre_kt = L2;
+      a.im = a.om = a.pm = map_flat(0, l2);
       a.post = POST_TW; a.tw_lo = T->wf_lo; a.tw_hi = T->wf_hi;
       a.tw_lbmod = l2; a.tw_shift = kLog30 - n;
-      if (ST) {  // coset factor of k = k2 + L2 k1; twiddle w_N^(k2 i1) = tw_fwd[k2 L1 + i1]
-        a.pre = PRE_TAB; a.pre_tab = pre;
+      if (ST) {  // coset factor of k = L2 k1 + k2 at L1 k2 + k1; twiddle w_N^(k2 i1) = tw_fwd[k2 L1 + i1]
+        a.pre = PRE_TAB; a.pre_tab = *pre; a.pm = map_flat(l1, 0);
         a.post = POST_TAB; a.post_tab = ST->tw_fwd;
-        a.p_lbdiv = 63; a.p_ls = L1; a.p_ts = 1;
+        a.qm = map_flat(l1, 0);
       }
       if ((rs = run_pass(ctx, st, a, items, L2)) != ZC_OK) return rs;
       if (mark) ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[7], st));
@@ -1341,17 +1391,14 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
         a.out[i] = out[i];
       }
       a.logL = l2;                     // rows over k2
-      a.in_bs_lo = L2; a.in_ts = 1;
-      a.out_bs_lo = L2; a.out_ts = 1;
+      a.im = a.om = map_flat(l2, 0);
       set_dft(a, T, false);
       if ((rs = run_pass(ctx, st, a, items, L1)) != ZC_OK) return rs;
     } else {
       a.logL = n;
-      a.in_bs_lo = 0; a.in_ts = 1;
-      a.out_bs_lo = 0; a.out_ts = 1;
-      a.pre_kb = 0; a.pre_kt = 1;
+      a.im = a.om = a.pm = map_flat(0, 0);
       if (ST) {
-        a.pre = PRE_TAB; a.pre_tab = pre;
+        a.pre = PRE_TAB; a.pre_tab = *pre;
       }
       if ((rs = run_pass(ctx, st, a, items, 1)) != ZC_OK) return rs;
       if (mark) ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[7], st));
@@ -1374,7 +1421,8 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     ctx->launches++;
   };
   for (uint64_t j = 0; j < s; j++) {
-    if ((rs = slice_lde(coef, slb, c, ST ? ST->coset + j * N : nullptr, j, j == 0)) != ZC_OK) return rs;
+    const FrcTab cs = ST ? ST->coset.at(j * N) : FrcTab();
+    if ((rs = slice_lde(coef, slb, c, ST ? &cs : nullptr, j, j == 0)) != ZC_OK) return rs;
     slice_gate(qhat + j * N, (ST ? ST->zinv : zinv) + j, nullptr);
   }
   ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[3], st));
@@ -1389,43 +1437,40 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       pass_defaults(a);
       a.in[0] = qin; a.out[0] = qin;
       a.logL = l2;                     // rows (j, i2) over i3
-      a.in_bs_lo = L2; a.in_ts = 1;
-      a.out_bs_lo = L2; a.out_ts = 1;
+      a.im = a.om = map_flat(l2, 0);
       set_dft(a, T, true);
       a.post = POST_TW; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.tw_lbmod = l1; a.tw_shift = kLog30 - n;
       if (ST) {  // w_N^-(i2 k3) = tw_inv[(b mod L1) L2 + k3]
         a.post = POST_TAB; a.post_tab = ST->tw_inv;
-        a.p_lbdiv = l1; a.p_hs = 0; a.p_ls = L2; a.p_ts = 1;
+        a.qm = map_low(l1, l2, 0);
       }
       if ((rs = run_pass(ctx, st, a, 1, s * L1)) != ZC_OK) return rs;
       pass_defaults(a);
       a.in[0] = qin; a.out[0] = qin;
       a.logL = l1;                     // columns (j, k3) over i2 within a slice
-      a.in_lbdiv = l2; a.in_bs_hi = N; a.in_bs_lo = 1; a.in_ts = L2;
-      a.out_lbdiv = l2; a.out_bs_hi = N; a.out_bs_lo = 1; a.out_ts = L2;
+      a.im = a.om = map_split(l2, n, 0, l2);
       set_dft(a, T, true);
       a.post = POST_OUTER; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.outer_lbdiv = l2; a.tw_shift = kLog30 - logm;
-      if (ST) {  // w_M^-(j k') 7^-k', k' = L2 k2 + k3: outer[j N + k']
+      if (ST) {  // w_M^-(j k') 7^-k', k' = L2 k2 + k3: outer[j N + L1 k3 + k2]
         if (s == 1) a.out[0] = qout;  // no cross-slice stage
         a.post = POST_TAB; a.post_tab = ST->outer;
-        a.p_lbdiv = l2; a.p_hs = N; a.p_ls = 1; a.p_ts = L2;
+        a.qm = map_split(l2, n, l1, 0);
       }
       if ((rs = run_pass(ctx, st, a, 1, s * L2)) != ZC_OK) return rs;
     } else {
       pass_defaults(a);
       a.in[0] = qin; a.out[0] = qin;
       a.logL = n;                      // one row per slice
-      a.in_bs_lo = N; a.in_ts = 1;
-      a.out_bs_lo = N; a.out_ts = 1;
+      a.im = a.om = map_flat(n, 0);
       set_dft(a, T, true);
       a.post = POST_OUTER; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.outer_lbdiv = 0; a.tw_shift = kLog30 - logm;
       if (ST) {
         if (s == 1) a.out[0] = qout;
         a.post = POST_TAB; a.post_tab = ST->outer;
-        a.p_lbdiv = 63; a.p_ls = N; a.p_ts = 1;
+        a.qm = map_flat(n, 0);
       }
       if ((rs = run_pass(ctx, st, a, 1, s)) != ZC_OK) return rs;
     }
@@ -1433,14 +1478,13 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     pass_defaults(a);
     a.in[0] = qin; a.out[0] = qout;
     a.logL = lb;                       // across slices
-    a.in_bs_lo = 1; a.in_ts = N;
-    a.out_bs_lo = 1; a.out_ts = N;
+    a.im = a.om = map_flat(0, n);
     set_dft(a, T, true);
     a.post = POST_FINAL; a.tw_lo = T->s7_lo; a.tw_hi = T->s7_hi;
-    a.fin_N = N;
+    a.fin_logN = n;
     if (ST) {  // 7^-(N t)
       a.post = POST_TAB; a.post_tab = ST->fin;
-      a.p_lbdiv = 63; a.p_ls = 0; a.p_ts = 1;
+      a.qm = map_low(0, 0, 0);
     }
     if ((rs = run_pass(ctx, st, a, 1, N)) != ZC_OK) return rs;
   }
@@ -1462,8 +1506,8 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     ctx->launches++;
     const fr* rin[1] = {rho};
     fr* rout[1] = {vsm};
-    if ((rs = slice_lde(rin, rout, 1, ST->step_coset, 0, false)) != ZC_OK) return rs;
-    if ((rs = slice_lde(coef, slb, c, ST->step_coset, 0, false)) != ZC_OK) return rs;
+    if ((rs = slice_lde(rin, rout, 1, &ST->step_coset, 0, false)) != ZC_OK) return rs;
+    if ((rs = slice_lde(coef, slb, c, &ST->step_coset, 0, false)) != ZC_OK) return rs;
     slice_gate(qhat + Mb, reinterpret_cast<const frc*>(ST->step_const), vsm);
     if ((rs = inverse(qhat + Mb, qv + Mb, 1, 0, n)) != ZC_OK) return rs;
     NttStepCombineArgs ca{};

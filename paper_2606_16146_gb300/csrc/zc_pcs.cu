@@ -300,7 +300,7 @@ zc_status zc_pcs_commit(zc_ctx* ctx, const zc_pcs_params* params, const void* co
     P->enc[j] = reinterpret_cast<fr*>(q);
     q += benc;
   }
-  frc* tab = reinterpret_cast<frc*>(q);
+  const FrcTab tab = FrcTab::make(q, S.W);
   q += btab;
   uint32_t* dig = reinterpret_cast<uint32_t*>(q);
   q += bdig;
