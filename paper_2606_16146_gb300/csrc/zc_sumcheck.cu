@@ -112,7 +112,8 @@ struct ScRoundArgs {
   ScState* st;
   fr* partials;
   uint8_t* proof;
-  fr kcomp;            // product gate: R^(2-d) mod r
+  frc kcomp;           // product gate: R^(1-d) mod r, the level of the product over level 0
+  frc mont;            // Plonk gate: R mod r, canonical to level 1
   const DevConst* C;
   const fr* tabs;
 };
@@ -206,7 +207,7 @@ struct ChalSmem {
   fr hd[kMaxPts];      // H(t) times the Lagrange denominator's inverse
   fr tmp[2][kMaxPts];
   fr cl[kMaxPts];      // c_i l_i(t)
-  fr alpha;
+  fr alpha, alpha_raw;  // level 1, canonical
   uint32_t msg[8 + 8 * kMaxPts];
 };
 static_assert(2 * kMaxPts >= 32, "tmp holds one partial sum per warp of a 1024-thread CTA");
@@ -292,10 +293,12 @@ __device__ void sc_challenge(ChalSmem& S, int np, int d, int i, ScState* st, uin
   if (t == 0) {
     uint32_t Sn[8];
     sha256_words<COLD>(S.msg, 8 + 8 * per, Sn);
-    const fr a = fr_mul(tr_squeeze<COLD>(Sn), C->r2);
+    const fr raw = tr_squeeze<COLD>(Sn);
+    const fr a = fr_mul(raw, C->r2);
     for (int q = 0; q < 8; q++) st->S[q] = Sn[q];
     st->alpha[i] = a;
     S.alpha = a;
+    S.alpha_raw = raw;
     if (release) {  // the next round needs only alpha: hand it off before c_i and the claim
       __threadfence();
       atomicExch(release, (uint32_t)(i + 1));
@@ -304,6 +307,10 @@ __device__ void sc_challenge(ChalSmem& S, int np, int d, int i, ScState* st, uin
   __syncthreads();
   const fr a = S.alpha;
   if (t == hs) st->ci = fr_mul(st->ci, fr_add(one_m_r, fr_mul(a, two_r_m1)));
+  if (COLD && t == hs + 32) {  // the next round is a launch of its own: it folds by the constant alpha
+    st->alphac[i].w = S.alpha_raw;
+    st->alphac[i].q = fr_quot(a);
+  }
   if (need_claim) {
     // next claim H_i(alpha) by Lagrange over the nodes 0..d
     if (t <= d) {
@@ -383,8 +390,8 @@ __device__ void sc_finish_round(const ScRoundArgs& A, int np) {
 // qR, qO, c, qC so only the running gate value per point stays live:
 //   f = a (qL + qM b) + qR b + qO c + qC.
 template <bool FIRST, bool COHERENT>
-__device__ __forceinline__ void plonk_pair(const fr* const* src, fr* const* dst, const DevConst* C,
-                                           uint64_t k, uint64_t h, const fr& alpha, uint32_t p0,
+__device__ __forceinline__ void plonk_pair(const fr* const* src, fr* const* dst, const frc& mont,
+                                           uint64_t k, uint64_t h, const frc& alpha, uint32_t p0,
                                            const fr& w, fr (&acc)[FIRST ? 4 : 3], uint32_t& bad) {
   constexpr int NF = FIRST ? 3 : 2;
   auto column = [&](int j, fr (&v)[NF], fr& dl) {
@@ -394,16 +401,16 @@ __device__ __forceinline__ void plonk_pair(const fr* const* src, fr* const* dst,
       hi = ldt<COHERENT>(src[j] + k + h);
       bad |= (!fr_is_canonical(lo)) | (!fr_is_canonical(hi));
       if (j >= 5) {
-        lo = to_mont(lo, C);
-        hi = to_mont(hi, C);
+        lo = fr_mulc(mont, lo);
+        hi = fr_mulc(mont, hi);
         st_fr(dst[j] + k, lo);
         st_fr(dst[j] + k + h, hi);
       }
     } else {
       const fr x0 = ldt<COHERENT>(src[j] + k), x1 = ldt<COHERENT>(src[j] + k + 2 * h);
       const fr y0 = ldt<COHERENT>(src[j] + k + h), y1 = ldt<COHERENT>(src[j] + k + 3 * h);
-      lo = fr_add(x0, fr_mul(alpha, fr_sub(x1, x0)));
-      hi = fr_add(y0, fr_mul(alpha, fr_sub(y1, y0)));
+      lo = fr_add(x0, fr_mulc(alpha, fr_sub_lazy(x1, x0)));
+      hi = fr_add(y0, fr_mulc(alpha, fr_sub_lazy(y1, y0)));
       st_fr(dst[j] + k, lo);
       st_fr(dst[j] + k + h, hi);
     }
@@ -499,8 +506,8 @@ __device__ __forceinline__ void prod_pair_g(const ScRoundArgs& A, Load load, int
     }
     const bool scale_ends = PP > 1 && pcnt >= 2;
     if (scale_ends) {
-      lo = fr_mul(lo, A.kcomp);
-      hi = fr_mul(hi, A.kcomp);
+      lo = fr_mulc(A.kcomp, lo);
+      hi = fr_mulc(A.kcomp, hi);
     }
     const fr dl = fr_sub(hi, lo);
     fr e = lo;
@@ -513,7 +520,7 @@ __device__ __forceinline__ void prod_pair_g(const ScRoundArgs& A, Load load, int
       else
         for (uint32_t s2 = tcur; s2 < tpt[p]; s2++) e = fr_add(e, dl);
       tcur = tpt[p];
-      prod[p] = fr_add(prod[p], scale_ends ? e : fr_mul(e, A.kcomp));
+      prod[p] = fr_add(prod[p], scale_ends ? e : fr_mulc(A.kcomp, e));
     }
   }
 #pragma unroll
@@ -752,11 +759,15 @@ __global__ void __launch_bounds__(256, MINB) k_sc_plonk_round(ScRoundArgs A) {
   fr acc[NP];
 #pragma unroll
   for (int p = 0; p < NP; p++) acc[p] = fr_zero();
-  const fr alpha = FIRST ? fr_zero() : A.st->alpha[i - 1];
+  __shared__ frc alpha;
+  if (!FIRST) {
+    if (threadIdx.x == 0) alpha = A.st->alphac[i - 1];
+    __syncthreads();
+  }
   const uint32_t p0 = FIRST ? 0u : A.st->p0[i];
   uint32_t bad = 0;
   for (uint64_t k = A.k0 + tid; k < kend; k += T)
-    plonk_pair<FIRST, false>(A.src, A.dst, A.C, k, h, alpha, p0, ld_fr(ehi + (k >> mlo)), acc, bad);
+    plonk_pair<FIRST, false>(A.src, A.dst, A.mont, k, h, alpha, p0, ld_fr(ehi + (k >> mlo)), acc, bad);
   if (FIRST && bad) atomicOr(&A.st->err, 1u);
   // each thread handled pairs with one fixed low part k_lo (k0 and T are
   // multiples of 2^mlo)
@@ -879,14 +890,14 @@ __global__ void __launch_bounds__(16 * kSmallPB) k_sc_plonk_rounds(ScRoundArgs A
 
 // MLE update by alpha_{round-1}: dst[j][k] = src[j][k] + alpha (src[j][k+h] - src[j][k])
 __global__ void __launch_bounds__(256) k_sc_fold(ScFoldArgs A) {
-  const fr alpha = A.st->alpha[A.round - 1];
+  const frc alpha = A.st->alphac[A.round - 1];
   const uint64_t total = A.h * (uint64_t)A.c;
   for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (uint64_t)gridDim.x * blockDim.x) {
     const int j = (int)(e / A.h);
     const uint64_t k = e - (uint64_t)j * A.h;
     const fr x0 = ld_fr_cs(A.src[j] + k), x1 = ld_fr_cs(A.src[j] + k + A.h);
-    st_fr(A.dst[j] + k, fr_add(x0, fr_mul(alpha, fr_sub(x1, x0))));
+    st_fr(A.dst[j] + k, fr_add(x0, fr_mulc(alpha, fr_sub_lazy(x1, x0))));
   }
 }
 
@@ -972,7 +983,7 @@ __global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
   const uint32_t mlo = A.m_lo[i];
   const fr* ehi = A.E + A.eq_hi[i];
   const fr* elo = A.E + A.eq_lo[i];
-  const fr alpha = A.st->alpha[i - 1];
+  const frc alpha = A.st->alphac[i - 1];
   const uint64_t h = A.h;
   uint32_t bad = 0;
   fr acc[PP];
@@ -989,7 +1000,7 @@ __global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
       if (k < h) {
         const uint64_t idx = k + (half ? h : 0);
         const fr x0 = ld_fr_cs(A.src[j] + idx), x1 = ld_fr_cs(A.src[j] + idx + 2 * h);
-        const fr v = fr_add(x0, fr_mul(alpha, fr_sub(x1, x0)));
+        const fr v = fr_add(x0, fr_mulc(alpha, fr_sub_lazy(x1, x0)));
         st_fr(A.dst[j] + idx, v);
         Vs[(size_t)rest * spb + p] = v;
       }
@@ -1361,7 +1372,8 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
   R.st = B.st;
   R.partials = B.partials;
   R.proof = B.proof;
-  R.kcomp = hC.rnegpow[d - 2];
+  R.kcomp = h_frc(hC.rnegpow[d - 1], hC);
+  R.mont = h_frc(hC.one, hC);
   R.C = dC;
   R.tabs = dtabs;
   R.v2 = v2 ? 1u : 0u;
