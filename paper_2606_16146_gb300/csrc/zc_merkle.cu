@@ -244,6 +244,22 @@ struct PcsLevelArgs {
   uint32_t words;      // words hashed per node (16 for a pair, 8 c for a leaf)
 };
 
+// SHA-256 of nwords big-endian message words by one thread
+__device__ void sha256_words(const uint32_t* w, uint32_t nwords, uint32_t out[8]) {
+  sha256_init(out);
+  const uint32_t nb = sha_blocks(nwords), end = 16 * nb;
+#pragma unroll 1
+  for (uint32_t b = 0; b < nb; b++) {
+    uint32_t blk[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const uint32_t e = 16 * b + i;
+      blk[i] = e < nwords ? w[e] : e == nwords ? 0x80000000u : e == end - 1 ? 32 * nwords : 0u;
+    }
+    sha256_compress(out, blk);
+  }
+}
+
 __global__ void k_pcs_level(PcsLevelArgs A) {
   const uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (u >= A.count) return;

@@ -622,31 +622,35 @@ struct NttZArgs {
   const DevConst* C;
 };
 
-__global__ void k_ntt_z(NttZArgs A) {
-  if (threadIdx.x != 0) return;
+// Transcript up to z (two warps, see ShaPair; again while z^N = 1) and the
+// powers z^(2^i), of which z^N is one.  Launched with 64 threads.
+__global__ void __launch_bounds__(64) k_ntt_z(NttZArgs A) {
+  __shared__ ShaPair Z;
+  __shared__ uint32_t blk[32];
+  __shared__ uint32_t again;
   const DevConst* C = A.C;
   uint32_t S[8];
   for (int i = 0; i < 8; i++) S[i] = A.S0[i];
-  for (int j = 0; j <= A.c; j++) tr_absorb32(S, A.roots + 32 * j);
-  fr z;
-  uint32_t err = 1;
+  tr_absorb32(Z, blk, S, A.roots, A.c + 1);
   for (int tries = 0; tries < 64; tries++) {
-    z = fr_mul(tr_squeeze(S), C->r2);
-    fr zn = z;
-    for (uint32_t i = 0; i < A.n; i++) zn = fr_mul(zn, zn);
-    if (!fr_equal(zn, C->one)) {
-      err = 0;
-      A.st->zpow_n = zn;
-      break;
+    const fr raw = tr_squeeze(Z, S);
+    if (threadIdx.x == 0) {
+      fr p = fr_mul(raw, C->r2);
+      A.st->z = p;
+      for (uint32_t i = 0; i < 31; i++) {
+        A.zpow[i] = p;
+        if (i == A.n) {
+          A.st->zpow_n = p;
+          again = fr_equal(p, C->one) ? 1u : 0u;
+        }
+        p = fr_mul(p, p);
+      }
     }
+    __syncthreads();
+    if (!again) return;
+    __syncthreads();
   }
-  A.st->z = z;
-  A.st->err |= err;
-  fr p = z;
-  for (int i = 0; i < 31; i++) {
-    A.zpow[i] = p;
-    p = fr_mul(p, p);
-  }
+  if (threadIdx.x == 0) A.st->err |= 1u;
 }
 
 // Evaluate sum_k x[k] z^k for each item (level-0 x); every warp takes a
@@ -1542,7 +1546,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     transcript_init_words(za.S0, ZC_FORM_NTT, gate, n, d, D.word);
     za.zpow = zpow;
     za.C = ctx->dconst;
-    k_ntt_z<<<1, 32, 0, st>>>(za);
+    k_ntt_z<<<1, 64, 0, st>>>(za);
     ctx->launches++;
   }
   ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[5], st));

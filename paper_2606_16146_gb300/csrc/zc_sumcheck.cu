@@ -208,7 +208,8 @@ struct ChalSmem {
   fr tmp[2][kMaxPts];
   fr cl[kMaxPts];      // c_i l_i(t)
   fr alpha, alpha_raw;  // level 1, canonical
-  uint32_t msg[8 + 8 * kMaxPts];
+  uint32_t msg[8 + 8 * kMaxPts + 24];  // the message, padded to whole blocks
+  ShaPair Z;
 };
 static_assert(2 * kMaxPts >= 32, "tmp holds one partial sum per warp of a 1024-thread CTA");
 
@@ -230,10 +231,10 @@ __device__ __forceinline__ void sc_put_value(ChalSmem& S, uint8_t* proof, int i,
 // derives a point, the claim H_i(alpha_i).  All threads of the CTA (at least
 // 128).  Independent steps run on different warps so the serial chain is
 // four multiplications and the hash up to alpha (two or three more for c_i
-// and the claim).  COLD: the hash uses the compact compression (a launch
-// that runs one challenge).  release: a flag that receives i + 1 as soon as
+// and the claim).  LAST: the challenge of a launch of one round; alpha_i is
+// also kept as a constant multiplier for the next launch.  release: a flag that receives i + 1 as soon as
 // alpha_i is out (the persistent round kernel's hand-off).
-template <bool COLD>
+template <bool LAST>
 __device__ void sc_challenge(ChalSmem& S, int np, int d, int i, ScState* st, uint8_t* proof,
                              const DevConst* C, const fr* tabs, bool need_claim, bool v2,
                              uint32_t* release = nullptr) {
@@ -263,6 +264,8 @@ __device__ void sc_challenge(ChalSmem& S, int np, int d, int i, ScState* st, uin
     }
   }
   if (t < 8) S.msg[t] = st->S[t];
+  const int per = v2 ? d + 1 : d + 2;
+  sha_pad(S.msg, 8 + 8 * per, t, blockDim.x);
   __syncthreads();
   // extrapolate H(d), H(d+1) from H(0..d-1) and the leading coefficient:
   // every product in parallel, then two sums
@@ -285,29 +288,29 @@ __device__ void sc_challenge(ChalSmem& S, int np, int d, int i, ScState* st, uin
   // G(t) = c_i l_i(t) H(t) at t = 0..d+1, or (v2) H(t) at t = 0..d; H is
   // at level 0 = canonical.  Other threads: H(t) / prod_{q != t} (t - q)
   // for the next claim.
-  const int per = v2 ? d + 1 : d + 2;
   if (t < per) sc_put_value(S, proof, i, per, t, v2 ? S.H[t] : fr_mul(S.H[t], S.cl[t]));
   const fr* dinv = tabs + C->lag_base[d];
   if (need_claim && t >= 32 && t - 32 <= d) S.hd[t - 32] = fr_mul(S.H[t - 32], dinv[t - 32]);
   __syncthreads();
-  if (t == 0) {
+  if (t < 64) {  // warps 0 and 1 hash together
     uint32_t Sn[8];
-    sha256_words<COLD>(S.msg, 8 + 8 * per, Sn);
-    const fr raw = tr_squeeze<COLD>(Sn);
-    const fr a = fr_mul(raw, C->r2);
-    for (int q = 0; q < 8; q++) st->S[q] = Sn[q];
-    st->alpha[i] = a;
-    S.alpha = a;
-    S.alpha_raw = raw;
-    if (release) {  // the next round needs only alpha: hand it off before c_i and the claim
-      __threadfence();
-      atomicExch(release, (uint32_t)(i + 1));
+    const fr raw = tr_hash_squeeze(S.Z, S.msg, 8 + 8 * per, Sn);
+    if (t == 0) {
+      const fr a = fr_mul(raw, C->r2);
+      for (int q = 0; q < 8; q++) st->S[q] = Sn[q];
+      st->alpha[i] = a;
+      S.alpha = a;
+      S.alpha_raw = raw;
+      if (release) {  // the next round needs only alpha: hand it off before c_i and the claim
+        __threadfence();
+        atomicExch(release, (uint32_t)(i + 1));
+      }
     }
   }
   __syncthreads();
   const fr a = S.alpha;
   if (t == hs) st->ci = fr_mul(st->ci, fr_add(one_m_r, fr_mul(a, two_r_m1)));
-  if (COLD && t == hs + 32) {  // the next round is a launch of its own: it folds by the constant alpha
+  if (LAST && t == hs + 32) {  // the next round is a launch of its own: it folds by the constant alpha
     st->alphac[i].w = S.alpha_raw;
     st->alphac[i].q = fr_quot(a);
   }
@@ -645,16 +648,21 @@ __device__ __forceinline__ void plonk_chunk_reduce(const fr& acc, fr* out) {
 // ---------------------------------------------------------------- kernels --
 
 // Transcript: absorb the column roots, squeeze r_1..r_n; reset per-proof state.
-// The hash chain is serial (thread 0); the n conversions to Montgomery form
-// run on n threads afterwards.  Launched with at least kMaxN threads.
-__global__ void k_sc_setup(ScSetupArgs A) {
+// The hash chain is serial (two warps, see ShaPair); the n conversions to
+// Montgomery form run on n threads afterwards.  Launched with 64 threads.
+__global__ void __launch_bounds__(64) k_sc_setup(ScSetupArgs A) {
   __shared__ fr raw[kMaxN];
+  __shared__ ShaPair Z;
+  __shared__ uint32_t blk[32];
   if (threadIdx.x < kMaxN) A.st->counter[threadIdx.x] = 0;
+  uint32_t S[8];
+  for (int i = 0; i < 8; i++) S[i] = A.S0[i];
+  tr_absorb32(Z, blk, S, A.roots, A.c);
+  for (int i = 0; i < A.n; i++) {
+    const fr x = tr_squeeze(Z, S);
+    if (threadIdx.x == 0) raw[i] = x;
+  }
   if (threadIdx.x == 0) {
-    uint32_t S[8];
-    for (int i = 0; i < 8; i++) S[i] = A.S0[i];
-    for (int j = 0; j < A.c; j++) tr_absorb32(S, A.roots + 32 * j);
-    for (int i = 0; i < A.n; i++) raw[i] = tr_squeeze(S);
     for (int i = 0; i < 8; i++) A.st->S[i] = S[i];
     A.st->claim = fr_zero();
     A.st->ci = A.C->one;
@@ -1343,7 +1351,7 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
   sa.c = c;
   sa.n = (int)n;
   sa.C = dC;
-  k_sc_setup<<<1, 32, 0, st>>>(sa);
+  k_sc_setup<<<1, 64, 0, st>>>(sa);
   ScEqArgs ea{};
   ea.st = B.st;
   ea.E = B.E;

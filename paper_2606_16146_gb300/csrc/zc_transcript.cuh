@@ -13,62 +13,89 @@ namespace zc {
 
 #if defined(__CUDACC__)
 
-// One compression for transcript hashing: COLD picks the compact copy, for a
-// hash that runs once in a launch (see zc_sha256.cuh).
-template <bool COLD>
-__device__ __forceinline__ void tr_compress(uint32_t h[8], const uint32_t w[16]) {
-  if (COLD) sha256_compress_small(h, w);
-  else sha256_compress_hot(h, w);
+// SHA-256 by two warps.  A transcript hash is one serial chain of
+// compressions, and the 24 instructions of a round (14 of the round itself, 10
+// of the message schedule) fill the ALU pipe of the SM quarter its warp runs
+// on: 3130 cycles a compression.  Warp 0 runs the rounds and warp 1, on another
+// quarter, the schedule: words 16..63 with their round constants, through
+// shared memory, sixteen at a time.  The first sixteen rounds need only the
+// message, so the schedule stays ahead, and a compression takes the rounds'
+// ~1920 cycles; both loops are short enough to be cheap when their code is
+// cold.  All lanes of a warp compute the same values.  The two warps meet four
+// times a block: when its words are in shared memory (and the previous block's
+// schedule has been read), and at each third of the schedule.
+struct ShaPair {
+  uint32_t kw[48];     // schedule words 16..63 plus round constants
+  uint32_t sq[16];     // the squeeze block: state, 0x43, padding
+};
+
+// both warps; the id is an immediate (with an id in a register a kernel
+// reserves all sixteen barriers)
+__device__ __forceinline__ void pair_sync() {
+  __syncwarp();
+  asm volatile("bar.sync 1, 64;" ::: "memory");
 }
 
-// SHA-256 of a word message in pieces: tr_blocks compresses the complete
-// 16-word blocks [b0, b1); tr_last compresses what remains after the last
-// complete block, with the padding and the bit length.
-template <bool COLD>
-__device__ inline void tr_blocks(uint32_t h[8], const uint32_t* w, uint32_t b0, uint32_t b1) {
-  uint32_t blk[16];
-  for (uint32_t b = b0; b < b1; b++) {
-#pragma unroll
-    for (int i = 0; i < 16; i++) blk[i] = w[16 * b + i];
-    tr_compress<COLD>(h, blk);
-  }
-}
-
-template <bool COLD>
-__device__ inline void tr_last(uint32_t h[8], const uint32_t* w, uint32_t nwords) {
-  uint32_t blk[16];
-  const uint32_t full = nwords / 16, rem = nwords - 16 * full;
-#pragma unroll
-  for (int i = 0; i < 16; i++) blk[i] = 0;
-  for (uint32_t i = 0; i < rem; i++) blk[i] = w[16 * full + i];
-  blk[rem] = 0x80000000u;
-  const uint64_t bits = (uint64_t)nwords * 32;
-  if (rem + 1 > 14) {
-    tr_compress<COLD>(h, blk);
-#pragma unroll
-    for (int i = 0; i < 16; i++) blk[i] = 0;
-  }
-  blk[14] = (uint32_t)(bits >> 32);
-  blk[15] = (uint32_t)bits;
-  tr_compress<COLD>(h, blk);
-}
-
-// SHA-256 over nwords big-endian message words (any count), digest in out.
-template <bool COLD = false>
-__device__ inline void sha256_words(const uint32_t* w, uint32_t nwords, uint32_t out[8]) {
-  sha256_init(out);
-  tr_blocks<COLD>(out, w, 0, nwords / 16);
-  tr_last<COLD>(out, w, nwords);
-}
-
-// S <- SHA-256(S | m) for a 32-byte message given as bytes
-__device__ inline void tr_absorb32(uint32_t S[8], const uint8_t* m) {
+// warp 1: the schedule of the block blk (shared memory)
+__device__ __forceinline__ void sha_pair_schedule(ShaPair& Z, const uint32_t* blk) {
   uint32_t w[16];
-  for (int i = 0; i < 8; i++) w[i] = S[i];
-  for (int i = 0; i < 8; i++)
-    w[8 + i] = ((uint32_t)m[4 * i] << 24) | ((uint32_t)m[4 * i + 1] << 16) |
-               ((uint32_t)m[4 * i + 2] << 8) | m[4 * i + 3];
-  sha256_words(w, 16, S);
+  pair_sync();
+#pragma unroll
+  for (int i = 0; i < 16; i++) w[i] = blk[i];
+#pragma unroll 1
+  for (int q = 0; q < 3; q++) {
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const uint32_t x15 = w[(i + 1) & 15], x2 = w[(i + 14) & 15];
+      const uint32_t s0 = sha_rotr(x15, 7) ^ sha_rotr(x15, 18) ^ (x15 >> 3);
+      const uint32_t s1 = sha_rotr(x2, 17) ^ sha_rotr(x2, 19) ^ (x2 >> 10);
+      w[i] = w[i] + s0 + w[(i + 9) & 15] + s1;
+      Z.kw[16 * q + i] = w[i] + kShaK[16 * q + 16 + i];
+    }
+    pair_sync();
+  }
+}
+
+// warp 0: h <- compress(h, blk)
+__device__ __forceinline__ void sha_pair_rounds(ShaPair& Z, const uint32_t* blk, uint32_t h[8]) {
+  uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
+  auto round = [&](uint32_t k) {
+    const uint32_t t1 = hh + (sha_rotr(e, 6) ^ sha_rotr(e, 11) ^ sha_rotr(e, 25)) + ((e & f) ^ (~e & g)) + k;
+    const uint32_t t2 = (sha_rotr(a, 2) ^ sha_rotr(a, 13) ^ sha_rotr(a, 22)) + ((a & b) | (c & (a | b)));
+    hh = g;
+    g = f;
+    f = e;
+    e = d + t1;
+    d = c;
+    c = b;
+    b = a;
+    a = t1 + t2;
+  };
+  pair_sync();
+#pragma unroll
+  for (int i = 0; i < 16; i++) round(kShaK[i] + blk[i]);
+#pragma unroll 1
+  for (int q = 0; q < 3; q++) {
+    pair_sync();
+#pragma unroll
+    for (int i = 0; i < 16; i++) round(Z.kw[16 * q + i]);
+  }
+  h[0] += a; h[1] += b; h[2] += c; h[3] += d;
+  h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
+}
+
+// One block by both warps (warp 0: h updated; warp 1: h untouched).
+__device__ __forceinline__ void sha_pair_block(ShaPair& Z, const uint32_t* blk, uint32_t h[8]) {
+  if (threadIdx.x < 32) sha_pair_rounds(Z, blk, h);
+  else sha_pair_schedule(Z, blk);
+}
+
+// Padding of a message of nwords words at w (room for the whole last block):
+// the words after the message, by the threads t, t + nt, ...
+__device__ __forceinline__ uint32_t sha_blocks(uint32_t nwords) { return (nwords + 3 + 15) / 16; }
+__device__ __forceinline__ void sha_pad(uint32_t* w, uint32_t nwords, uint32_t t, uint32_t nt) {
+  const uint32_t end = 16 * sha_blocks(nwords);
+  for (uint32_t i = nwords + t; i < end; i += nt) w[i] = i == nwords ? 0x80000000u : i == end - 1 ? 32 * nwords : 0u;
 }
 
 // int_le(digest) mod r as a canonical element (2^256 < 3r: at most two subtractions)
@@ -88,19 +115,62 @@ __device__ inline fr digest_mod_r(const uint32_t h[8]) {
   return x;
 }
 
-// S <- SHA-256(S | 0x43); returns the canonical challenge
-template <bool COLD = false>
-__device__ inline fr tr_squeeze(uint32_t S[8]) {
-  uint32_t w[16];
-  for (int i = 0; i < 8; i++) w[i] = S[i];
-  w[8] = 0x43800000u;  // the byte 0x43, then the padding bit
-  for (int i = 9; i < 15; i++) w[i] = 0;
-  w[15] = 33 * 8;
-  uint32_t h[8];
-  sha256_init(h);
-  tr_compress<COLD>(h, w);
-  for (int i = 0; i < 8; i++) S[i] = h[i];
-  return digest_mod_r(h);
+// the squeeze block of the state S (warp 0's lanes; both warps call)
+__device__ __forceinline__ void tr_squeeze_block(ShaPair& Z, const uint32_t S[8]) {
+  if (threadIdx.x < 16) {
+    const int i = threadIdx.x;
+    uint32_t v = i == 8 ? 0x43800000u : i == 15 ? 33 * 8 : 0u;  // the byte 0x43, then the padding bit; the length
+#pragma unroll
+    for (int q = 0; q < 8; q++) v = i == q ? S[q] : v;
+    Z.sq[i] = v;
+  }
+}
+
+// S <- SHA-256(S | 0x43) and the canonical challenge, warps 0 and 1 (values in
+// warp 0)
+__device__ __forceinline__ fr tr_squeeze(ShaPair& Z, uint32_t S[8]) {
+  tr_squeeze_block(Z, S);
+  sha256_init(S);
+  sha_pair_block(Z, Z.sq, S);
+  return digest_mod_r(S);
+}
+
+// S <- SHA-256(w) for the padded message w (shared memory) of nwords words,
+// then a squeeze; one copy of the compression serves both.  Warps 0 and 1
+// (values in warp 0).
+__device__ __forceinline__ fr tr_hash_squeeze(ShaPair& Z, const uint32_t* w, uint32_t nwords, uint32_t S[8]) {
+  const uint32_t nb = sha_blocks(nwords);
+  sha256_init(S);
+#pragma unroll 1
+  for (uint32_t b = 0; b <= nb; b++) {
+    if (b == nb) {
+      tr_squeeze_block(Z, S);
+      sha256_init(S);
+    }
+    sha_pair_block(Z, b < nb ? w + 16 * b : Z.sq, S);
+  }
+  return digest_mod_r(S);
+}
+
+// S <- SHA-256(S | m_j) for c 32-byte messages at m (global memory), warps 0
+// and 1 (S in warp 0).  blk: 32 words of shared memory.
+__device__ __forceinline__ void tr_absorb32(ShaPair& Z, uint32_t* blk, uint32_t S[8], const uint8_t* m, int c) {
+  if (threadIdx.x < 16) blk[16 + threadIdx.x] = threadIdx.x == 0 ? 0x80000000u : threadIdx.x == 15 ? 512 : 0u;
+#pragma unroll 1
+  for (int j = 0; j < 2 * c; j++) {
+    if (!(j & 1)) {
+      if (threadIdx.x < 16) {
+        const int i = threadIdx.x;
+        const uint8_t* p = m + 16 * j + 4 * (i & 7);
+        uint32_t v = ((uint32_t)p[0] << 24) | ((uint32_t)p[1] << 16) | ((uint32_t)p[2] << 8) | p[3];
+#pragma unroll
+        for (int q = 0; q < 8; q++) v = i == q ? S[q] : v;
+        blk[i] = v;
+      }
+      sha256_init(S);
+    }
+    sha_pair_block(Z, blk + 16 * (j & 1), S);
+  }
 }
 
 #endif
