@@ -48,7 +48,6 @@ constexpr uint64_t kSmallPairsPlonk = 1ull << 14;  // rounds with at most this m
 constexpr uint64_t kChunkPairsPlonk = 1ull << 14;  // Plonk rounds 2.. with at most this many: 16 threads per pair
 constexpr uint64_t kQuadPairsPlonk = 1ull << 17;   // and up to this many: 4 threads per pair
 constexpr uint64_t kFusePairsProd = 1ull << 16;    // product rounds 2.. with at most this many: fused update
-constexpr int kPP = 3;  // product gate: points per thread
 constexpr int kSmallPB = 16;  // pairs per chunk of the 16-threads-per-pair kernel (256 threads)
 constexpr int kQuadPB = 32;   // pairs per chunk of the 4-threads-per-pair kernel (128 threads)
 constexpr int kBigPB = 64;    // ... in the cooperative kernel's rounds above small_pairs (256 threads)
@@ -58,6 +57,7 @@ constexpr int kBigPB = 64;    // ... in the cooperative kernel's rounds above sm
 constexpr uint32_t kCoopQuadMinN = 20;
 constexpr int kTailPB = 32;   // pairs per chunk in the tail (512 threads)
 constexpr int kTailThreads = 16 * kTailPB;
+constexpr size_t kTailDynMax = 160 << 10;  // product gate: tables kept in shared memory (65 columns of 64 entries: 130 KB)
 
 // ------------------------------------------------------------------ args --
 
@@ -97,7 +97,7 @@ struct ScRoundArgs {
   int round;           // 0-based; first round of the tail for k_sc_tail
   int n, c;
   uint32_t gate, d;
-  int G;               // product gate: threads per pair
+  uint32_t tail_smem;  // tail: the tables stay in (dynamic) shared memory
   uint32_t spb;        // product gate: pairs per CTA (at most 256 / threads per pair)
   uint32_t nwork;      // CTAs that evaluate pairs (round 1 may add one for the inverses)
   uint32_t full;       // evaluate H at all of 0..d-1 (no point derived from the claim)
@@ -463,7 +463,7 @@ __device__ __forceinline__ uint32_t prod_point(int p, int np, bool full, uint32_
 }
 
 // Product gate f = q w1 .. w_{d-1} - o, or sum gate f = g_1 .. g_d + g_{d+1}
-// + .. + g_c, pair k: this thread's kPP points.  load(j, lo, hi) supplies
+// + .. + g_c, pair k: this thread's points.  load(j, lo, hi) supplies
 // column j of the pair (global memory or shared).  The degree-1 part (-o, or
 // the sum of the single columns) is added up at level 0 over the pair's two
 // ends first, then brought to the product's level 1-d by one kcomp
@@ -572,21 +572,16 @@ __device__ __forceinline__ fr plonk_at(const PlonkChunkSmem<PB>& S, int j, int p
   return pt == 2 ? fr_add(hi, dl) : dl;
 }
 
-template <int PB, int TPP, bool FULL, bool COHERENT>
-__device__ __forceinline__ void plonk_chunk(PlonkChunkSmem<PB>& S, const fr* const* src, fr* const* dst,
-                                            uint64_t h, uint64_t kbase, const fr& alpha, uint32_t p0,
-                                            const fr* ehi, const fr* elo, uint32_t mlo, fr& acc) {
-  constexpr int NPT = FULL ? 4 : 3, NF = NPT - 1, NITEM = 3 * NF + 2;
-  static_assert(TPP >= NPT, "one point per thread in phase 3");
+template <int PB, int TPP, bool COHERENT>
+__device__ __forceinline__ void plonk_chunk_fold(PlonkChunkSmem<PB>& S, const fr* const* src, fr* const* dst,
+                                                 uint64_t h, uint64_t kbase, const fr& alpha) {
   const int t = threadIdx.x, p = t % PB, slot = t / PB;
   const uint64_t k = kbase + p;
-  const bool live = k < h;
-  auto point = [&](int f) { return FULL ? f : (f == 0 ? (int)p0 : 2); };  // finite point f
 #pragma unroll
   for (int item = slot; item < 16; item += TPP) {
     const int j = item >> 1, half = item & 1;
     const uint64_t e = k + (half ? h : 0);
-    if (live) {
+    if (k < h) {
       const fr x0 = ldt<COHERENT>(src[j] + e), x1 = ldt<COHERENT>(src[j] + e + 2 * h);
       const fr v = fr_add(x0, fr_mul(alpha, fr_sub(x1, x0)));
       st_fr(dst[j] + e, v);
@@ -594,6 +589,18 @@ __device__ __forceinline__ void plonk_chunk(PlonkChunkSmem<PB>& S, const fr* con
     }
   }
   __syncthreads();
+}
+
+// Phases 2 and 3 on the folded values in S.V.
+template <int PB, int TPP, bool FULL, bool COHERENT>
+__device__ __forceinline__ void plonk_chunk_eval(PlonkChunkSmem<PB>& S, uint64_t h, uint64_t kbase, uint32_t p0,
+                                                 const fr* ehi, const fr* elo, uint32_t mlo, fr& acc) {
+  constexpr int NPT = FULL ? 4 : 3, NF = NPT - 1, NITEM = 3 * NF + 2;
+  static_assert(TPP >= NPT, "one point per thread in phase 3");
+  const int t = threadIdx.x, p = t % PB, slot = t / PB;
+  const uint64_t k = kbase + p;
+  const bool live = k < h;
+  auto point = [&](int f) { return FULL ? f : (f == 0 ? (int)p0 : 2); };  // finite point f
 #pragma unroll
   for (int q = slot; q < NITEM; q += TPP) {
     if (live) {
@@ -625,6 +632,14 @@ __device__ __forceinline__ void plonk_chunk(PlonkChunkSmem<PB>& S, const fr* con
     acc = fr_add(acc, fr_mul(v, S.U[NITEM - 1][p]));
   }
   __syncthreads();
+}
+
+template <int PB, int TPP, bool FULL, bool COHERENT>
+__device__ __forceinline__ void plonk_chunk(PlonkChunkSmem<PB>& S, const fr* const* src, fr* const* dst,
+                                            uint64_t h, uint64_t kbase, const fr& alpha, uint32_t p0,
+                                            const fr* ehi, const fr* elo, uint32_t mlo, fr& acc) {
+  plonk_chunk_fold<PB, TPP, COHERENT>(S, src, dst, h, kbase, alpha);
+  plonk_chunk_eval<PB, TPP, FULL, COHERENT>(S, h, kbase, p0, ehi, elo, mlo, acc);
 }
 
 // Sum the per-thread values of plonk_chunk over pairs: out[q] for q < NPT.
@@ -912,7 +927,7 @@ __global__ void __launch_bounds__(256) k_sc_fold(ScFoldArgs A) {
 // A product CTA's partial sums: point q is the sum of red[sl G + q / PP][q % PP]
 // over its spb pair slots.  Warps take points, lanes take slots.
 template <int PP>
-__device__ __forceinline__ void prod_cta_sums(const fr (&red)[256][PP], int np, int G, int spb, fr* out) {
+__device__ __forceinline__ void prod_cta_sums(const fr (*red)[PP], int np, int G, int spb, fr* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int q = warp; q < np; q += nw) {
     const int gq = q / PP, pq = q % PP;
@@ -1037,15 +1052,21 @@ __global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
 }
 
 // All rounds from A.round on, their challenges and the final values, in one
-// CTA of kTailThreads threads.  Tables are read with coherent loads: they
-// are rewritten between rounds inside this launch.
+// CTA of kTailThreads threads.  Latency is all there is here, so the folded
+// tables stay in shared memory from one round to the next when they fit
+// (A.tail_smem; the Plonk gate's chunk holds them anyway when the first round
+// has one chunk), a round's work is spread over all threads (product gate: one
+// point per thread), and every point is summed by a warp of its own.
+// Measured per round (product gate, d = 8: three points per thread, tables
+// through L2, points summed one after the other): 45 us, of which 19.5 the
+// evaluation and 9.6 the sums; the challenge is 10 to 14.
 template <bool PLONK>
-__global__ void __launch_bounds__(PLONK ? kTailThreads : 256, 1) k_sc_tail(ScRoundArgs A) {
+__global__ void __launch_bounds__(kTailThreads, 1) k_sc_tail(ScRoundArgs A) {
   __shared__ ChalSmem S;
   __shared__ fr pg[kMaxPts];
+  extern __shared__ __align__(16) unsigned char tail_dyn[];
   const DevConst* C = A.C;
   const int n = A.n, c = A.c, d = (int)A.d;
-  constexpr bool plonk = PLONK;
   const uint64_t N = 1ull << n;
   uint32_t bad = 0;
   // source of round i's pairs: the input for round 0, then the folded tables
@@ -1056,54 +1077,72 @@ __global__ void __launch_bounds__(PLONK ? kTailThreads : 256, 1) k_sc_tail(ScRou
     const uint32_t mlo = A.m_lo[i];
     const fr* ehi = A.E + A.eq_hi[i];
     const fr* elo = A.E + A.eq_lo[i];
-    int np;
+    const bool here = i > A.round && A.tail_smem;  // the tables are in shared memory
     if constexpr (PLONK) {
-      {  // i >= 1: round 1 never runs in the Plonk tail
-        np = 4;
-        fr acc = fr_zero();
-        const fr alpha = A.st->alpha[i - 1];
-        __shared__ PlonkChunkSmem<kTailPB> PS;
+      // i >= 1: round 1 never runs in the Plonk tail
+      fr acc = fr_zero();
+      const fr alpha = A.st->alpha[i - 1];
+      auto& PS = *reinterpret_cast<PlonkChunkSmem<kTailPB>*>(tail_dyn);
+      if (here) {
+        // entry e < 2h of the last table and its partner e + 2h are V[j][0][e] and V[j][1][e]
+        const int p = threadIdx.x % kTailPB, slot = threadIdx.x / kTailPB, j = slot >> 1, half = slot & 1;
+        fr v;
+        if (p < (int)h) {
+          const int e = half * (int)h + p;
+          const fr x0 = PS.V[j][0][e], x1 = PS.V[j][1][e];
+          v = fr_add(x0, fr_mul(alpha, fr_sub_lazy(x1, x0)));
+        }
+        __syncthreads();
+        if (p < (int)h) PS.V[j][half][p] = v;
+        __syncthreads();
+        plonk_chunk_eval<kTailPB, 16, true, true>(PS, h, 0, 0u, ehi, elo, mlo, acc);
+      } else {
         for (uint64_t kb = 0; kb < h; kb += kTailPB)
           plonk_chunk<kTailPB, 16, true, true>(PS, cur, A.dst, h, kb, alpha, 0u, ehi, elo, mlo, acc);
-        plonk_chunk_reduce<kTailPB, 4>(acc, pg);
+        for (int j = 0; j < c; j++) cur[j] = A.dst[j];
       }
-      for (int j = 0; j < c; j++) cur[j] = A.dst[j];
+      plonk_chunk_reduce<kTailPB, 4>(acc, pg);
     } else {
-      if (i > 0) {
-        const fr alpha = A.st->alpha[i - 1];
+      const bool first = i == 0;
+      const int np = d + 1;  // every tail round evaluates all of 0..d-1 and infinity (no derived point)
+      fr* const V = reinterpret_cast<fr*>(tail_dyn);
+      const uint64_t ld = N >> A.round;  // entries of a column in shared memory
+      if (!first || A.tail_smem) {
+        const fr alpha = first ? fr_zero() : A.st->alpha[i - 1];
         for (uint64_t e = threadIdx.x; e < 2 * h * (uint64_t)c; e += blockDim.x) {
           const int j = (int)(e / (2 * h));
           const uint64_t k = e - (uint64_t)j * 2 * h;
-          const fr x0 = ld_fr_l2(cur[j] + k), x1 = ld_fr_l2(cur[j] + k + 2 * h);
-          st_fr(A.dst[j] + k, fr_add(x0, fr_mul(alpha, fr_sub(x1, x0))));
+          fr x0 = cur[j][k];
+          if (!first) x0 = fr_add(x0, fr_mul(alpha, fr_sub_lazy(cur[j][k + 2 * h], x0)));
+          if (A.tail_smem) V[j * ld + k] = x0;
+          else st_fr(A.dst[j] + k, x0);
         }
         __syncthreads();
-        for (int j = 0; j < c; j++) cur[j] = A.dst[j];
+        if (i == A.round || !A.tail_smem)
+          for (int j = 0; j < c; j++) cur[j] = A.tail_smem ? V + j * ld : A.dst[j];
       }
-      // every tail round evaluates all of 0..d-1 and infinity (no derived point)
-      const bool first = i == 0;
-      np = d + 1;
-      const int G = A.G;
-      const int g = threadIdx.x % G;
-      const uint64_t nslots = blockDim.x / G;
-      const int pbeg = g * kPP, pcnt = max(0, min(kPP, np - pbeg));
-      fr acc[kPP];
-      uint32_t tpt[kPP];
-#pragma unroll
-      for (int p = 0; p < kPP; p++) {
-        acc[p] = fr_zero();
-        tpt[p] = p < pcnt ? prod_point(pbeg + p, np, true, 0u) : 0u;
+      const int slot = threadIdx.x / np, p = threadIdx.x % np, nslots = kTailThreads / np;
+      fr acc[1] = {fr_zero()};
+      const uint32_t tpt[1] = {prod_point(p, np, true, 0u)};
+      if (slot < nslots) {
+        for (uint64_t k = slot; k < h; k += nslots) {
+          const fr w = fr_mul(ld_fr_cg(ehi + (k >> mlo)), ld_fr_cg(elo + (k & ((1ull << mlo) - 1))));
+          prod_pair_g<1>(
+              A,
+              [&](int j, fr& lo, fr& hi) {
+                lo = cur[j][k];
+                hi = cur[j][k + h];
+              },
+              1, tpt, first, w, acc, bad);
+        }
       }
-      for (uint64_t k = threadIdx.x / G; k < h && pcnt > 0; k += nslots) {
-        const fr w = fr_mul(ld_fr_cg(ehi + (k >> mlo)), ld_fr_cg(elo + (k & ((1ull << mlo) - 1))));
-        prod_pair<kPP, true>(A, cur, k, h, pcnt, tpt, first, w, acc, bad);
-      }
-      // sum each point over all threads (threads outside its group add zero)
-      for (int p = 0; p < np; p++) {
-        fr v[1] = {(p >= pbeg && p < pbeg + pcnt) ? acc[p - pbeg] : fr_zero()};
-        block_sum<1>(v, pg + p);
-      }
+      __shared__ fr red[kTailThreads][1];
+      red[threadIdx.x][0] = acc[0];
+      __syncthreads();
+      prod_cta_sums<1>(red, np, np, (int)min((uint64_t)nslots, h), pg);
+      __syncthreads();
     }
+    const int np = PLONK ? 4 : d + 1;
     for (int p = threadIdx.x; p < np; p += blockDim.x) S.Hc[p] = pg[p];
     __syncthreads();
     sc_challenge<false>(S, np, d, i, A.st, A.proof, C, A.tabs, false, A.v2 != 0);
@@ -1115,9 +1154,17 @@ __global__ void __launch_bounds__(PLONK ? kTailThreads : 256, 1) k_sc_tail(ScRou
   if (threadIdx.x < (unsigned)c) {
     const int j = threadIdx.x;
     const fr alpha = A.st->alpha[n - 1];
-    const fr x0 = ld_fr_l2(cur[j]), x1 = ld_fr_l2(cur[j] + 1);
+    fr x0, x1;
+    if (PLONK && A.tail_smem) {
+      auto& PS = *reinterpret_cast<PlonkChunkSmem<kTailPB>*>(tail_dyn);
+      x0 = PS.V[j][0][0];
+      x1 = PS.V[j][1][0];
+    } else {
+      x0 = cur[j][0];
+      x1 = cur[j][1];
+    }
     fr v = fr_add(x0, fr_mul(alpha, fr_sub(x1, x0)));
-    if (plonk && j >= 5) v = from_mont(v);
+    if (PLONK && j >= 5) v = from_mont(v);
     for (int q = 0; q < 8; q++)
       for (int b = 0; b < 4; b++) pv[32 * j + 4 * q + b] = (uint8_t)(v.v[q] >> (8 * b));
   }
@@ -1152,7 +1199,7 @@ struct ScBuffers {
 };
 
 struct ScPlan {
-  int c, G, grid_plonk, grid_prod, npmax;
+  int c, grid_plonk, grid_prod, npmax;
   uint64_t tail_pairs, small_pairs, chunk_pairs;
   int grid_chunk, grid_quad;
   int grid_rounds;      // co-resident CTAs of the persistent round kernel
@@ -1165,21 +1212,46 @@ struct ScPlan {
   EqTask tasks[2 * kMaxN];
 };
 
-// grid: most CTAs per round kernel (0: two per SM); tail_log: the tail takes
-// over at 2^tail_log pairs (0: the gate's default).
-// The fused product kernel takes up to 48 KB of dynamic shared memory on top
-// of its static arrays: opt in once per device.
-static void ensure_prod_fused_attr() {
+// Unique id of the current CUDA context (0 if the driver cannot say).  A
+// cudaDeviceReset followed by new work creates a new primary context in
+// which the static arrays are fresh, so set-up must run again there.
+static unsigned long long current_context_id() {
+  typedef int (*GetCurrentFn)(void**);
+  typedef int (*GetIdFn)(void*, unsigned long long*);
+  static GetCurrentFn get_cur = nullptr;
+  static GetIdFn get_id = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaDriverEntryPointQueryResult q1, q2;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", (void**)&get_cur, 12000, cudaEnableDefault, &q1) !=
+            cudaSuccess || q1 != cudaDriverEntryPointSuccess)
+      get_cur = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", (void**)&get_id, 12000, cudaEnableDefault, &q2) !=
+            cudaSuccess || q2 != cudaDriverEntryPointSuccess)
+      get_id = nullptr;
+    cudaGetLastError();
+  });
+  void* cu = nullptr;
+  unsigned long long id = 0;
+  if (get_cur && get_id && get_cur(&cu) == 0 && cu && get_id(cu, &id) == 0) return id;
+  return 0;
+}
+
+// Kernels whose shared memory passes 48 KB opt in, once per device and context.
+static void ensure_smem_attr() {
   static std::mutex mu;
-  static bool done[64] = {};
+  static unsigned long long done[64] = {};  // context id, plus one
   int dev = 0;
   cudaGetDevice(&dev);
+  const unsigned long long id = current_context_id() + 1;
   std::lock_guard<std::mutex> lk(mu);
-  if (dev < 0 || dev >= 64 || done[dev]) return;
+  if (dev < 0 || dev >= 64 || done[dev] == id) return;
   cudaFuncSetAttribute(k_sc_prod_fused<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
   cudaFuncSetAttribute(k_sc_prod_fused<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
   cudaFuncSetAttribute(k_sc_plonk_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRoundsDyn);
-  done[dev] = true;
+  cudaFuncSetAttribute(k_sc_tail<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlonkChunkSmem<kTailPB>));
+  cudaFuncSetAttribute(k_sc_tail<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailDynMax);
+  done[dev] = id;
 }
 
 // Points per thread of a product round with np points over h pairs: one
@@ -1223,14 +1295,12 @@ static ScPlan sc_plan(const zc_params* p, int SMs, int grid = 0, int tail_log = 
   const uint32_t n = p->n, d = p->d;
   const bool plonk = p->gate == ZC_GATE_PLONK;
   P.c = gate_ncols(p->gate, d);
-  P.G = 1;
-  while (P.G * kPP < (int)d + 1) P.G *= 2;
   // default: one wave of resident CTAs for the Plonk kernels (register bound,
   // one CTA per SM), two waves for the product kernel
   P.grid_plonk = grid > 0 ? grid : SMs * resident_ctas(plonk_round_fn(minb == 1 ? 1 : 2));
   P.ppt = ppt == 1 || ppt == 3 ? ppt : 0;  // 0: per round (see prod_ppt)
   P.fuse_pairs = fuse > 0 ? 1ull << fuse : kFusePairsProd;
-  ensure_prod_fused_attr();
+  ensure_smem_attr();
   P.grid_prod = grid > 0 ? grid
                          : 2 * SMs * std::max(resident_ctas(reinterpret_cast<const void*>(k_sc_prod_round<1>)),
                                               resident_ctas(reinterpret_cast<const void*>(k_sc_prod_round<3>)));
@@ -1376,7 +1446,6 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
   R.c = c;
   R.gate = gate;
   R.d = d;
-  R.G = P.G;
   R.st = B.st;
   R.partials = B.partials;
   R.proof = B.proof;
@@ -1554,10 +1623,15 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
     R.dst[j] = B.tab[j];
   }
   R.nwork = 1;
-  if (plonk)
-    k_sc_tail<true><<<1, kTailThreads, 0, st>>>(R);
-  else
-    k_sc_tail<false><<<1, 256, 0, st>>>(R);
+  const uint64_t ht = N >> (i + 1);  // pairs of the tail's first round
+  if (plonk) {
+    R.tail_smem = i < n && ht <= (uint64_t)kTailPB ? 1u : 0u;
+    k_sc_tail<true><<<1, kTailThreads, sizeof(PlonkChunkSmem<kTailPB>), st>>>(R);
+  } else {
+    const uint64_t bytes = 2 * ht * (uint64_t)c * sizeof(fr);
+    R.tail_smem = i < n && bytes <= kTailDynMax ? 1u : 0u;
+    k_sc_tail<false><<<1, kTailThreads, R.tail_smem ? bytes : 0, st>>>(R);
+  }
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
 }
@@ -1714,32 +1788,6 @@ struct StaticDev {
 };
 static StaticDev g_static_dev[kStaticMaxDevices];
 static std::mutex g_static_mu;
-
-// Unique id of the current CUDA context (0 if the driver cannot say).  A
-// cudaDeviceReset followed by new work creates a new primary context in
-// which the static arrays are fresh, so set-up must run again there.
-static unsigned long long current_context_id() {
-  typedef int (*GetCurrentFn)(void**);
-  typedef int (*GetIdFn)(void*, unsigned long long*);
-  static GetCurrentFn get_cur = nullptr;
-  static GetIdFn get_id = nullptr;
-  static bool looked = false;
-  if (!looked) {  // called under g_static_mu
-    cudaDriverEntryPointQueryResult q1, q2;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", (void**)&get_cur, 12000, cudaEnableDefault, &q1) !=
-            cudaSuccess || q1 != cudaDriverEntryPointSuccess)
-      get_cur = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", (void**)&get_id, 12000, cudaEnableDefault, &q2) !=
-            cudaSuccess || q2 != cudaDriverEntryPointSuccess)
-      get_id = nullptr;
-    cudaGetLastError();
-    looked = true;
-  }
-  void* cu = nullptr;
-  unsigned long long id = 0;
-  if (get_cur && get_id && get_cur(&cu) == 0 && cu && get_id(cu, &id) == 0) return id;
-  return 0;
-}
 
 // Set-up for the current device: look up the device addresses of the static
 // arrays and copy the field constants into them.  Runs on the first call per
