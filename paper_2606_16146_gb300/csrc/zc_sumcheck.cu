@@ -302,6 +302,8 @@ __device__ void sc_challenge(ChalSmem& S, int np, int d, int i, ScState* st, uin
       S.alpha = a;
       S.alpha_raw = raw;
       if (release) {  // the next round needs only alpha: hand it off before c_i and the claim
+        st->alphac[i].w = raw;
+        st->alphac[i].q = fr_quot(a);
         __threadfence();
         atomicExch(release, (uint32_t)(i + 1));
       }
@@ -987,27 +989,25 @@ __global__ void __launch_bounds__(256, PP == 1 ? 3 : 2) k_sc_prod_round(ScRoundA
 }
 
 // Product-gate round i >= 2 with the MLE update fused: each CTA first
-// folds the (d+1) columns of its spb pairs by alpha_{i-1} (all threads,
-// coalesced; written back and kept in shared memory), then evaluates them
-// from shared memory as k_sc_prod_round does.  Dynamic shared memory:
-// (d+1) x 2 x spb elements.
-template <int PP>
-__global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
-  extern __shared__ __align__(16) fr Vs[];
-  const int i = A.round;
+// folds the columns of its spb pairs by alpha_{i-1} (all threads, coalesced;
+// written back and kept in shared memory), then evaluates them from shared
+// memory as k_sc_prod_round does, and sums its points into out[0..np).
+// Vs: c x 2 x spb elements.
+template <int PP, bool COHERENT>
+__device__ __forceinline__ void prod_fused_round(const ScRoundArgs& A, fr* Vs, const fr* const* src, int i, uint64_t h,
+                                                 bool full, int spb, uint32_t nwork, fr* out) {
   const int d = (int)A.d, c = A.c;
-  const bool full = A.full != 0;
   const int np = full ? d + 1 : d;
   const uint32_t p0 = full ? 0u : A.st->p0[i];
   const int G = (np + PP - 1) / PP;
-  const int spb = (int)A.spb;
   const int slot = (int)threadIdx.x / G, g = (int)threadIdx.x % G;
   const int pbeg = g * PP, pcnt = max(0, min(PP, np - pbeg));
   const uint32_t mlo = A.m_lo[i];
   const fr* ehi = A.E + A.eq_hi[i];
   const fr* elo = A.E + A.eq_lo[i];
-  const frc alpha = A.st->alphac[i - 1];
-  const uint64_t h = A.h;
+  frc alpha;
+  alpha.w = ldx<COHERENT>(&A.st->alphac[i - 1].w);
+  alpha.q = ldx<COHERENT>(&A.st->alphac[i - 1].q);
   uint32_t bad = 0;
   fr acc[PP];
   uint32_t tpt[PP];
@@ -1016,13 +1016,13 @@ __global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
     acc[p] = fr_zero();
     tpt[p] = p < pcnt ? prod_point(pbeg + p, np, full, p0) : 0u;
   }
-  for (uint64_t kb = (uint64_t)blockIdx.x * spb; kb < h; kb += (uint64_t)A.nwork * spb) {
+  for (uint64_t kb = (uint64_t)blockIdx.x * spb; kb < h; kb += (uint64_t)nwork * spb) {
     for (int e = threadIdx.x; e < c * 2 * spb; e += blockDim.x) {
       const int p = e % spb, rest = e / spb, half = rest & 1, j = rest >> 1;
       const uint64_t k = kb + p;
       if (k < h) {
         const uint64_t idx = k + (half ? h : 0);
-        const fr x0 = ld_fr_cs(A.src[j] + idx), x1 = ld_fr_cs(A.src[j] + idx + 2 * h);
+        const fr x0 = ldt<COHERENT>(src[j] + idx), x1 = ldt<COHERENT>(src[j] + idx + 2 * h);
         const fr v = fr_add(x0, fr_mulc(alpha, fr_sub_lazy(x1, x0)));
         st_fr(A.dst[j] + idx, v);
         Vs[(size_t)rest * spb + p] = v;
@@ -1046,9 +1046,75 @@ __global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
 #pragma unroll
   for (int p = 0; p < PP; p++) red[threadIdx.x][p] = acc[p];
   __syncthreads();
-  prod_cta_sums<PP>(red, np, G, spb, A.partials + (size_t)blockIdx.x * np);
+  prod_cta_sums<PP>(red, np, G, spb, out);
   __syncthreads();
+}
+
+// One such round per launch.  Dynamic shared memory: (d+1) x 2 x spb elements.
+template <int PP>
+__global__ void __launch_bounds__(256, 2) k_sc_prod_fused(ScRoundArgs A) {
+  extern __shared__ __align__(16) fr Vs[];
+  const int np = A.full ? (int)A.d + 1 : (int)A.d;
+  prod_fused_round<PP, false>(A, Vs, A.src, A.round, A.h, A.full != 0, (int)A.spb, A.nwork,
+                              A.partials + (size_t)blockIdx.x * np);
   sc_finish_round(A, np);
+}
+
+// Pairs per CTA of a fused round with np points on c columns: at most two fold
+// items and one point per thread.
+__host__ __device__ __forceinline__ int prod_fused_spb(int np, int c) {
+  const int a = 256 / np, b = 256 / c;
+  const int m = a < b ? a : b;
+  return m > 1 ? m : 1;
+}
+
+// Product-gate rounds [A.round, A.round_end) in one cooperative launch, one
+// point per thread: hand-offs and their bounds as in k_sc_plonk_rounds.  One
+// launch per round cost ~48 us a round at d = 8 (32 at d = 2), of which the
+// launch and the challenge's cold code are a third.
+constexpr size_t kProdRoundsDyn = 2 * 256 * sizeof(fr);
+__global__ void __launch_bounds__(256, 2) k_sc_prod_rounds(ScRoundArgs A) {
+  extern __shared__ __align__(16) fr Vs[];
+  __shared__ ChalSmem CS;
+  __shared__ int flag;  // 1: this CTA runs the challenge; 2: a wait gave up
+  const uint32_t G = gridDim.x;
+  const uint64_t N = 1ull << A.n;
+  const int d = (int)A.d;
+  for (int i = A.round; i < A.round_end; i++) {
+    const uint64_t h = N >> (i + 1);
+    const bool full = h <= A.small_pairs;
+    const int np = full ? d + 1 : d, spb = prod_fused_spb(np, A.c);
+    const uint32_t nwork = (uint32_t)min((h + spb - 1) / spb, (uint64_t)G);
+    if (blockIdx.x < nwork)
+      prod_fused_round<1, true>(A, Vs, i == A.round ? (const fr* const*)A.src : (const fr* const*)A.dst, i, h, full,
+                                spb, nwork, A.partials + (size_t)blockIdx.x * np);
+    if (threadIdx.x == 0) {
+      __threadfence();
+      const unsigned prev = atomicAdd(&A.st->counter[i], 1u);
+      flag = prev == G - 1 ? 1 : 0;
+    }
+    __syncthreads();
+    if (flag == 1) {
+      __threadfence();
+      sc_sum_partials(CS, A.partials, nwork, np);
+      sc_challenge<false>(CS, np, d, i, A.st, A.proof, A.C, A.tabs, h / 2 > A.small_pairs, A.v2 != 0, &A.st->go);
+    } else {
+      if (threadIdx.x == 0) {
+        uint32_t polls = 0;
+        while (ld_acquire_u32(&A.st->go) < (uint32_t)(i + 1)) {
+          if (++polls > A.spin_limit) {
+            atomicOr(&A.st->err, 2u);
+            flag = 2;
+            break;
+          }
+          __nanosleep(256);
+        }
+      }
+      __syncthreads();
+      if (flag == 2) return;
+    }
+    __syncthreads();
+  }
 }
 
 // All rounds from A.round on, their challenges and the final values, in one
@@ -1202,10 +1268,11 @@ struct ScPlan {
   int c, grid_plonk, grid_prod, npmax;
   uint64_t tail_pairs, small_pairs, chunk_pairs;
   int grid_chunk, grid_quad;
-  int grid_rounds;      // co-resident CTAs of the persistent round kernel
+  int grid_rounds;      // co-resident CTAs of the persistent round kernels
+  int grid_prod_rounds;
   uint64_t quad_pairs;  // Plonk rounds 2.. in (chunk_pairs, quad_pairs]: 4 threads per pair
   int minb;  // Plonk round kernels: resident CTAs per SM they are compiled for
-  int ppt;   // product round kernel: points per thread (1 or kPP; 0: by round, prod_ppt)
+  int ppt;   // product round kernel: points per thread (1 or 3; 0: by round, prod_ppt)
   uint64_t fuse_pairs;  // product rounds 2.. with at most this many pairs fold inside the evaluation
   int upload_chunks = 0;  // round 1 in this many pair-range launches (host columns), 0: one launch
   uint32_t eq_total, eq_hi[kMaxN], eq_lo[kMaxN], mlo[kMaxN];
@@ -1309,6 +1376,7 @@ static ScPlan sc_plan(const zc_params* p, int SMs, int grid = 0, int tail_log = 
   P.chunk_pairs = chunk_log > 0 ? 1ull << chunk_log : kChunkPairsPlonk;
   P.grid_chunk = SMs * resident_ctas(reinterpret_cast<const void*>(k_sc_plonk_chunk<16, kSmallPB, false>));
   P.grid_rounds = SMs * resident_ctas(reinterpret_cast<const void*>(k_sc_plonk_rounds), 16 * kSmallPB, kRoundsDyn);
+  P.grid_prod_rounds = SMs * resident_ctas(reinterpret_cast<const void*>(k_sc_prod_rounds), 256, kProdRoundsDyn);
   P.quad_pairs = quad_log > 0 ? 1ull << quad_log : kQuadPairsPlonk;
   P.grid_quad = SMs * resident_ctas(reinterpret_cast<const void*>(k_sc_plonk_chunk<4, kQuadPB, false>), 4 * kQuadPB);
   P.minb = minb == 1 ? 1 : 2;
@@ -1551,12 +1619,33 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
       }
       *launches += 1;
     } else {
+      if (i > 0 && h <= P.fuse_pairs && persistent && P.ppt != 3 && h / 2 > tail_pairs) {
+        // every remaining round before the tail in one cooperative launch
+        uint32_t end = i;
+        while (end < n && (N >> (end + 1)) > tail_pairs) end++;
+        R.round_end = (int)end;
+        R.spin_limit = persistent_spin_limit();
+        R.small_pairs = P.small_pairs;
+        const int spb = prod_fused_spb(R.full ? (int)d + 1 : (int)d, c);
+        const uint32_t G = (uint32_t)std::min<uint64_t>(std::min<uint64_t>((h + spb - 1) / spb, (uint64_t)P.grid_prod),
+                                                        (uint64_t)P.grid_prod_rounds);
+        R.nwork = G;
+        void* kargs[] = {&R};
+        if (G >= 2 && cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_sc_prod_rounds), dim3(G), dim3(256),
+                                                  kargs, kProdRoundsDyn, st) == cudaSuccess) {
+          for (int j = 0; j < c; j++) cur[j] = B.tab[j];
+          *launches += 1;
+          i = end;
+          break;
+        }
+        cudaGetLastError();  // not co-resident here: the per-round kernels below
+      }
       if (i > 0 && h <= P.fuse_pairs) {
         // fold fused into the evaluation (rounds 2..)
         const int npr = R.full ? (int)d + 1 : (int)d;
         const int ppt = prod_ppt(P.ppt, npr, h);
         // at most two fold items per thread: the round is latency-bound
-        const int G = (npr + ppt - 1) / ppt, spb = std::max(1, std::min(256 / G, 256 / c));
+        const int spb = prod_fused_spb((npr + ppt - 1) / ppt, c);
         R.spb = (uint32_t)spb;
         R.nwork = (uint32_t)std::min<uint64_t>((h + spb - 1) / spb, (uint64_t)P.grid_prod);
         const size_t dyn = sizeof(fr) * (size_t)c * 2 * spb;
