@@ -496,7 +496,7 @@ __device__ __forceinline__ void prod_pair_g(const ScRoundArgs& A, Load load, int
         tcur = tpt[p];
         x = e;
       }
-      prod[p] = j == 0 ? x : fr_mul(prod[p], x);
+      prod[p] = j == 0 ? x : fr_mul_inl(prod[p], x);
     }
   }
   if (c > d) {
@@ -530,7 +530,7 @@ __device__ __forceinline__ void prod_pair_g(const ScRoundArgs& A, Load load, int
   }
 #pragma unroll
   for (int p = 0; p < PP; p++)
-    if (p < pcnt) acc[p] = fr_add(acc[p], fr_mul(prod[p], w));
+    if (p < pcnt) acc[p] = fr_add(acc[p], fr_mul_inl(prod[p], w));
 }
 
 template <int PP, bool COHERENT>
