@@ -7,11 +7,11 @@
 // (the last leaf is shorter when 64 does not divide L), node =
 // SHA-256(left | right), and at a level with an odd count the last node
 // moves up unchanged; root = SHA-256(le64(len) | top).  One thread hashes
-// one 2 KB leaf; a CTA reduces its 128 leaves to one node in shared memory;
-// a second kernel reduces the CTA nodes of each column.  The CTAs' leaf
-// ranges start at multiples of 128, so their subtrees are the global tree's
-// first seven levels (a ragged last CTA's node arrives at level 7 unchanged,
-// as the odd last node of every level above it).
+// one 2 KB leaf; a CTA reduces its 128 (or 32) leaves to one node in shared
+// memory; a second kernel reduces the CTA nodes of each column.  The CTAs' leaf
+// ranges start at multiples of 128 (32), so their subtrees are the global
+// tree's first seven (five) levels (a ragged last CTA's node arrives at that
+// level unchanged, as the odd last node of every level above it).
 #include "zc_internal.cuh"
 #include "zc_transcript.cuh"
 
@@ -19,6 +19,7 @@ namespace zc {
 
 constexpr int kLeafElems = 64;
 constexpr int kLeafCta = 128;
+constexpr int kOnePairCtas = 152;  // one CTA per SM
 
 struct RootLeafArgs {
   const fr* col[kMaxCols];
@@ -86,27 +87,107 @@ __device__ __forceinline__ void sha256_node(const uint32_t* l, const uint32_t* r
   }
   sha256_init(out);
   sha256_compress(out, w);
+  uint32_t v[8];
 #pragma unroll
-  for (int i = 0; i < 16; i++) w[i] = 0;
-  w[0] = 0x80000000u;
-  w[15] = 512;
-  sha256_compress(out, w);
+  for (int i = 0; i < 8; i++) v[i] = out[i];
+#pragma unroll
+  for (int t = 0; t < 64; t++) sha_round(v, kShaPadKw.v[t]);
+#pragma unroll
+  for (int i = 0; i < 8; i++) out[i] += v[i];
 }
 
-__global__ void __launch_bounds__(kLeafCta) k_root_leaves(RootLeafArgs A) {
-  __shared__ uint32_t dig[kLeafCta][9];
+// barrier of one pair of warps (ids are immediates: an id in a register
+// reserves all sixteen)
+__device__ __forceinline__ void leaf_pair_sync(int pair) {
+  __syncwarp();
+  if (pair == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+  else if (pair == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
+  else if (pair == 2) asm volatile("bar.sync 3, 64;" ::: "memory");
+  else asm volatile("bar.sync 4, 64;" ::: "memory");
+}
+
+// 32 PAIRS leaves per CTA, one leaf per lane of a pair of warps: the first
+// warp runs the rounds, the second loads the leaf and computes the schedule, a
+// quarter of a block ahead, through shared memory.  A leaf is 33 blocks one
+// after the other, so with few leaves the time is theirs: on one warp the
+// rounds, the schedule and the block's loads added up to 3 us a block (100 us
+// whatever the size).  One pair per CTA keeps its two warps on two SM
+// quarters.  With many leaves (four pairs per CTA) the ALU pipe bounds both
+// forms, but the loads no longer wait in the chain (8 x 2^20 elements: 408 ->
+// 375 us).
+template <int PAIRS>
+__global__ void __launch_bounds__(64 * PAIRS) k_root_leaves(RootLeafArgs A) {
+  constexpr int kCta = 32 * PAIRS;
+  __shared__ uint32_t kw[PAIRS][64][32];
+  __shared__ uint32_t dig[kCta][9];
   const int c = blockIdx.y;
-  const uint64_t leaf = (uint64_t)blockIdx.x * kLeafCta + threadIdx.x;
-  uint64_t cnt64 = A.nleaves - (uint64_t)blockIdx.x * kLeafCta;
-  const uint32_t cnt = cnt64 < kLeafCta ? (uint32_t)cnt64 : kLeafCta;
-  uint32_t h[8];
-  if (threadIdx.x < cnt) {
-    const uint8_t* p = reinterpret_cast<const uint8_t*>(A.col[c] + leaf * A.per);
+  const int lane = threadIdx.x & 31, pair = (threadIdx.x >> 5) % PAIRS, id = 32 * pair + lane;
+  const bool rounds = threadIdx.x < kCta;
+  const uint64_t leaf = (uint64_t)blockIdx.x * kCta + id;
+  uint64_t cnt64 = A.nleaves - (uint64_t)blockIdx.x * kCta;
+  const uint32_t cnt = cnt64 < kCta ? (uint32_t)cnt64 : kCta;
+  // the leaf's 32-byte elements, and its 64-byte blocks with the padding
+  uint32_t elems = 0;
+  if ((uint32_t)id < cnt) {
     const uint64_t left = A.L - leaf * A.per;
-    const uint32_t elems = left < A.per ? (uint32_t)left : A.per;
-    sha256_device_mem(p, elems * 32, h);
+    elems = left < A.per ? (uint32_t)left : A.per;
+  }
+  const uint32_t nb = elems ? elems / 2 + 1 : 0, nbmax = __reduce_max_sync(0xffffffffu, nb);
+  uint32_t h[8];
+  sha256_init(h);
+  if (rounds) {
+    for (uint32_t b = 0; b < nbmax; b++) {
+      uint32_t v[8];
 #pragma unroll
-    for (int i = 0; i < 8; i++) dig[threadIdx.x][i] = h[i];
+      for (int i = 0; i < 8; i++) v[i] = h[i];
+#pragma unroll 1
+      for (int q = 0; q < 4; q++) {
+        leaf_pair_sync(pair);
+#pragma unroll
+        for (int i = 0; i < 16; i++) sha_round(v, kw[pair][16 * q + i][lane]);
+      }
+      if (b < nb) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) h[i] += v[i];
+      }
+    }
+  } else {
+    const uint4* p = reinterpret_cast<const uint4*>(A.col[c] + leaf * A.per);
+    // element e of the leaf as two 16-byte words, or the padding after the last
+    auto load = [&](uint32_t b, uint4 (&x)[4]) {
+#pragma unroll
+      for (int i = 0; i < 4; i++) x[i] = 2 * b + (i >> 1) < elems ? __ldg(p + 4 * b + i) : make_uint4(0, 0, 0, 0);
+    };
+    uint4 x[4];
+    load(0, x);
+    for (uint32_t b = 0; b < nbmax; b++) {
+      uint32_t w[16];
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        w[4 * i] = sha_bswap(x[i].x);
+        w[4 * i + 1] = sha_bswap(x[i].y);
+        w[4 * i + 2] = sha_bswap(x[i].z);
+        w[4 * i + 3] = sha_bswap(x[i].w);
+      }
+      if (b + 1 >= nb) {
+        w[elems & 1 ? 8 : 0] = 0x80000000u;
+        w[15] = elems * 256;
+      }
+      if (b + 1 < nbmax) load(b + 1, x);
+#pragma unroll
+      for (int i = 0; i < 16; i++) kw[pair][i][lane] = w[i] + kShaK[i];
+      leaf_pair_sync(pair);
+#pragma unroll 1
+      for (int q = 1; q < 4; q++) {
+#pragma unroll
+        for (int i = 0; i < 16; i++) kw[pair][16 * q + i][lane] = sha_sched(w, i) + kShaK[16 * q + i];
+        leaf_pair_sync(pair);
+      }
+    }
+  }
+  if (rounds) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) dig[id][i] = h[i];
   }
   for (uint32_t w = cnt; w > 1; w = (w + 1) / 2) {
     __syncthreads();
@@ -184,17 +265,28 @@ zc_status launch_roots(zc_ctx* ctx, const fr* const* dcols, int c, uint64_t L, u
   la.L = L;
   la.per = L < (uint64_t)kLeafElems ? (uint32_t)L : (uint32_t)kLeafElems;
   la.nleaves = (L + la.per - 1) / la.per;
-  la.ctas = (uint32_t)((la.nleaves + kLeafCta - 1) / kLeafCta);
-  size_t words = (size_t)c * la.ctas * 8;
-  uint32_t* nodes = ctx->arena.take<uint32_t>(words);
-  uint32_t* tmp = ctx->arena.take<uint32_t>(words);
-  if (!nodes || !tmp) {
+  // few leaves: one pair of warps per CTA, at most one CTA per SM (its larger
+  // node arrays must fit; the scratch need counts four pairs per CTA)
+  uint32_t* nodes = nullptr;
+  uint32_t* tmp = nullptr;
+  bool one = false;
+  const size_t used = ctx->arena.used;
+  auto carve = [&](int leaves) {
+    la.ctas = (uint32_t)((la.nleaves + leaves - 1) / leaves);
+    nodes = ctx->arena.take<uint32_t>((size_t)c * la.ctas * 8);
+    tmp = ctx->arena.take<uint32_t>((size_t)c * la.ctas * 8);
+    if (!nodes || !tmp) ctx->arena.used = used;
+    return nodes && tmp;
+  };
+  if ((uint64_t)c * la.nleaves <= 32ull * kOnePairCtas) one = carve(32);
+  if (!one && !carve(kLeafCta)) {
     ctx->err = "root: scratch arena too small";
     return ZC_ERR_OOM;
   }
   la.nodes = nodes;
   dim3 grid(la.ctas, c);
-  k_root_leaves<<<grid, kLeafCta, 0, st>>>(la);
+  if (one) k_root_leaves<1><<<grid, 64, 0, st>>>(la);
+  else k_root_leaves<4><<<grid, 2 * kLeafCta, 0, st>>>(la);
   ctx->launches++;
   RootTopArgs ta{};
   ta.nodes = nodes;
@@ -204,6 +296,7 @@ zc_status launch_roots(zc_ctx* ctx, const fr* const* dcols, int c, uint64_t L, u
   ta.roots = droots;
   k_root_top<<<c, 256, 0, st>>>(ta);
   ctx->launches++;
+  ctx->arena.used = used;  // the nodes are free again for what follows on the stream
   ZC_CUDA_TRY(ctx, cudaGetLastError());
   return ZC_OK;
 }

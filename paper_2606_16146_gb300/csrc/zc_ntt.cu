@@ -618,7 +618,8 @@ struct NttZArgs {
   int c;
   uint32_t n;
   uint32_t S0[8];
-  fr* zpow;              // z^(2^i), i < 31 (level 1)
+  fr* zpow;              // z^(2^i), i < nz (level 1)
+  uint32_t nz;           // powers the openings use, z^N and z^32 among them
   const DevConst* C;
 };
 
@@ -637,7 +638,7 @@ __global__ void __launch_bounds__(64) k_ntt_z(NttZArgs A) {
     if (threadIdx.x == 0) {
       fr p = fr_mul(raw, C->r2);
       A.st->z = p;
-      for (uint32_t i = 0; i < 31; i++) {
+      for (uint32_t i = 0; i < A.nz; i++) {
         A.zpow[i] = p;
         if (i == A.n) {
           A.st->zpow_n = p;
@@ -1545,6 +1546,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     za.n = n;
     transcript_init_words(za.S0, ZC_FORM_NTT, gate, n, d, D.word);
     za.zpow = zpow;
+    za.nz = std::max<uint32_t>(logm + (D.step ? 1 : 0), std::max<uint32_t>(n, 5)) + 1;
     za.C = ctx->dconst;
     k_ntt_z<<<1, 64, 0, st>>>(za);
     ctx->launches++;

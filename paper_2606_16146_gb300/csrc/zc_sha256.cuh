@@ -29,7 +29,7 @@ ZC_SHA_K_DECL const uint32_t kShaK[64] = {
 #if !defined(__CUDACC__)
 static const uint32_t* sha_k_host() { return kShaK; }
 #else
-static const uint32_t kShaKHost[64] = {
+static constexpr uint32_t kShaKHost[64] = {
     0x428a2f98, 0x71374491, 0xb5c0fbcf, 0xe9b5dba5, 0x3956c25b, 0x59f111f1, 0x923f82a4, 0xab1c5ed5,
     0xd807aa98, 0x12835b01, 0x243185be, 0x550c7dc3, 0x72be5d74, 0x80deb1fe, 0x9bdc06a7, 0xc19bf174,
     0xe49b69c1, 0xefbe4786, 0x0fc19dc6, 0x240ca1cc, 0x2de92c6f, 0x4a7484aa, 0x5cb0a9dc, 0x76f988da,
@@ -55,6 +55,49 @@ ZC_HD uint32_t sha_bswap(uint32_t x) {
   return (x >> 24) | ((x >> 8) & 0xff00u) | ((x << 8) & 0xff0000u) | (x << 24);
 #endif
 }
+
+#if defined(__CUDACC__)
+// Schedule words plus round constants of the padding block that ends a
+// 64-byte message (0x80, zeros, the length 512): the same for every tree node.
+struct ShaPadKw {
+  uint32_t v[64];
+};
+constexpr uint32_t sha_rotr_c(uint32_t x, int n) { return (x >> n) | (x << (32 - n)); }
+constexpr ShaPadKw sha_pad_kw() {
+  ShaPadKw k{};
+  uint32_t w[64] = {0x80000000u, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 512};
+  for (int t = 16; t < 64; t++)
+    w[t] = w[t - 16] + (sha_rotr_c(w[t - 15], 7) ^ sha_rotr_c(w[t - 15], 18) ^ (w[t - 15] >> 3)) + w[t - 7] +
+           (sha_rotr_c(w[t - 2], 17) ^ sha_rotr_c(w[t - 2], 19) ^ (w[t - 2] >> 10));
+  for (int t = 0; t < 64; t++) k.v[t] = w[t] + kShaKHost[t];
+  return k;
+}
+static __device__ __constant__ const ShaPadKw kShaPadKw = sha_pad_kw();
+
+// One round; kw is the schedule word plus the round constant.
+__device__ __forceinline__ void sha_round(uint32_t (&s)[8], uint32_t kw) {
+  const uint32_t a = s[0], b = s[1], c = s[2], e = s[4], f = s[5], g = s[6];
+  const uint32_t t1 = s[7] + (sha_rotr(e, 6) ^ sha_rotr(e, 11) ^ sha_rotr(e, 25)) + ((e & f) ^ (~e & g)) + kw;
+  const uint32_t t2 = (sha_rotr(a, 2) ^ sha_rotr(a, 13) ^ sha_rotr(a, 22)) + ((a & b) | (c & (a | b)));
+  s[7] = g;
+  s[6] = f;
+  s[5] = e;
+  s[4] = s[3] + t1;
+  s[3] = c;
+  s[2] = b;
+  s[1] = a;
+  s[0] = t1 + t2;
+}
+
+// schedule words 16 q + 16 .. from the ring w of the sixteen before, i of q
+__device__ __forceinline__ uint32_t sha_sched(uint32_t (&w)[16], int i) {
+  const uint32_t x15 = w[(i + 1) & 15], x2 = w[(i + 14) & 15];
+  const uint32_t s0 = sha_rotr(x15, 7) ^ sha_rotr(x15, 18) ^ (x15 >> 3);
+  const uint32_t s1 = sha_rotr(x2, 17) ^ sha_rotr(x2, 19) ^ (x2 >> 10);
+  w[i] = w[i] + s0 + w[(i + 9) & 15] + s1;
+  return w[i];
+}
+#endif
 
 // Compress one 64-byte block given as 16 big-endian message words.
 ZC_HD void sha256_compress(uint32_t h[8], const uint32_t w_in[16]) {

@@ -45,43 +45,27 @@ __device__ __forceinline__ void sha_pair_schedule(ShaPair& Z, const uint32_t* bl
 #pragma unroll 1
   for (int q = 0; q < 3; q++) {
 #pragma unroll
-    for (int i = 0; i < 16; i++) {
-      const uint32_t x15 = w[(i + 1) & 15], x2 = w[(i + 14) & 15];
-      const uint32_t s0 = sha_rotr(x15, 7) ^ sha_rotr(x15, 18) ^ (x15 >> 3);
-      const uint32_t s1 = sha_rotr(x2, 17) ^ sha_rotr(x2, 19) ^ (x2 >> 10);
-      w[i] = w[i] + s0 + w[(i + 9) & 15] + s1;
-      Z.kw[16 * q + i] = w[i] + kShaK[16 * q + 16 + i];
-    }
+    for (int i = 0; i < 16; i++) Z.kw[16 * q + i] = sha_sched(w, i) + kShaK[16 * q + 16 + i];
     pair_sync();
   }
 }
 
 // warp 0: h <- compress(h, blk)
 __device__ __forceinline__ void sha_pair_rounds(ShaPair& Z, const uint32_t* blk, uint32_t h[8]) {
-  uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
-  auto round = [&](uint32_t k) {
-    const uint32_t t1 = hh + (sha_rotr(e, 6) ^ sha_rotr(e, 11) ^ sha_rotr(e, 25)) + ((e & f) ^ (~e & g)) + k;
-    const uint32_t t2 = (sha_rotr(a, 2) ^ sha_rotr(a, 13) ^ sha_rotr(a, 22)) + ((a & b) | (c & (a | b)));
-    hh = g;
-    g = f;
-    f = e;
-    e = d + t1;
-    d = c;
-    c = b;
-    b = a;
-    a = t1 + t2;
-  };
+  uint32_t v[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) v[i] = h[i];
   pair_sync();
 #pragma unroll
-  for (int i = 0; i < 16; i++) round(kShaK[i] + blk[i]);
+  for (int i = 0; i < 16; i++) sha_round(v, kShaK[i] + blk[i]);
 #pragma unroll 1
   for (int q = 0; q < 3; q++) {
     pair_sync();
 #pragma unroll
-    for (int i = 0; i < 16; i++) round(Z.kw[16 * q + i]);
+    for (int i = 0; i < 16; i++) sha_round(v, Z.kw[16 * q + i]);
   }
-  h[0] += a; h[1] += b; h[2] += c; h[3] += d;
-  h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
+#pragma unroll
+  for (int i = 0; i < 8; i++) h[i] += v[i];
 }
 
 // One block by both warps (warp 0: h updated; warp 1: h untouched).
