@@ -665,6 +665,16 @@ struct NttOpenArgs {
   uint32_t seg;       // elements per warp segment (multiple of 32)
 };
 
+// Steps per warp segment of the openings: a segment ends in one product by
+// z^base (up to log2 M products), which 128 steps hide; with fewer than ~512
+// such segments in the longest vector the chain of steps is the time, so the
+// segments get shorter, down to 8 steps (n = 12: one warp per column and 128
+// steps took 128 us).
+static uint32_t open_steps(uint64_t M) {
+  const uint64_t m = M / (32 * 512);
+  return (uint32_t)(m < 8 ? 8 : m > 128 ? 128 : m);
+}
+
 __device__ fr zpow_of(const fr* zp, uint64_t e, const fr& one) {
   fr acc = one;
   for (int i = 0; e; i++, e >>= 1)
@@ -1564,13 +1574,14 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     oa.len[c] = M;
     oa.zpow = zpow;
     oa.partials = opart;
-    oa.nblk = nblk_open;
-    oa.seg = 32 * 128;
-    k_ntt_open<<<dim3(nblk_open, c + 1), 256, 0, st>>>(oa, ctx->dconst);
+    oa.seg = 32 * open_steps(M);
+    const uint32_t nblk = (uint32_t)std::min<uint64_t>(nblk_open, (M + 8ull * oa.seg - 1) / (8ull * oa.seg));
+    oa.nblk = nblk;
+    k_ntt_open<<<dim3(nblk, c + 1), 256, 0, st>>>(oa, ctx->dconst);
     ctx->launches++;
     NttFinalArgs fa{};
     fa.partials = opart;
-    fa.nblk = nblk_open;
+    fa.nblk = nblk;
     fa.c = c;
     fa.gate = gate;
     fa.n = n;
