@@ -142,6 +142,8 @@ struct NttPassArgs {
   uint32_t logL;          // sub-DFT length
   uint32_t logW;          // sub-DFTs per CTA
   uint32_t B;             // sub-DFTs (a CTA's surplus ones are neither read nor written)
+  uint32_t out_y, pre_y;  // slice blockIdx.y: elements from one slice's outputs, and pre factors, to the next's
+  uint32_t in_y;          // ... and inputs (0: every slice reads the same)
   NttMap im, om;          // element (b, t) of a column
   FrcTab dft;             // stage twiddles, forward or inverse
   frc w8, w4, w83;        // w_8, w_4, w_8^3
@@ -272,7 +274,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   // lanes to an element; a warp copies its own slots only.
   {
     const uint32_t half = tid & 1;
-    const char* in = reinterpret_cast<const char*>(A.in[item]) + 16 * half;
+    const char* in = reinterpret_cast<const char*>(A.in[item] + (size_t)A.in_y * blockIdx.y) + 16 * half;
 #pragma unroll
     for (int s = 0; s < 2; s++) {
       const uint32_t i = (tid & ~31u) + ((tid & 31) >> 1) + 16 * s;
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
       // groups, and there k = j
       const uint32_t j = elt(tid), km = (1u << logNs) - 1;
       const FrcTab first = base.at(tw ? (ptrdiff_t)(stage_tab(logNs, lr) + (FAST ? j & km : 0)) - (ptrdiff_t)(km + 1)
-                                     : (ptrdiff_t)index(m, tid));
+                                     : (ptrdiff_t)index(m, tid) + (fin ? 0 : (ptrdiff_t)A.pre_y * blockIdx.y));
       auto fac = [&](int p) {
         if (tw) {
           const uint32_t g = p & ((1u << lg) - 1), r = (uint32_t)p >> lg;
@@ -383,7 +385,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   // of its own element and swaps the other for that half of its neighbour's.
   // Without a post table the values are lazy: reduced, or multiplied here.
   const bool odd = tid & 1;
-  char* const out = reinterpret_cast<char*>(A.out[item]) + 16 * odd;
+  char* const out = reinterpret_cast<char*>(A.out[item] + (size_t)A.out_y * blockIdx.y) + 16 * odd;
   char* const oe = out + sizeof(fr) * (size_t)index(A.om, tid & ~1u);  // the even lane's element
   char* const oo = out + sizeof(fr) * (size_t)index(A.om, tid | 1u);
 #pragma unroll
@@ -513,8 +515,9 @@ __global__ void k_ntt_slice_tables(NttSliceTabArgs A) {
   }
 }
 
-struct NttGateArgs {
+struct NttGateArgs {      // slice blockIdx.y of the launch
   const fr* col[kMaxCols];  // slice evaluations, level 1
+  uint64_t col_y;           // elements from one slice's evaluations to the next's
   fr* qhat;                 // slice output
   const frc* zinv;          // constant of this slice
   const fr* sub;            // nullptr, or values subtracted after the scaling (level 1)
@@ -525,26 +528,28 @@ struct NttGateArgs {
 // f at the slice points, times the slice constant 1 / (z_H M): Plonk; product
 // q w1 .. w_{d-1} - o; sum g_1 .. g_d + g_{d+1} + .. + g_c (all at level 1).
 __global__ void __launch_bounds__(256) k_ntt_gate(NttGateArgs A) {
-  const frc zi = ld_frc(A.zinv);
+  const frc zi = ld_frc(A.zinv + blockIdx.y);
+  const uint64_t cy = A.col_y * blockIdx.y;
+  auto col = [&](uint32_t j, uint64_t p) { return ld_fr(A.col[j] + cy + p); };
   for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < A.N;
        p += (uint64_t)gridDim.x * blockDim.x) {
     fr f;
     if (A.gate == ZC_GATE_PLONK) {
       // a (qL + qM b) + qR b + qO c with one reduction for the three products
-      const fr b = ld_fr(A.col[6] + p);
-      const fr u = fr_add(ld_fr(A.col[0] + p), fr_mul_inl(ld_fr(A.col[2] + p), b));
-      f = fr_mul_sum3(ld_fr(A.col[5] + p), u, ld_fr(A.col[1] + p), b, ld_fr(A.col[3] + p), ld_fr(A.col[7] + p));
-      f = fr_add(f, ld_fr(A.col[4] + p));
+      const fr b = col(6, p);
+      const fr u = fr_add(col(0, p), fr_mul_inl(col(2, p), b));
+      f = fr_mul_sum3(col(5, p), u, col(1, p), b, col(3, p), col(7, p));
+      f = fr_add(f, col(4, p));
     } else {
-      f = ld_fr(A.col[0] + p);
-      for (uint32_t j = 1; j < A.d; j++) f = fr_mul_inl(f, ld_fr(A.col[j] + p));
-      if (A.gate == ZC_GATE_PRODUCT) f = fr_sub(f, ld_fr(A.col[A.d] + p));
+      f = col(0, p);
+      for (uint32_t j = 1; j < A.d; j++) f = fr_mul_inl(f, col(j, p));
+      if (A.gate == ZC_GATE_PRODUCT) f = fr_sub(f, col(A.d, p));
       else
-        for (uint32_t j = A.d; j < A.c; j++) f = fr_add(f, ld_fr(A.col[j] + p));
+        for (uint32_t j = A.d; j < A.c; j++) f = fr_add(f, col(j, p));
     }
     f = fr_mulc(zi, f);
     if (A.sub) f = fr_sub(f, ld_fr(A.sub + p));
-    st_fr(A.qhat + p, f);
+    st_fr(A.qhat + A.N * blockIdx.y + p, f);
   }
 }
 
@@ -827,7 +832,7 @@ static zc_status ensure_tables(zc_ctx* ctx, cudaStream_t st, NttTables** out) {
 // resident CTAs per SM (caps registers).  The context's tuning picks the tile
 // and residency.
 template <int MAXT, int MINB>
-static void launch_pass_variant(const NttPassArgs& a, uint32_t grid, uint32_t tile, cudaStream_t st) {
+static void launch_pass_variant(const NttPassArgs& a, dim3 grid, uint32_t tile, cudaStream_t st) {
   if (a.logL >= 3 && tile >= 512 && !(a.B & ((1u << a.logW) - 1)) && a.pre != PRE_COSET &&
       (a.post == POST_NONE || a.post == POST_TAB))
     k_ntt_pass<MAXT, MINB, true><<<grid, tile / 8, tile * sizeof(fr), st>>>(a);
@@ -864,7 +869,7 @@ static void set_dft(NttPassArgs& a, const NttTables* T, bool inverse) {
 }
 
 // launch one batched pass over `items` columns
-static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int items, uint64_t B) {
+static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int items, uint64_t B, uint32_t slices = 1) {
   const uint32_t logL = a.logL;
   uint32_t logTile = (uint32_t)ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_TILE_LOG);
   const int minb = ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_MINB);
@@ -879,7 +884,7 @@ static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int item
   const uint32_t tile = 1u << (a.logW + logL);
   a.items = (uint32_t)items;
   a.B = (uint32_t)B;
-  const uint32_t grid = (uint32_t)(blocks * (uint64_t)items);
+  const dim3 grid((uint32_t)(blocks * (uint64_t)items), slices);
   if (logTile == 12) launch_pass_variant<512, 1>(a, grid, tile, st);
   else if (logTile == 11 && minb != 1) launch_pass_variant<256, 2>(a, grid, tile, st);
   else if (logTile == 11) launch_pass_variant<256, 1>(a, grid, tile, st);
@@ -1184,6 +1189,16 @@ zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st) {
   return cudaStreamSynchronize(st) == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
 }
 
+// Slices of N2 per launch: while one slice's passes have at most two waves of
+// CTAs (1024 elements each, four per SM), several slices share a launch: each
+// alone leaves most of the GPU idle for as long as a full one (n = 12: 3 x 54
+// us of the proof's 670).
+static uint32_t slices_per_launch(int sm_count, int c, uint64_t N, uint64_t s) {
+  uint32_t k = 1;
+  while (2 * k <= s && 2 * k * ((uint64_t)c * N / 1024 + 1) <= 8ull * sm_count) k *= 2;
+  return k;
+}
+
 zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, int on_dev,
                     const uint8_t (*roots)[32], cudaStream_t st, uint8_t* proof,
                     bool proof_on_dev, void* q_out, int q_on_dev) {
@@ -1217,14 +1232,28 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   const uint32_t nlo = 1u << hbits, nhi = 1u << (n - hbits);
   const uint32_t nblk_open = 2 * (uint32_t)ctx->sm_count;
   const bool q_direct = q_out && q_on_dev;
-  zc_status s1 = ensure_arena(ctx, ntt_scratch_bytes(p, ctx->sm_count, q_direct));
+  // several slices per launch take more scratch than the proof needs: used
+  // when the arena has it or may grow, never on lanes (captured, or a block of
+  // the serving pool) and within the memory budget
+  const size_t need = ntt_scratch_bytes(p, ctx->sm_count, q_direct);
+  const uint64_t Na = std::max<uint64_t>(N, 8);  // buffers of 256 bytes at least
+  uint32_t sb = slices_per_launch(ctx->sm_count, c, N, s);
+  const size_t more = (size_t)(sb - 1) * c * Na * sizeof(fr);
+  if (ctx->arena.cap < need + more &&
+      (ctx->table_owner || ctx->arena_borrowed || (ctx->budget && need + more > ctx->budget) ||
+       ensure_arena(ctx, need + more) != ZC_OK)) {
+    ctx->err.clear();
+    sb = 1;
+  }
+  zc_status s1 = ensure_arena(ctx, need);
   if (s1 != ZC_OK) return s1;
   Arena& ar = ctx->arena;
   ar.reset();
   fr* coef[kMaxCols];
   fr* slb[kMaxCols];
   for (int j = 0; j < c; j++) coef[j] = ar.take<fr>(N);
-  for (int j = 0; j < c; j++) slb[j] = ar.take<fr>(N);
+  fr* const slices = ar.take<fr>((size_t)sb * c * Na);
+  for (int j = 0; j < c; j++) slb[j] = slices + j * Na;
   fr* qhat = ar.take<fr>(M);
   fr* qv = q_direct ? static_cast<fr*>(q_out) : ar.take<fr>(M);
   fr* rho = D.step ? ar.take<fr>(N) : nullptr;   // q_big reduced mod x^N - sigma^N
@@ -1254,6 +1283,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     ctx->err = "step-radix domain: per-size tables unavailable";
     return ZC_ERR_OOM;
   }
+  if (!ST) sb = 1;
 
   // N1's first pass (rows over i2, twiddled) for the columns [j0, j1)
   auto n1_first = [&](const fr* const* in, int j0, int j1) -> zc_status {
@@ -1373,10 +1403,10 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
 
   // ---- N2: per slice, coset NTT of every column, gate, divide by z_H.
   // slice_lde: the coset NTT of the `items` coefficient vectors in[] into
-  // out[] on one slice, with the coset factor table pre (per-size tables)
+  // out[] on one slice, or on sb slices from j on, with the coset factor table pre (per-size tables)
   // or slice j's two-level tables (without them).
   auto slice_lde = [&](const fr* const* in, fr* const* out, int items, const FrcTab* pre, uint64_t j,
-                       bool mark) -> zc_status {
+                       bool mark, uint32_t sb) -> zc_status {
     NttPassArgs a;
     pass_defaults(a);
     for (int i = 0; i < items; i++) {
@@ -1387,6 +1417,8 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     a.pre_lo = tlo + j * nlo;
     a.pre_hi = thi + j * nhi;
     a.pre_shift = hbits;
+    a.out_y = (uint32_t)(c * Na);
+    a.pre_y = (uint32_t)N;
     set_dft(a, T, false);
     if (two) {
       a.logL = l1;                     // columns over k1: k = L2 k1 + k2
@@ -1398,7 +1430,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
         a.post = POST_TAB; a.post_tab = ST->tw_fwd;
         a.qm = map_flat(l1, 0);
       }
-      if ((rs = run_pass(ctx, st, a, items, L2)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, items, L2, sb)) != ZC_OK) return rs;
       if (mark) ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[7], st));
       pass_defaults(a);
       for (int i = 0; i < items; i++) {
@@ -1407,23 +1439,25 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       }
       a.logL = l2;                     // rows over k2
       a.im = a.om = map_flat(l2, 0);
+      a.in_y = a.out_y = (uint32_t)(c * Na);
       set_dft(a, T, false);
-      if ((rs = run_pass(ctx, st, a, items, L1)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, items, L1, sb)) != ZC_OK) return rs;
     } else {
       a.logL = n;
       a.im = a.om = a.pm = map_flat(0, 0);
       if (ST) {
         a.pre = PRE_TAB; a.pre_tab = *pre;
       }
-      if ((rs = run_pass(ctx, st, a, items, 1)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, items, 1, sb)) != ZC_OK) return rs;
       if (mark) ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[7], st));
     }
     return ZC_OK;
   };
   // gate and division by z_H (constant zi on the slice), minus sub if given
-  auto slice_gate = [&](fr* out, const frc* zi, const fr* sub) {
+  auto slice_gate = [&](fr* out, const frc* zi, const fr* sub, uint32_t sb) {
     NttGateArgs ga{};
     for (int i = 0; i < c; i++) ga.col[i] = slb[i];
+    ga.col_y = c * Na;
     ga.qhat = out;
     ga.zinv = zi;
     ga.sub = sub;
@@ -1432,13 +1466,13 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     ga.d = d;
     ga.c = (uint32_t)c;
     uint32_t gb = (uint32_t)std::min<uint64_t>((N + 255) / 256, (uint64_t)ctx->sm_count * 8);
-    k_ntt_gate<<<gb, 256, 0, st>>>(ga);
+    k_ntt_gate<<<dim3(gb, sb), 256, 0, st>>>(ga);
     ctx->launches++;
   };
-  for (uint64_t j = 0; j < s; j++) {
+  for (uint64_t j = 0; j < s; j += sb) {
     const FrcTab cs = ST ? ST->coset.at(j * N) : FrcTab();
-    if ((rs = slice_lde(coef, slb, c, ST ? &cs : nullptr, j, j == 0)) != ZC_OK) return rs;
-    slice_gate(qhat + j * N, (ST ? ST->zinv : zinv) + j, nullptr);
+    if ((rs = slice_lde(coef, slb, c, ST ? &cs : nullptr, j, j == 0, sb)) != ZC_OK) return rs;
+    slice_gate(qhat + j * N, (ST ? ST->zinv : zinv) + j, nullptr, sb);
   }
   ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[3], st));
 
@@ -1521,9 +1555,9 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     ctx->launches++;
     const fr* rin[1] = {rho};
     fr* rout[1] = {vsm};
-    if ((rs = slice_lde(rin, rout, 1, &ST->step_coset, 0, false)) != ZC_OK) return rs;
-    if ((rs = slice_lde(coef, slb, c, &ST->step_coset, 0, false)) != ZC_OK) return rs;
-    slice_gate(qhat + Mb, reinterpret_cast<const frc*>(ST->step_const), vsm);
+    if ((rs = slice_lde(rin, rout, 1, &ST->step_coset, 0, false, 1)) != ZC_OK) return rs;
+    if ((rs = slice_lde(coef, slb, c, &ST->step_coset, 0, false, 1)) != ZC_OK) return rs;
+    slice_gate(qhat + Mb, reinterpret_cast<const frc*>(ST->step_const), vsm, 1);
     if ((rs = inverse(qhat + Mb, qv + Mb, 1, 0, n)) != ZC_OK) return rs;
     NttStepCombineArgs ca{};
     ca.q = qv;
@@ -1604,10 +1638,10 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     ZC_CUDA_TRY(ctx, cudaMemcpyAsync(q_out, qv, M * sizeof(fr), cudaMemcpyDeviceToHost, st));
   }
   ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[6], st));
-  // dominant launch: one N2 column pass over all c columns of a slice
+  // dominant launch: one N2 column pass over all c columns of sb slices
   const double Lc = two ? (double)l1 : (double)n;
-  ctx->dom_mulmods = (double)c * (double)N / 2 * Lc + (double)c * (double)N;
-  ctx->dom_bytes = 2.0 * 32 * c * (double)N;
+  ctx->dom_mulmods = sb * ((double)c * (double)N / 2 * Lc + (double)c * (double)N);
+  ctx->dom_bytes = sb * (2.0 * 32 * c * (double)N);
   ctx->dom_a = 2;
   ctx->dom_b = 7;
   if (!proof_on_dev || !on_dev || (q_out && !q_direct)) {
