@@ -386,16 +386,34 @@ static fr host_gate(uint32_t gate, uint32_t d, const fr* x, const DevConst& C) {
   return pr;
 }
 
-static fr host_lagrange(const fr* y, int m, const fr& x, const DevConst& C) {
-  fr acc = fr_zero();
+// 1 / prod_{q != t} (t - q) for the nodes t = 0..m-1, one inversion for all
+static std::vector<fr> host_lagrange_dens(int m, const DevConst& C) {
+  std::vector<fr> den(m), pre(m + 1, h_from_u64(1));
   for (int t = 0; t < m; t++) {
-    fr num = h_from_u64(1), den = h_from_u64(1);
-    for (int s = 0; s < m; s++) {
-      if (s == t) continue;
-      num = h_canon_mul(num, fr_sub_g(x, h_from_u64((uint64_t)s)), C);
-      den = h_canon_mul(den, h_signed(t - s), C);
-    }
-    acc = fr_add_g(acc, h_canon_mul(y[t], h_canon_mul(num, h_inv(den, C), C), C));
+    den[t] = h_from_u64(1);
+    for (int q = 0; q < m; q++)
+      if (q != t) den[t] = h_canon_mul(den[t], h_signed(t - q), C);
+    pre[t + 1] = h_canon_mul(pre[t], den[t], C);
+  }
+  fr inv = h_inv(pre[m], C);
+  for (int t = m - 1; t >= 0; t--) {
+    const fr d = den[t];
+    den[t] = h_canon_mul(inv, pre[t], C);
+    inv = h_canon_mul(inv, d, C);
+  }
+  return den;
+}
+
+// the polynomial with values y at 0..m-1, at x (dinv: host_lagrange_dens(m))
+static fr host_lagrange(const fr* y, int m, const fr* dinv, const fr& x, const DevConst& C) {
+  // prod_{q != t} (x - q) from prefix and suffix products
+  std::vector<fr> suf(m + 1, h_from_u64(1));
+  for (int t = m - 1; t > 0; t--) suf[t] = h_canon_mul(suf[t + 1], fr_sub_g(x, h_from_u64((uint64_t)t)), C);
+  fr acc = fr_zero(), pre = h_from_u64(1);
+  for (int t = 0; t < m; t++) {
+    const fr w = h_canon_mul(h_canon_mul(pre, suf[t + 1], C), dinv[t], C);
+    acc = fr_add_g(acc, h_canon_mul(y[t], w, C));
+    pre = h_canon_mul(pre, fr_sub_g(x, h_from_u64((uint64_t)t)), C);
   }
   return acc;
 }
@@ -437,6 +455,7 @@ static zc_status sumcheck_replay(const zc_params* p, const void* const* cols, co
   const fr one1 = h_from_u64(1);
   const uint8_t* pp = proof + 16;
   std::vector<fr> G(per);
+  const std::vector<fr> dinv = host_lagrange_dens((int)per, C);
   for (uint32_t i = 0; i < n; i++) {
     for (uint32_t t = 0; t < per; t++)
       if (!h_from_bytes(pp + 32 * t, &G[t])) return ZC_ERR_ARG;
@@ -449,7 +468,7 @@ static zc_status sumcheck_replay(const zc_params* p, const void* const* cols, co
     tr.absorb(pp, 32 * (size_t)per);
     pp += 32 * (size_t)per;
     al[i] = tr.squeeze();
-    claim = host_lagrange(G.data(), (int)per, al[i], C);
+    claim = host_lagrange(G.data(), (int)per, dinv.data(), al[i], C);
     if (v2) {
       const fr li = fr_add_g(h_canon_mul(fr_sub_g(one1, r[i]), fr_sub_g(one1, al[i]), C),
                              h_canon_mul(r[i], al[i], C));

@@ -430,12 +430,11 @@ zc_status zc_pcs_open(zc_pcs* P, const uint8_t (*alpha)[32], const uint8_t (*val
   ga.m = S.m;
   const uint64_t tot = (uint64_t)S.t * S.c * S.m;
   k_pcs_gather<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(ga);
-  std::vector<uint8_t> cols((size_t)tot * 32);
-  PCS_TRY(ctx, cudaMemcpyAsync(cols.data(), dg, cols.size(), cudaMemcpyDeviceToHost, st));
+  // the queried columns go straight to their places between the paths
+  const size_t per = (size_t)S.c * S.m * 32, pitch = per + 32 * (size_t)S.logW;
+  PCS_TRY(ctx, cudaMemcpy2DAsync(pp, pitch, dg, per, per, S.t, cudaMemcpyDeviceToHost, st));
   PCS_TRY(ctx, cudaStreamSynchronize(st));
-  const size_t per = (size_t)S.c * S.m * 32;
   for (uint32_t s2 = 0; s2 < S.t; s2++) {
-    std::memcpy(pp, &cols[s2 * per], per);
     pp += per;
     uint64_t off = 0, cnt = S.W, idx = ks[s2];
     for (uint32_t lv = 0; lv < S.logW; lv++) {

@@ -102,42 +102,52 @@ __device__ __forceinline__ uint32_t sha_sched(uint32_t (&w)[16], int i) {
 // Compress one 64-byte block given as 16 big-endian message words.
 ZC_HD void sha256_compress(uint32_t h[8], const uint32_t w_in[16]) {
 #if defined(__CUDA_ARCH__)
-  const uint32_t* K = kShaK;
-#elif defined(__CUDACC__)
+  uint32_t w[16], v[8];
+#pragma unroll
+  for (int i = 0; i < 16; i++) w[i] = w_in[i];
+#pragma unroll
+  for (int i = 0; i < 8; i++) v[i] = h[i];
+#pragma unroll
+  for (int t = 0; t < 64; t++) sha_round(v, (t < 16 ? w[t] : sha_sched(w, t & 15)) + kShaK[t]);
+#pragma unroll
+  for (int i = 0; i < 8; i++) h[i] += v[i];
+#else
+#if defined(__CUDACC__)
   const uint32_t* K = kShaKHost;
 #else
   const uint32_t* K = sha_k_host();
 #endif
-  uint32_t w[16];
-#pragma unroll
+  // eight rounds per step with the registers renamed instead of moved (host
+  // compilers do not unroll the round loop by themselves)
+  uint32_t w[16], s[8];
   for (int i = 0; i < 16; i++) w[i] = w_in[i];
-  uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
-#pragma unroll
-  for (int t = 0; t < 64; t++) {
-    uint32_t wt;
-    if (t < 16) {
-      wt = w[t];
-    } else {
-      uint32_t x15 = w[(t + 1) & 15], x2 = w[(t + 14) & 15];
-      uint32_t s0 = sha_rotr(x15, 7) ^ sha_rotr(x15, 18) ^ (x15 >> 3);
-      uint32_t s1 = sha_rotr(x2, 17) ^ sha_rotr(x2, 19) ^ (x2 >> 10);
-      wt = w[t & 15] + s0 + w[(t + 9) & 15] + s1;
-      w[t & 15] = wt;
-    }
-    uint32_t t1 = hh + (sha_rotr(e, 6) ^ sha_rotr(e, 11) ^ sha_rotr(e, 25)) + ((e & f) ^ (~e & g)) +
-                  K[t] + wt;
-    uint32_t t2 = (sha_rotr(a, 2) ^ sha_rotr(a, 13) ^ sha_rotr(a, 22)) + ((a & b) | (c & (a | b)));
-    hh = g;
-    g = f;
-    f = e;
-    e = d + t1;
-    d = c;
-    c = b;
-    b = a;
-    a = t1 + t2;
+  for (int i = 0; i < 8; i++) s[i] = h[i];
+  auto round = [](uint32_t a, uint32_t b, uint32_t c, uint32_t& d, uint32_t e, uint32_t f, uint32_t g, uint32_t& x,
+                  uint32_t kw) {
+    const uint32_t t1 = x + (sha_rotr(e, 6) ^ sha_rotr(e, 11) ^ sha_rotr(e, 25)) + ((e & f) ^ (~e & g)) + kw;
+    d += t1;
+    x = t1 + (sha_rotr(a, 2) ^ sha_rotr(a, 13) ^ sha_rotr(a, 22)) + ((a & b) | (c & (a | b)));
+  };
+  for (int t = 0; t < 64; t += 8) {
+    if (t >= 16)
+      for (int i = t & 15; i < (t & 15) + 8; i++) {
+        const uint32_t x15 = w[(i + 1) & 15], x2 = w[(i + 14) & 15];
+        w[i] += (sha_rotr(x15, 7) ^ sha_rotr(x15, 18) ^ (x15 >> 3)) + w[(i + 9) & 15] +
+                (sha_rotr(x2, 17) ^ sha_rotr(x2, 19) ^ (x2 >> 10));
+      }
+    const uint32_t* k = K + t;
+    const uint32_t* u = w + (t & 15);
+    round(s[0], s[1], s[2], s[3], s[4], s[5], s[6], s[7], k[0] + u[0]);
+    round(s[7], s[0], s[1], s[2], s[3], s[4], s[5], s[6], k[1] + u[1]);
+    round(s[6], s[7], s[0], s[1], s[2], s[3], s[4], s[5], k[2] + u[2]);
+    round(s[5], s[6], s[7], s[0], s[1], s[2], s[3], s[4], k[3] + u[3]);
+    round(s[4], s[5], s[6], s[7], s[0], s[1], s[2], s[3], k[4] + u[4]);
+    round(s[3], s[4], s[5], s[6], s[7], s[0], s[1], s[2], k[5] + u[5]);
+    round(s[2], s[3], s[4], s[5], s[6], s[7], s[0], s[1], k[6] + u[6]);
+    round(s[1], s[2], s[3], s[4], s[5], s[6], s[7], s[0], k[7] + u[7]);
   }
-  h[0] += a; h[1] += b; h[2] += c; h[3] += d;
-  h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
+  for (int i = 0; i < 8; i++) h[i] += s[i];
+#endif
 }
 
 ZC_HD void sha256_init(uint32_t h[8]) {
@@ -170,6 +180,17 @@ struct Sha256 {
     }
   }
   ZC_HD void update(const uint8_t* m, uint64_t len) {
+    while (len && nbytes) {
+      put_byte(*m++);
+      len--;
+    }
+    for (; len >= 64; m += 64, len -= 64) {  // whole blocks; blk stays zero
+      uint32_t w[16];
+      for (int i = 0; i < 16; i++)
+        w[i] = ((uint32_t)m[4 * i] << 24) | ((uint32_t)m[4 * i + 1] << 16) | ((uint32_t)m[4 * i + 2] << 8) | m[4 * i + 3];
+      sha256_compress(h, w);
+      total += 64;
+    }
     for (uint64_t i = 0; i < len; i++) put_byte(m[i]);
   }
   // 32-bit little-endian words, e.g. a field element's limbs
