@@ -19,6 +19,7 @@ namespace zc {
 
 constexpr int kLeafElems = 64;
 constexpr int kLeafCta = 128;
+constexpr uint64_t kTopNodes = 1024;  // commitment tree: from here up in one CTA (512 threads, a node each)
 constexpr int kOnePairCtas = 152;  // one CTA per SM
 
 struct RootLeafArgs {
@@ -362,6 +363,23 @@ __global__ void k_pcs_level(PcsLevelArgs A) {
   for (int i = 0; i < 8; i++) A.out[8 * u + i] = h[i];
 }
 
+// The tree's levels from cnt nodes (a power of two, at in) up to the top, each
+// level after the one below it: one CTA, where a launch per level took 7 us of
+// which the node hash is 2.5.
+__global__ void __launch_bounds__(512) k_pcs_top(uint32_t* in, uint64_t cnt) {
+  for (; cnt > 1; cnt /= 2) {
+    uint32_t* out = in + 8 * cnt;
+    for (uint64_t u = threadIdx.x; u < cnt / 2; u += blockDim.x) {
+      uint32_t h[8];
+      sha256_node(in + 16 * u, in + 16 * u + 8, h);
+#pragma unroll
+      for (int i = 0; i < 8; i++) out[8 * u + i] = h[i];
+    }
+    __syncthreads();
+    in = out;
+  }
+}
+
 zc_status pcs_hash_tree(zc_ctx* ctx, const fr* const* enc, int c, uint64_t m, uint64_t W, uint32_t* dig,
                         uint32_t* tree, cudaStream_t st) {
   PcsDigestArgs da{};
@@ -382,6 +400,11 @@ zc_status pcs_hash_tree(zc_ctx* ctx, const fr* const* enc, int c, uint64_t m, ui
   ctx->launches++;
   uint64_t off = 0;
   for (uint64_t cnt = W; cnt > 1; cnt /= 2) {
+    if (cnt <= kTopNodes) {
+      k_pcs_top<<<1, 512, 0, st>>>(tree + 8 * off, cnt);
+      ctx->launches++;
+      break;
+    }
     la.in = tree + 8 * off;
     la.out = tree + 8 * (off + cnt);
     la.count = cnt / 2;
