@@ -419,6 +419,60 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   }
 }
 
+// The same pass for launches too small to fill the GPU: two elements per
+// thread and radix-2 stages, so a thread's chain is a product per stage instead
+// of a dozen, on four times the threads (n = 12: a pass takes 20 to 30 us with
+// eight elements per thread, of which the products in a row are most).  Element
+// tid + NT p, p < 2; the stages exchange through two tiles in turn.  Whole
+// tiles, 2 <= L <= 1024, all factors from tables.
+__global__ void __launch_bounds__(512) k_ntt_pass_small(NttPassArgs A) {
+  extern __shared__ __align__(16) uint4 sm_planes[];
+  const uint32_t NT = blockDim.x, tid = threadIdx.x;
+  const uint32_t item = blockIdx.x % A.items;
+  const uint32_t logL = A.logL, logW = A.logW, Wm = (1u << logW) - 1;
+  const uint32_t b = ((blockIdx.x / A.items) << logW) + (tid & Wm);  // NT is a multiple of W
+  const uint32_t t0 = tid >> logW, t1 = (tid + NT) >> logW;
+  const fr* in = A.in[item] + (size_t)A.in_y * blockIdx.y;
+  fr x0 = ld_fr(in + A.im.at(b, t0)), x1 = ld_fr(in + A.im.at(b, t1));
+  if (A.err && !(fr_is_canonical(x0) && fr_is_canonical(x1))) atomicOr(A.err, 1u);
+  if (A.pre == PRE_TAB) {
+    const FrcTab f = A.pre_tab.at((ptrdiff_t)A.pre_y * blockIdx.y);
+    x0 = fr_mulc(f.ld(A.pm.at(b, t0)), x0);
+    x1 = fr_mulc(f.ld(A.pm.at(b, t1)), x1);
+  }
+  for (uint32_t logNs = 0; logNs < logL; logNs++) {
+    if (logNs > 0) {
+      // w_{2 Ns}^k = w_4096^(4 k'), k' = k 512 / Ns: the radix-8 table at stride 512, r = 4
+      const uint32_t k = t0 & ((1u << logNs) - 1);
+      x0 = fr_reduce1(x0);
+      x1 = fr_mulc(A.dft.ld(stage_tab(9, 3) + 3 * 512 + (k << (9 - logNs))), x1);
+    }
+    const fr y0 = fr_add_lazy(x0, x1), y1 = fr_sub_lazy(x0, x1);
+    if (logNs + 1 == logL) {
+      x0 = y0;
+      x1 = y1;
+      break;
+    }
+    const SmTile sm{sm_planes + (logNs & 1) * 4 * NT, 2 * NT};
+    const uint32_t ls = logNs + logW, q = ((tid >> ls) << (ls + 1)) + (tid & ((1u << ls) - 1));
+    sm.put(q, y0);
+    sm.put(q + (1u << ls), y1);
+    __syncthreads();
+    x0 = sm.get(tid);
+    x1 = sm.get(tid + NT);
+  }
+  if (A.post == POST_TAB) {
+    x0 = fr_mulc(A.post_tab.ld(A.qm.at(b, t0)), x0);
+    x1 = fr_mulc(A.post_tab.ld(A.qm.at(b, t1)), x1);
+  } else {
+    x0 = fr_reduce1(x0);
+    x1 = fr_reduce1(x1);
+  }
+  fr* out = A.out[item] + (size_t)A.out_y * blockIdx.y;
+  st_fr(out + A.om.at(b, t0), x0);
+  st_fr(out + A.om.at(b, t1), x1);
+}
+
 // ----------------------------------------------------- per-size tables --
 // For one (n, log2 s): the four-step twiddles of size N in both directions,
 // the coset factors (7 w_M^j)^k / N of every slice (level 2, which also
@@ -841,6 +895,7 @@ static void launch_pass_variant(const NttPassArgs& a, dim3 grid, uint32_t tile, 
 }
 
 static void set_pass_attributes() {
+  cudaFuncSetAttribute(k_ntt_pass_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 * 64);
   cudaFuncSetAttribute(k_ntt_pass<128, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 * 32);
   cudaFuncSetAttribute(k_ntt_pass<128, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 * 32);
   cudaFuncSetAttribute(k_ntt_pass<256, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2048 * 32);
@@ -860,6 +915,12 @@ static void ensure_pass_attributes(int dev) {
   }
 }
 
+// Launches of at most this many elements take two per thread (proofs by limit
+// 2^17 / 2^18 / 2^19 / 2^20: n = 14 472, 474, 461, 462 us; n = 16 834, 815,
+// 822, 838; n = 17 1320, 1322, 1308, 1405; with eight always n = 12 441
+// against 390).
+constexpr uint64_t kSmallElems = 1ull << 19;
+
 static void set_dft(NttPassArgs& a, const NttTables* T, bool inverse) {
   const frc* c = inverse ? T->c_inv : T->c_fwd;
   a.dft = inverse ? T->dft_inv : T->dft_fwd;
@@ -871,6 +932,20 @@ static void set_dft(NttPassArgs& a, const NttTables* T, bool inverse) {
 // launch one batched pass over `items` columns
 static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int items, uint64_t B, uint32_t slices = 1) {
   const uint32_t logL = a.logL;
+  // few elements: two per thread, tiles of 256 (or one sub-DFT)
+  if (logL >= 1 && logL <= 10 && (uint64_t)items * slices * (B << logL) <= kSmallElems && a.pre != PRE_COSET &&
+      (a.post == POST_NONE || a.post == POST_TAB)) {
+    const uint32_t lt = std::max<uint32_t>(logL, 8);
+    if ((B << logL) % (1ull << lt) == 0) {
+      a.logW = lt - logL;
+      a.items = (uint32_t)items;
+      a.B = (uint32_t)B;
+      const dim3 grid((uint32_t)((B >> a.logW) * (uint64_t)items), slices);
+      k_ntt_pass_small<<<grid, 1u << (lt - 1), 2 * sizeof(fr) << lt, st>>>(a);
+      ctx->launches++;
+      return ZC_OK;
+    }
+  }
   uint32_t logTile = (uint32_t)ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_TILE_LOG);
   const int minb = ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_MINB);
   if (logTile < logL) logTile = logL < 10 ? 10 : logL;
