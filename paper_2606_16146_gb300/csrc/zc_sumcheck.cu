@@ -593,6 +593,29 @@ __device__ __forceinline__ void plonk_chunk_fold(PlonkChunkSmem<PB>& S, const fr
   __syncthreads();
 }
 
+// Phase 1 of round 1: the input's values instead of folded ones, checked, the
+// wires brought to level 1, every column copied to dst (the later rounds of the
+// launch read all their tables there).
+template <int PB, int TPP>
+__device__ __forceinline__ void plonk_chunk_load(PlonkChunkSmem<PB>& S, const fr* const* src, fr* const* dst,
+                                                 uint64_t h, uint64_t kbase, const frc& mont, uint32_t& bad) {
+  const int t = threadIdx.x, p = t % PB, slot = t / PB;
+  const uint64_t k = kbase + p;
+#pragma unroll
+  for (int item = slot; item < 16; item += TPP) {
+    const int j = item >> 1, half = item & 1;
+    const uint64_t e = k + (half ? h : 0);
+    if (k < h) {
+      fr v = ldt<true>(src[j] + e);
+      bad |= !fr_is_canonical(v);
+      if (j >= 5) v = fr_mulc(mont, v);
+      st_fr(dst[j] + e, v);
+      S.V[j][half][p] = v;
+    }
+  }
+  __syncthreads();
+}
+
 // Phases 2 and 3 on the folded values in S.V.
 template <int PB, int TPP, bool FULL, bool COHERENT>
 __device__ __forceinline__ void plonk_chunk_eval(PlonkChunkSmem<PB>& S, uint64_t h, uint64_t kbase, uint32_t p0,
@@ -831,7 +854,9 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
   return v;
 }
 
-// Plonk rounds [A.round, A.round_end) in one cooperative launch, so the
+// Plonk rounds [A.round, A.round_end) in one cooperative launch (for small
+// proofs from round 1 on: as a launch of its own, one pair per thread, it took
+// 57 us at n = 12, most of it cold code), so the
 // latency-bound rounds pay no launch between them and their challenge code
 // stays warm.  Rounds with more than A.small_pairs pairs take 4 threads per
 // pair and derive one of H(0), H(1) from the claim (as k_sc_plonk_chunk<4,
@@ -858,14 +883,23 @@ __global__ void __launch_bounds__(16 * kSmallPB) k_sc_plonk_rounds(ScRoundArgs A
   const uint64_t N = 1ull << A.n;
   for (int i = A.round; i < A.round_end; i++) {
     const uint64_t h = N >> (i + 1);
-    const bool big = h > A.small_pairs;
+    const bool big = i > 0 && h > A.small_pairs;
     const int np = big ? 3 : 4;
     const uint64_t pb = big ? kBigPB : kSmallPB;
     const uint32_t nwork = (uint32_t)min((h + pb - 1) / pb, (uint64_t)G);
-    const fr alpha = ld_fr_l2(&A.st->alpha[i - 1]);
+    const fr alpha = i > 0 ? ld_fr_l2(&A.st->alpha[i - 1]) : fr_zero();
     const fr* const* src = i == A.round ? (const fr* const*)A.src : (const fr* const*)A.dst;
     fr acc = fr_zero();
-    if (big) {
+    if (i == 0) {  // round 1 (never derives a point)
+      uint32_t bad = 0;
+      if (blockIdx.x < nwork)
+        for (uint64_t kb = (uint64_t)blockIdx.x * kSmallPB; kb < h; kb += (uint64_t)nwork * kSmallPB) {
+          plonk_chunk_load<kSmallPB, 16>(S, src, A.dst, h, kb, A.mont, bad);
+          plonk_chunk_eval<kSmallPB, 16, true, true>(S, h, kb, 0u, A.E + A.eq_hi[i], A.E + A.eq_lo[i], A.m_lo[i], acc);
+        }
+      if (bad) atomicOr(&A.st->err, 1u);
+      plonk_chunk_reduce<kSmallPB, 4>(acc, part);
+    } else if (big) {
       const uint32_t p0 = A.st->p0[i];
       if (blockIdx.x < nwork)
         for (uint64_t kb = (uint64_t)blockIdx.x * kBigPB; kb < h; kb += (uint64_t)nwork * kBigPB)
@@ -1459,7 +1493,7 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
                             const ScBuffers& B, const DevConst* dC, const fr* dtabs,
                             const DevConst& hC, int skip_point, cudaStream_t st,
                             uint32_t* launches, cudaEvent_t* ev, bool v2 = false,
-                            bool persistent = false, const ScUpload* up = nullptr) {
+                            bool persistent = false, const ScUpload* up = nullptr, bool* round1_fused = nullptr) {
   const uint32_t gate = p->gate, n = p->n, d = p->d;
   const int c = P.c;
   const uint64_t N = 1ull << n;
@@ -1554,7 +1588,10 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
       R.dst[j] = B.tab[j];
     }
     const uint64_t coop_max = n >= kCoopQuadMinN ? std::max(P.chunk_pairs, P.quad_pairs) : P.chunk_pairs;
-    if (plonk && i > 0 && h <= coop_max && persistent && (R.full || n >= kCoopQuadMinN) && h / 2 > tail_pairs) {
+    // small proofs: round 1 as well, when no later round needs the inverses
+    const bool coop1 = i == 0 && !need_inv && !up && h <= 2 * P.chunk_pairs;
+    if (plonk && (coop1 || (i > 0 && h <= coop_max)) && persistent && (R.full || n >= kCoopQuadMinN) &&
+        h / 2 > tail_pairs) {
       // every remaining round before the tail in one cooperative launch
       // (those above small_pairs derive a point, the others evaluate every point)
       uint32_t end = i;
@@ -1562,7 +1599,7 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
       R.round_end = (int)end;
       R.spin_limit = persistent_spin_limit();
       R.small_pairs = P.small_pairs;
-      const uint64_t pb0 = h > P.small_pairs ? (uint64_t)kBigPB : (uint64_t)kSmallPB;
+      const uint64_t pb0 = i > 0 && h > P.small_pairs ? (uint64_t)kBigPB : (uint64_t)kSmallPB;
       const uint32_t G = (uint32_t)std::min<uint64_t>(
           std::min<uint64_t>((h + pb0 - 1) / pb0, (uint64_t)P.grid_chunk), (uint64_t)P.grid_rounds);
       R.nwork = G;
@@ -1571,6 +1608,8 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
                                                 dim3(16 * kSmallPB), kargs, kRoundsDyn, st) == cudaSuccess) {
         for (int j = 0; j < 8; j++) cur[j] = B.tab[j];
         *launches += 1;
+        if (i == 0 && ev) cudaEventRecord(ev[3], st);
+        if (i == 0 && round1_fused) *round1_fused = true;
         i = end;
         break;
       }
@@ -1817,8 +1856,11 @@ zc_status sumcheck_prove(zc_ctx* ctx, const zc_params* p, const void* const* col
   }
   ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[1], st));
   uint32_t launches = 0;
+  bool fused = false;
   s = sc_enqueue(p, Pm, src, B, ctx->dconst, ctx->dtabs, ctx->hconst, ctx->skip_point, st, &launches,
-                 ctx->ev, v2, persistent_allowed(ctx, st), chunked ? &up : nullptr);
+                 ctx->ev, v2, persistent_allowed(ctx, st), chunked ? &up : nullptr, &fused);
+  // round 1 in the cooperative launch: the events bracket its rounds' whole work
+  if (fused) ctx->dom_mulmods = (double)(N - 1) * ((d + 1) * (g_mul + 1) + 1 + c);
   ctx->launches += launches;
   if (s != ZC_OK) {
     ctx->err = "kernel launch failed";
