@@ -414,7 +414,8 @@ zc_status zc_serve(zc_ctx* ctx, const zc_request* reqs, uint32_t count, const zc
  *                        round 2 at the earliest); 1..24, default 5.
  *   ZC_TUNE_SC_SMALL_LOG SumCheck: rounds 2.. with at most 2^value pairs
  *                        evaluate both H(0) and H(1) instead of deriving one
- *                        from the claim; 1..24, default 14.
+ *                        from the claim; 1..24, default 14 (Plonk gate from
+ *                        n = 20 on: 13).
  *   ZC_TUNE_SC_CHUNK_LOG SumCheck, Plonk gate: rounds 2.. with at most 2^value
  *                        pairs spread each pair over 16 threads; 1..24,
  *                        default 14.  From n = 20 on, the rounds inside the
