@@ -781,9 +781,14 @@ __global__ void __launch_bounds__(256) k_ntt_open(NttOpenArgs A, const DevConst*
     const uint64_t cnt = A.seg < len - base ? A.seg : len - base;
     const uint32_t mcount = (uint32_t)((cnt + 31) / 32);
     fr acc = fr_zero();
-    for (int32_t m = (int32_t)mcount - 1; m >= 0; m--) {
+    auto value = [&](int32_t m) {
       const uint64_t k = base + lane + 32ull * (uint32_t)m;
-      const fr xk = k < len ? ld_fr(x + k) : fr_zero();
+      return m >= 0 && k < len ? ld_fr(x + k) : fr_zero();
+    };
+    fr nx = value((int32_t)mcount - 1);  // the next step's value is loaded during the present product
+    for (int32_t m = (int32_t)mcount - 1; m >= 0; m--) {
+      const fr xk = nx;
+      nx = value(m - 1);
       // while the warp's accumulators and values are all zero (the zero top
       // of an honest quotient) the step would multiply zeros: skip it
       if (__all_sync(0xffffffffu, fr_is_zero(acc) && fr_is_zero(xk))) continue;
