@@ -392,6 +392,12 @@ __device__ void sc_finish_round(const ScRoundArgs& A, int np) {
 
 // ------------------------------------------------------- per-pair work --
 
+// x0 + alpha (x1 - x0), one out-of-line copy for the sixteen folds of a pair
+// (inlined, 38 KB of code: n = 22 2598 against 2548 us); alpha in shared memory
+static __device__ __noinline__ fr fold_call(const frc* alpha, fr x0, fr x1) {
+  return fr_add(x0, fr_mulc(*alpha, fr_sub_lazy(x1, x0)));
+}
+
 // Plonk gate, pair k of a round: loads (and, after round 1, folds by
 // alpha) every column, evaluates at the finite points and infinity and adds
 // eq-weighted values into acc.  Columns stream in the order b, qM, qL, a,
@@ -417,8 +423,8 @@ __device__ __forceinline__ void plonk_pair(const fr* const* src, fr* const* dst,
     } else {
       const fr x0 = ldt<COHERENT>(src[j] + k), x1 = ldt<COHERENT>(src[j] + k + 2 * h);
       const fr y0 = ldt<COHERENT>(src[j] + k + h), y1 = ldt<COHERENT>(src[j] + k + 3 * h);
-      lo = fr_add(x0, fr_mulc(alpha, fr_sub_lazy(x1, x0)));
-      hi = fr_add(y0, fr_mulc(alpha, fr_sub_lazy(y1, y0)));
+      lo = fold_call(&alpha, x0, x1);
+      hi = fold_call(&alpha, y0, y1);
       st_fr(dst[j] + k, lo);
       st_fr(dst[j] + k + h, hi);
     }
