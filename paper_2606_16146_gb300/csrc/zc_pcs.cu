@@ -75,9 +75,9 @@ __global__ void k_pcs_sum_chunks(const fr* part, uint64_t count, uint32_t chunks
 struct PcsGatherArgs {
   const fr* enc[kMaxCols];
   const uint32_t* k;  // t queried positions
-  fr* out;            // [s][j][i]
+  fr* out;            // [s][j][i], the queries' columns pitch elements apart
   uint32_t c, t;
-  uint64_t m;
+  uint64_t m, pitch;
 };
 
 __global__ void k_pcs_gather(PcsGatherArgs A) {
@@ -85,7 +85,7 @@ __global__ void k_pcs_gather(PcsGatherArgs A) {
   const uint64_t per = (uint64_t)A.c * A.m;
   if (e >= per * A.t) return;
   const uint64_t s = e / per, r = e - s * per, j = r / A.m, i = r - j * A.m;
-  st_fr(A.out + e, ld_fr(A.enc[j] + (uint64_t)A.k[s] * A.m + i));
+  st_fr(A.out + s * A.pitch + r, ld_fr(A.enc[j] + (uint64_t)A.k[s] * A.m + i));
 }
 
 // ---------------------------------------------------------------- host --
@@ -350,7 +350,7 @@ zc_status zc_pcs_open(zc_pcs* P, const uint8_t (*alpha)[32], const uint8_t (*val
   // device buffers of the opening
   const size_t ncoef = std::max<uint64_t>(S.m, (uint64_t)S.c * S.m);
   const size_t bcoef = align_up(ncoef * sizeof(fr), 256), bu = align_up((S.c + 1) * S.w * sizeof(fr), 256);
-  const size_t bq = align_up(S.t * 4, 256), bg = align_up((size_t)S.t * S.c * S.m * sizeof(fr), 256);
+  const size_t bq = align_up(S.t * 4, 256), bg = align_up((size_t)S.t * (S.c * S.m + S.logW) * sizeof(fr), 256);
   // partial sums: chunks of kRows rows, enough CTAs to fill the GPU
   constexpr uint32_t kRows = 32;
   const uint32_t ch_u = (uint32_t)((S.m + kRows - 1) / kRows);
@@ -397,6 +397,11 @@ zc_status zc_pcs_open(zc_pcs* P, const uint8_t (*alpha)[32], const uint8_t (*val
   PCS_TRY(ctx, cudaMemcpyAsync(dcoef, co.data(), S.m * sizeof(fr), cudaMemcpyHostToDevice, st));
   k_pcs_combine<<<dim3((unsigned)((S.w + 255) / 256), S.c, ch_u), 256, 0, st>>>(ca);
   k_pcs_sum_chunks<<<(unsigned)((S.c * S.w + 255) / 256), 256, 0, st>>>(dpart, S.c * S.w, ch_u, du);
+  // Meanwhile the host touches the proof's pages: a copy to pages that the
+  // caller has not written yet takes its page faults one by one in the copy
+  // (n = 22, 50.8 MB: 52.6 ms an opening against 12.3; 19.3 through a buffer
+  // of its own).
+  for (size_t o = 20; o < need; o += 4096) proof[o] = 0;
   PCS_TRY(ctx, cudaMemcpyAsync(pp, du, (size_t)S.c * S.w * sizeof(fr), cudaMemcpyDeviceToHost, st));
   PCS_TRY(ctx, cudaStreamSynchronize(st));
   tr.absorb(pp, (size_t)S.c * S.w * 32);
@@ -428,11 +433,13 @@ zc_status zc_pcs_open(zc_pcs* P, const uint8_t (*alpha)[32], const uint8_t (*val
   ga.c = S.c;
   ga.t = S.t;
   ga.m = S.m;
+  ga.pitch = S.c * S.m + S.logW;
   const uint64_t tot = (uint64_t)S.t * S.c * S.m;
   k_pcs_gather<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(ga);
-  // the queried columns go straight to their places between the paths
-  const size_t per = (size_t)S.c * S.m * 32, pitch = per + 32 * (size_t)S.logW;
-  PCS_TRY(ctx, cudaMemcpy2DAsync(pp, pitch, dg, per, per, S.t, cudaMemcpyDeviceToHost, st));
+  // the columns leave at the proof's distances, in one copy straight to their
+  // places; the paths then fill the gaps
+  const size_t per = (size_t)S.c * S.m * 32;
+  PCS_TRY(ctx, cudaMemcpyAsync(pp, dg, (size_t)S.t * ga.pitch * sizeof(fr), cudaMemcpyDeviceToHost, st));
   PCS_TRY(ctx, cudaStreamSynchronize(st));
   for (uint32_t s2 = 0; s2 < S.t; s2++) {
     pp += per;
