@@ -192,7 +192,9 @@ zc_status zc_roots(zc_ctx* ctx, const zc_params* params, const void* const* cols
 /* Device-side timing of the last prove call on ctx, from CUDA events the
  * library records on the call's stream.  Writes min(cap, 10) values:
  * [0..5] phase times in ms.  SumCheck: roots, transcript r + eq tables,
- * round-1 evaluation kernel, rounds 2..n, final values + proof out.  NTT:
+ * round-1 evaluation kernel (Plonk proofs up to n = 16: also the further
+ * rounds of the cooperative launch that starts with round 1), rounds 2..n,
+ * final values + proof out.  NTT:
  * roots, INTT_H, slice LDE + gate + divide, q INTT, q root + z, openings +
  * proof out.  [6] time of the dominant kernel launch (ms), [7] its
  * algorithmic modular multiplications, [8] its algorithmic DRAM bytes,

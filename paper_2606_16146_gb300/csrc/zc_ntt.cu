@@ -19,10 +19,14 @@
 //   * The gate is pointwise, so qhat keeps that order, which is exactly the
 //     input order of N3 written as a three-digit reversed-input transform
 //     (slice digit outermost); N3's output, q, is natural.
-// Twiddles between passes come from two-level power tables of the 2^30-th
-// root of unity (w^e = HI[e >> 15] * LO[e & 32767]).  The coset factor
-// (7 w_M^j)^k / N of N2 is a two-level table per slice applied on load, with
-// the Montgomery conversion folded in (inputs are canonical, "level 0").
+// Every factor of a transform is a constant: the stages' twiddles, the
+// twiddles between passes, the coset factors (7 w_M^j)^k / N of N2 with the
+// conversion to Montgomery form in them (columns and coefficients are
+// canonical, "level 0") and the outer twiddles of N3 with 7^-k and the
+// conversion back come from tables of (w, floor(2^256 w / r)) pairs, per size
+// and in the lanes' order.  Sizes whose tables do not fit the cache use
+// two-level power tables of the 2^30-th root of unity
+// (w^e = HI[e >> 15] * LO[e & 32767]).
 #include <algorithm>
 #include <cstring>
 
@@ -502,7 +506,7 @@ __global__ void __launch_bounds__(256) k_ntt_cross(NttPassArgs A) {
 
 // ----------------------------------------------------- per-size tables --
 // For one (n, log2 s): the four-step twiddles of size N in both directions,
-// the coset factors (7 w_M^j)^k / N of every slice (level 2, which also
+// the coset factors (7 w_M^j)^k / N of every slice (times R, which also
 // converts canonical coefficients to Montgomery form), the outer twiddles of
 // the quotient INTT with its scale 7^-k, all as constant multipliers (frc).
 // The scale's other part, 7^-(N t) of the cross-slice stage's output t, is a
@@ -1339,21 +1343,19 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   const uint32_t nlo = 1u << hbits, nhi = 1u << (n - hbits);
   const uint32_t nblk_open = 2 * (uint32_t)ctx->sm_count;
   const bool q_direct = q_out && q_on_dev;
-  // several slices per launch take more scratch than the proof needs: used
-  // when the arena has it or may grow, never on lanes (captured, or a block of
-  // the serving pool) and within the memory budget
+  // several slices per launch take more scratch than the proof needs: as many
+  // as the arena has room for.  It is allocated larger only when it has to be
+  // allocated anyway, never moved for this (a captured graph may use it), nor
+  // on lanes and within the memory budget.
   const size_t need = ntt_scratch_bytes(p, ctx->sm_count, q_direct);
   const uint64_t Na = std::max<uint64_t>(N, 8);  // buffers of 256 bytes at least
   uint32_t sb = slices_per_launch(ctx->sm_count, c, N, s);
-  const size_t more = (size_t)(sb - 1) * c * Na * sizeof(fr);
-  if (ctx->arena.cap < need + more &&
-      (ctx->table_owner || ctx->arena_borrowed || (ctx->budget && need + more > ctx->budget) ||
-       ensure_arena(ctx, need + more) != ZC_OK)) {
+  auto more = [&] { return (size_t)(sb - 1) * c * Na * sizeof(fr); };
+  if (ctx->arena.cap < need && !ctx->table_owner && !ctx->arena_borrowed && ensure_arena(ctx, need + more()) != ZC_OK)
     ctx->err.clear();
-    sb = 1;
-  }
   zc_status s1 = ensure_arena(ctx, need);
   if (s1 != ZC_OK) return s1;
+  while (sb > 1 && ctx->arena.cap < need + more()) sb /= 2;
   Arena& ar = ctx->arena;
   ar.reset();
   fr* coef[kMaxCols];

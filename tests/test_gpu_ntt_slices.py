@@ -32,3 +32,17 @@ def test_slices_share_a_launch_or_not(gate, n, d, lb):
     for p, q in got:
         assert proof_bytes(p) == want_p
         assert np.asarray(q).tobytes() == want_q.tobytes()
+
+
+def test_slices_as_the_scratch_has_room():
+    """A context whose scratch, sized by another shape, holds two of the four slices."""
+    ctx = zc.Context(0, max_n=14, max_d=4)
+    try:
+        for gate, d in ((2, 4), (1, 3)):
+            cols = witness.generate(gate, 13, d, 9500 + d)
+            p, q = ctx.prove_ntt(gate, 13, d, to_device(cols))
+            want_p, want_q = oracle.prove_ntt(gate, 13, d, cols)
+            assert proof_bytes(p) == want_p
+            assert np.asarray(q).tobytes() == want_q.tobytes()
+    finally:
+        ctx.close()
