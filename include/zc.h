@@ -113,7 +113,12 @@ typedef struct {
 } zc_params;
 
 /* device: CUDA ordinal.  max_n / max_d: largest instance the context will
- * accept (scratch grows on demand up to mem_budget_bytes; 0 = no budget). */
+ * accept (scratch grows on demand up to mem_budget_bytes; 0 = no budget).
+ * The NTT form's factor tables are kept per size beside the scratch, up to 24
+ * GiB per context (the least recently used size goes first, never one that a
+ * batch graph reads); sizes without tables prove the same bytes more slowly.
+ * The environment variable ZC_NTT_TABLE_BYTES, if set when the context is set
+ * up, lowers that limit (for tests of the routes without tables). */
 typedef struct {
   int device;
   uint32_t max_n, max_d;
@@ -220,7 +225,8 @@ typedef struct zc_batch zc_batch;
 
 /* Allocate everything a batch needs, then capture its whole launch sequence
  * into one CUDA graph.  The graph keeps the given pointers: relaunching it
- * proves whatever the column buffers hold at launch time. */
+ * proves whatever the column buffers hold at launch time.  The factor tables
+ * it reads stay until zc_batch_destroy, whatever the context proves meanwhile. */
 zc_status zc_batch_create(zc_ctx* ctx, uint32_t count, const zc_form* forms, const zc_params* params,
                           const void* const* const* cols, uint8_t* const* proofs, void* const* q_outs,
                           zc_batch** out);

@@ -709,6 +709,8 @@ zc_status zc_setup(const zc_setup_opts* opts, zc_ctx** out) {
   ctx->budget = opts->mem_budget_bytes;
   const char* sp = std::getenv("ZC_SUMCHECK_DERIVED_POINT");
   ctx->skip_point = (sp && sp[0] == '0') ? 1 : 0;
+  const char* tb = std::getenv("ZC_NTT_TABLE_BYTES");
+  if (tb) ctx->ntt_cache_budget = std::min<size_t>(ctx->ntt_cache_budget, std::strtoull(tb, nullptr, 10));
   if (cudaSetDevice(ctx->device) != cudaSuccess) {
     delete ctx;
     return ZC_ERR_CUDA;
@@ -744,10 +746,7 @@ void zc_destroy(zc_ctx* ctx) {
   if (ctx->up_fork) cudaEventDestroy(ctx->up_fork);
   if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
   if (ctx->arena.base) cudaFree(ctx->arena.base);
-  for (auto& t : ctx->ntt_cache) {
-    if (t.mem) cudaFree(t.mem);
-    if (t.step_mem) cudaFree(t.step_mem);
-  }
+  ctx->ntt_cache.clear();
   if (ctx->dconst) cudaFree(ctx->dconst);
   if (ctx->dtabs) cudaFree(ctx->dtabs);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);

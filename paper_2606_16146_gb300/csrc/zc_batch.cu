@@ -101,8 +101,9 @@ static int lanes_for(const zc_ctx* ctx, uint32_t count) {
   return (int)std::min<uint32_t>(count, (uint32_t)want);
 }
 
+// holds: shares of the NTT tables the batch reads, to be kept as long as it may run.
 zc_status batch_prepare(zc_ctx* ctx, uint32_t count, const zc_form* forms, const zc_params* params,
-                        const bool* q_direct, cudaStream_t st) {
+                        const bool* q_direct, cudaStream_t st, NttHolds* holds) {
   for (uint32_t i = 0; i < count; i++) {
     zc_status s = check_params(ctx, &params[i], forms[i]);
     if (s != ZC_OK) return s;
@@ -119,7 +120,7 @@ zc_status batch_prepare(zc_ctx* ctx, uint32_t count, const zc_form* forms, const
                          : ntt_scratch_bytes(&params[i], ctx->sm_count, q_direct ? q_direct[i] : false);
     need[lane[i]] = std::max(need[lane[i]], b);
     if (forms[i] == ZC_FORM_NTT) {
-      s = ntt_prepare(ctx, &params[i], st);
+      s = ntt_prepare(ctx, &params[i], st, holds);
       if (s != ZC_OK) return s;
     }
   }
@@ -204,6 +205,7 @@ struct zc_batch {
   cudaStream_t capture = nullptr;
   uint32_t count = 0;
   uint32_t launches = 0;
+  zc::NttHolds holds;  // the tables its kernels read
 };
 
 using namespace zc;
@@ -236,7 +238,8 @@ zc_status zc_prove_batch(zc_ctx* ctx, uint32_t count, const zc_form* forms, cons
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   std::vector<char> qd(count, 0);
   for (uint32_t i = 0; i < count; i++) qd[i] = (q_outs && q_outs[i]) ? 1 : 0;
-  s = batch_prepare(ctx, count, forms, params, reinterpret_cast<const bool*>(qd.data()), st);
+  NttHolds holds;
+  s = batch_prepare(ctx, count, forms, params, reinterpret_cast<const bool*>(qd.data()), st, &holds);
   if (s != ZC_OK) return s;
   return batch_enqueue(ctx, count, forms, params, cols, st, proofs, q_outs);
 }
@@ -260,7 +263,7 @@ zc_status zc_batch_create(zc_ctx* ctx, uint32_t count, const zc_form* forms, con
   }
   std::vector<char> qd(count, 0);
   for (uint32_t i = 0; i < count; i++) qd[i] = (q_outs && q_outs[i]) ? 1 : 0;
-  s = batch_prepare(ctx, count, forms, params, reinterpret_cast<const bool*>(qd.data()), b->capture);
+  s = batch_prepare(ctx, count, forms, params, reinterpret_cast<const bool*>(qd.data()), b->capture, &b->holds);
   if (s == ZC_OK) {
     if (cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       s = ZC_ERR_CUDA;

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -141,9 +142,22 @@ struct zc_ctx {
   }
   // per-size NTT tables (twiddles, coset factors, quotient scale), built on
   // first use of a size; see zc_ntt.cu
+  struct NttTableMem {
+    void *mem = nullptr, *step_mem = nullptr;
+    NttTableMem() = default;
+    NttTableMem(const NttTableMem&) = delete;
+    NttTableMem& operator=(const NttTableMem&) = delete;
+    ~NttTableMem() {
+      if (mem) cudaFree(mem);
+      if (step_mem) cudaFree(step_mem);
+    }
+  };
   struct NttSizeTables {
     uint32_t n = 0, lb = 0, l1 = 0;
-    void* mem = nullptr;
+    // Shared with the batch graphs captured over these tables (a captured
+    // launch keeps their addresses): while anyone else holds it, the entry is
+    // not evicted.
+    std::shared_ptr<NttTableMem> own;
     size_t bytes = 0;
     uint64_t stamp = 0;
     zc::FrcTab tw_fwd, tw_inv, coset, outer;
@@ -154,8 +168,7 @@ struct zc_ctx {
     // sigma = 7 w_{2M}; constants: [0], [1] the small part's z_H inverse
     // times kappa^-1 N^-1 (frc), [2] 7^M (level 1), [8 + m] sigma^(mN) kappa^-1,
     // m < 2^lb (level 1), kappa = sigma^M - 7^M.
-    void* step_mem = nullptr;
-    size_t step_bytes = 0;
+    size_t step_bytes = 0;    // 0: not built
     zc::FrcTab step_coset;
     zc::fr *step_unscale = nullptr, *step_const = nullptr;
   };
@@ -256,8 +269,10 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
 // scratch bytes one proof needs (device columns, device roots computed)
 size_t sumcheck_scratch_bytes(const zc_ctx* ctx, const zc_params* p);
 size_t ntt_scratch_bytes(const zc_params* p, int sm_count, bool q_direct);
-// allocation-time set-up of the NTT form for one size (tables, attributes)
-zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st);
+// allocation-time set-up of the NTT form for one size (tables, attributes);
+// holds receives a share of the size's tables: they stay until it is dropped
+typedef std::vector<std::shared_ptr<void>> NttHolds;
+zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st, NttHolds* holds);
 // batch/serving lanes: child contexts with their own stream and scratch
 zc_status make_lanes(zc_ctx* ctx, int K);
 void destroy_lanes(zc_ctx* ctx);

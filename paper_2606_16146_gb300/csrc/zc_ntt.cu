@@ -1004,11 +1004,36 @@ static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int item
   return ZC_OK;
 }
 
+// Room for `bytes` more of tables within the context's budget: the least
+// recently used sizes go, but never one that a captured batch graph or a set
+// being prepared holds.  False when that leaves too little (must: what can go
+// goes, and the budget is passed by the rest).
+static bool table_room(zc_ctx* ctx, size_t bytes, bool must, cudaStream_t st) {
+  size_t used = 0, held = 0;
+  for (auto& e : ctx->ntt_cache) {
+    used += e.bytes + e.step_bytes;
+    if (e.own.use_count() > 1) held += e.bytes + e.step_bytes;
+  }
+  if (!must && held + bytes > ctx->ntt_cache_budget) return false;
+  while (used + bytes > ctx->ntt_cache_budget) {
+    size_t old = SIZE_MAX;
+    for (size_t i = 0; i < ctx->ntt_cache.size(); i++)
+      if (ctx->ntt_cache[i].own.use_count() == 1 &&
+          (old == SIZE_MAX || ctx->ntt_cache[i].stamp < ctx->ntt_cache[old].stamp))
+        old = i;
+    if (old == SIZE_MAX) break;
+    cudaStreamSynchronize(st);
+    used -= ctx->ntt_cache[old].bytes + ctx->ntt_cache[old].step_bytes;
+    ctx->ntt_cache.erase(ctx->ntt_cache.begin() + old);
+  }
+  return true;
+}
+
 // The per-size tables of (n, lb), built on first use; nullptr when they
 // would exceed the context's table budget (the passes then form every factor
 // from the two-level power tables instead).
 static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint32_t n, uint32_t lb,
-                                          uint32_t l1, uint32_t l2, cudaStream_t st) {
+                                          uint32_t l1, uint32_t l2, bool step, cudaStream_t st) {
   zc_ctx* ctx = user->table_owner ? user->table_owner : user;
   const uint64_t N = 1ull << n, M = N << lb;
   for (auto& e : ctx->ntt_cache)
@@ -1019,28 +1044,19 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
   const uint64_t s = 1ull << lb;
   const size_t bytes = sizeof(frc) * (2 * N + 2 * M + 2 * s);
   if (ctx->ntt_cache_frozen || bytes > ctx->ntt_cache_budget) return nullptr;
-  size_t used = 0;
-  for (auto& e : ctx->ntt_cache) used += e.bytes + e.step_bytes;
-  while (!ctx->ntt_cache.empty() && used + bytes > ctx->ntt_cache_budget) {
-    size_t old = 0;
-    for (size_t i = 1; i < ctx->ntt_cache.size(); i++)
-      if (ctx->ntt_cache[i].stamp < ctx->ntt_cache[old].stamp) old = i;
-    cudaStreamSynchronize(st);
-    cudaFree(ctx->ntt_cache[old].mem);
-    if (ctx->ntt_cache[old].step_mem) cudaFree(ctx->ntt_cache[old].step_mem);
-    used -= ctx->ntt_cache[old].bytes + ctx->ntt_cache[old].step_bytes;
-    ctx->ntt_cache.erase(ctx->ntt_cache.begin() + old);
-  }
+  if (!table_room(ctx, bytes, step, st)) return nullptr;  // a step-radix domain has no other route
   zc_ctx::NttSizeTables e;
-  if (cudaMalloc(&e.mem, bytes) != cudaSuccess) {
+  e.own = std::make_shared<zc_ctx::NttTableMem>();
+  if (cudaMalloc(&e.own->mem, bytes) != cudaSuccess) {
     cudaGetLastError();
+    e.own->mem = nullptr;
     return nullptr;
   }
   e.n = n;
   e.lb = lb;
   e.l1 = l1;
   e.bytes = bytes;
-  frc* q = static_cast<frc*>(e.mem);
+  frc* q = static_cast<frc*>(e.own->mem);
   e.tw_fwd = FrcTab::make(q, N); q += N;
   e.tw_inv = FrcTab::make(q, N); q += N;
   e.coset = FrcTab::make(q, M); q += M;
@@ -1067,7 +1083,6 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
     if (cudaMemcpyAsync(e.fin.p, hc.data(), sizeof(frc) * 2 * s, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
       cudaGetLastError();
-      cudaFree(e.mem);
       return nullptr;
     }
   }
@@ -1159,7 +1174,7 @@ static bool ntt_two_pass(const zc_ctx* ctx, uint32_t n) {
 // The step-radix tables of a cache entry (lb = k): built once, with the
 // host-computed constants of the small part.  False if they cannot be made.
 static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables* T, cudaStream_t st) {
-  if (e->step_mem) return true;
+  if (e->step_bytes) return true;
   zc_ctx* ctx = user->table_owner ? user->table_owner : user;
   if (ctx->ntt_cache_frozen) return false;
   const uint32_t n = e->n, lb = e->lb;
@@ -1214,7 +1229,7 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables*
     cudaFree(mem);
     return false;
   }
-  e->step_mem = mem;
+  e->own->step_mem = mem;
   e->step_bytes = bytes;
   e->step_coset = coset;
   e->step_unscale = unscale;
@@ -1284,7 +1299,7 @@ zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uin
   return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
 }
 
-zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st) {
+zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st, NttHolds* holds) {
   ensure_pass_attributes(ctx->device);
   NttTables* T = nullptr;
   zc_status s0 = ensure_tables(ctx, st, &T);
@@ -1292,7 +1307,8 @@ zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st) {
   const NttDomain D = domain_of(p);
   const uint32_t n = p->n, lb = D.k;
   const bool two = ntt_two_pass(ctx, n);
-  zc_ctx::NttSizeTables* ST = size_tables(ctx, T, n, lb, two ? (n + 1) / 2 : n, two ? n / 2 : 0, st);
+  zc_ctx::NttSizeTables* ST = size_tables(ctx, T, n, lb, two ? (n + 1) / 2 : n, two ? n / 2 : 0, D.step, st);
+  if (ST) holds->push_back(ST->own);
   if (D.step && (!ST || !step_tables(ctx, ST, T, st))) {
     ctx->err = "step-radix domain: tables unavailable";
     return ZC_ERR_OOM;
@@ -1387,7 +1403,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   const uint32_t l2 = two ? n / 2 : 0;         // second digit
   const uint64_t L1 = 1ull << l1, L2 = 1ull << l2;
   zc_status rs;
-  zc_ctx::NttSizeTables* ST = size_tables(ctx, T, n, lb, l1, l2, st);
+  zc_ctx::NttSizeTables* ST = size_tables(ctx, T, n, lb, l1, l2, D.step, st);
   if (D.step && (!ST || !step_tables(ctx, ST, T, st))) {
     ctx->err = "step-radix domain: per-size tables unavailable";
     return ZC_ERR_OOM;

@@ -150,9 +150,10 @@ zc_status zc_serve(zc_ctx* ctx, const zc_request* reqs, uint32_t count, const zc
     L->arena_borrowed = true;
   }
   cudaStream_t prep = ctx->lane_streams[0];
+  NttHolds holds;  // no request's tables go to make room for another's
   for (uint32_t i = 0; i < count; i++) {
     if (reqs[i].form != ZC_FORM_NTT || fp[i] > budget) continue;
-    s = ntt_prepare(ctx, &reqs[i].params, prep);
+    s = ntt_prepare(ctx, &reqs[i].params, prep, &holds);
     if (s != ZC_OK) {
       release_lane_arenas(ctx);
       return s;
