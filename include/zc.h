@@ -114,7 +114,7 @@ typedef struct {
 
 /* device: CUDA ordinal.  max_n / max_d: largest instance the context will
  * accept (scratch grows on demand up to mem_budget_bytes; 0 = no budget).
- * The NTT form's factor tables are kept per size beside the scratch, up to 24
+ * The NTT form's factor tables are kept per size beside the scratch, up to 32
  * GiB per context (the least recently used size goes first, never one that a
  * batch graph reads); sizes without tables prove the same bytes more slowly.
  * The environment variable ZC_NTT_TABLE_BYTES, if set when the context is set

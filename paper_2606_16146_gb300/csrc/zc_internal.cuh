@@ -174,8 +174,10 @@ struct zc_ctx {
   };
   std::vector<NttSizeTables> ntt_cache;
   uint64_t ntt_cache_clock = 0;
-  // 24 GiB holds every size that 16 GiB of 32-byte entries did
-  size_t ntt_cache_budget = 24ull << 30;
+  // A size takes 64 (2 N + 2 M + 2 s) bytes (M = s N; Plonk n = 22 2.7 GB, n =
+  // 24 10.7 GB), at most twice the 32 (2 N + 3 M + s) of 32-byte entries, so 32
+  // GiB hold every set of sizes that 16 GiB of those held.
+  size_t ntt_cache_budget = 32ull << 30;
   // While a prepared batch is being enqueued (possibly under graph capture)
   // the cache neither allocates nor evicts; a missing size falls back to the
   // two-level power tables.

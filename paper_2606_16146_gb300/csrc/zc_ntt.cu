@@ -1171,17 +1171,25 @@ static bool ntt_two_pass(const zc_ctx* ctx, uint32_t n) {
   return n >= (uint32_t)(t > 0 ? t : 12) && n >= 2;
 }
 
+// coset factors (frc), unscale factors, 8 + 2^lb constants
+static size_t step_table_bytes(uint32_t n, uint32_t lb) { return sizeof(fr) * ((3ull << n) + 8 + (1ull << lb)); }
+
 // The step-radix tables of a cache entry (lb = k): built once, with the
 // host-computed constants of the small part.  False if they cannot be made.
-static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables* e, const NttTables* T, cudaStream_t st) {
+static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables*& e, const NttTables* T, cudaStream_t st) {
   if (e->step_bytes) return true;
   zc_ctx* ctx = user->table_owner ? user->table_owner : user;
   if (ctx->ntt_cache_frozen) return false;
+  // room for them too, with this entry held; e moves as others go
+  const std::shared_ptr<zc_ctx::NttTableMem> own = e->own;
+  table_room(ctx, step_table_bytes(e->n, e->lb), true, st);
+  for (auto& t : ctx->ntt_cache)
+    if (t.own == own) e = &t;
   const uint32_t n = e->n, lb = e->lb;
   const uint64_t N = 1ull << n, M = N << lb, parts = 1ull << lb;
   if (n + lb + 1 > (uint32_t)kLog30 || parts > 64) return false;
   const size_t nconst = 8 + parts;
-  const size_t bytes = sizeof(fr) * (3 * N + nconst);
+  const size_t bytes = step_table_bytes(n, lb);
   void* mem = nullptr;
   if (cudaMalloc(&mem, bytes) != cudaSuccess) {
     cudaGetLastError();

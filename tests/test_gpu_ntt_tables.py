@@ -103,3 +103,40 @@ def test_prepared_sets_past_the_limit(monkeypatch, shapes):
             prove(ctx, x)
     finally:
         ctx.close()
+
+
+def test_step_tables_count(monkeypatch):
+    """The step-radix part of a size makes room for itself as the size does."""
+    a, b = instance(1, 7, 3, 2, 9630), instance(1, 8, 3, 0x101, 9631)
+    ctx = ctx_with(monkeypatch, table_bytes(7, 2) + table_bytes(8, 1))
+    try:
+        first = prove(ctx, a)
+        assert prove(ctx, a) < first  # its tables are there
+        prove(ctx, b)
+        assert prove(ctx, a) == first  # they went for b's
+        prove(ctx, b)
+    finally:
+        ctx.close()
+
+
+def test_default_limit_holds_three_large_sizes():
+    """25 GiB of tables in one prepared set (12.5 GiB with 32-byte entries), none without them."""
+    import torch
+    shapes = [(witness.gate_sum(0), 24, 2, 1), (witness.gate_sum(0), 24, 3, 2), (witness.gate_sum(0), 23, 2, 3)]
+    assert sum(table_bytes(n, lb) for _, n, _, lb in shapes) > 24 << 30
+    cols = [torch.empty(32 << 24, dtype=torch.uint8, device="cuda") for _ in range(3)]  # captured, never launched
+    proofs = [torch.empty(zc.proof_size(g, n, d, zc.ZC_FORM_NTT), dtype=torch.uint8, device="cuda")
+              for g, n, d, _ in shapes]
+
+    def kernels(idx):
+        ctx = zc.Context(0, max_n=24, max_d=4)
+        try:
+            g = ctx.batch_graph([zc.ZC_FORM_NTT] * len(idx), [shapes[i] for i in idx],
+                                [cols[:shapes[i][2]] for i in idx], [proofs[i] for i in idx], None)
+            k = g.kernels
+            g.close()
+            return k
+        finally:
+            ctx.close()
+
+    assert kernels([0, 1, 2]) == sum(kernels([i]) for i in range(3))
