@@ -226,7 +226,8 @@ typedef struct zc_batch zc_batch;
 /* Allocate everything a batch needs, then capture its whole launch sequence
  * into one CUDA graph.  The graph keeps the given pointers: relaunching it
  * proves whatever the column buffers hold at launch time.  The factor tables
- * it reads stay until zc_batch_destroy, whatever the context proves meanwhile. */
+ * it reads and its scratch stay until zc_batch_destroy, whatever the context
+ * proves meanwhile. */
 zc_status zc_batch_create(zc_ctx* ctx, uint32_t count, const zc_form* forms, const zc_params* params,
                           const void* const* const* cols, uint8_t* const* proofs, void* const* q_outs,
                           zc_batch** out);

@@ -83,7 +83,7 @@ zc_status ensure_arena(zc_ctx* ctx, size_t bytes) {
   }
   if (ctx->arena.base) {
     cudaDeviceSynchronize();
-    cudaFree(ctx->arena.base);
+    ctx->arena_own.reset();
     ctx->arena.base = nullptr;
     ctx->arena.cap = 0;
   }
@@ -95,6 +95,7 @@ zc_status ensure_arena(zc_ctx* ctx, size_t bytes) {
     ctx->err = std::string("cudaMalloc scratch: ") + cudaGetErrorString(e);
     return ZC_ERR_OOM;
   }
+  ctx->arena_own = std::shared_ptr<void>(p, [](void* q) { cudaFree(q); });
   ctx->arena.base = static_cast<char*>(p);
   ctx->arena.cap = want;
   ctx->arena.used = 0;
@@ -745,7 +746,7 @@ void zc_destroy(zc_ctx* ctx) {
   for (cudaEvent_t e : ctx->up_ev) cudaEventDestroy(e);
   if (ctx->up_fork) cudaEventDestroy(ctx->up_fork);
   if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
-  if (ctx->arena.base) cudaFree(ctx->arena.base);
+  ctx->arena_own.reset();
   ctx->ntt_cache.clear();
   if (ctx->dconst) cudaFree(ctx->dconst);
   if (ctx->dtabs) cudaFree(ctx->dtabs);

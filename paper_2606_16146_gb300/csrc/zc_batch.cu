@@ -101,9 +101,9 @@ static int lanes_for(const zc_ctx* ctx, uint32_t count) {
   return (int)std::min<uint32_t>(count, (uint32_t)want);
 }
 
-// holds: shares of the NTT tables the batch reads, to be kept as long as it may run.
+// holds: shares of the NTT tables and the lane scratch the batch uses, to be kept as long as it may run.
 zc_status batch_prepare(zc_ctx* ctx, uint32_t count, const zc_form* forms, const zc_params* params,
-                        const bool* q_direct, cudaStream_t st, NttHolds* holds) {
+                        const bool* q_direct, cudaStream_t st, Holds* holds) {
   for (uint32_t i = 0; i < count; i++) {
     zc_status s = check_params(ctx, &params[i], forms[i]);
     if (s != ZC_OK) return s;
@@ -130,6 +130,7 @@ zc_status batch_prepare(zc_ctx* ctx, uint32_t count, const zc_form* forms, const
       ctx->err = ctx->lanes[k]->err;
       return s;
     }
+    holds->push_back(ctx->lanes[k]->arena_own);
   }
   return cudaDeviceSynchronize() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
 }
@@ -181,7 +182,6 @@ zc_status batch_enqueue(zc_ctx* ctx, uint32_t count, const zc_form* forms, const
 void destroy_lanes(zc_ctx* ctx) {
   for (size_t k = 0; k < ctx->lanes.size(); k++) {
     zc_ctx* L = ctx->lanes[k];
-    if (L->arena.base && !L->arena_borrowed) cudaFree(L->arena.base);
     if (L->pinned) cudaFreeHost(L->pinned);
     for (int i = 0; i < 8; i++)
       if (L->ev[i]) cudaEventDestroy(L->ev[i]);
@@ -205,7 +205,7 @@ struct zc_batch {
   cudaStream_t capture = nullptr;
   uint32_t count = 0;
   uint32_t launches = 0;
-  zc::NttHolds holds;  // the tables its kernels read
+  zc::Holds holds;  // the tables and the scratch its kernels use
 };
 
 using namespace zc;
@@ -238,7 +238,7 @@ zc_status zc_prove_batch(zc_ctx* ctx, uint32_t count, const zc_form* forms, cons
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   std::vector<char> qd(count, 0);
   for (uint32_t i = 0; i < count; i++) qd[i] = (q_outs && q_outs[i]) ? 1 : 0;
-  NttHolds holds;
+  Holds holds;
   s = batch_prepare(ctx, count, forms, params, reinterpret_cast<const bool*>(qd.data()), st, &holds);
   if (s != ZC_OK) return s;
   return batch_enqueue(ctx, count, forms, params, cols, st, proofs, q_outs);

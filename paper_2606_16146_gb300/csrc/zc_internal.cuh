@@ -120,6 +120,7 @@ struct zc_ctx {
   zc::fr* dtabs = nullptr;        // per-degree tables (device)
   std::vector<zc::fr> htabs;      // host copy
   zc::Arena arena;               // per-call scratch
+  std::shared_ptr<void> arena_own;  // its memory, unless borrowed; batch graphs hold shares of their lanes'
   bool arena_borrowed = false;   // arena is a block of the serving pool (not freed here)
   void* pinned = nullptr;        // small pinned staging buffer
   size_t pinned_cap = 0;
@@ -200,6 +201,9 @@ struct zc_ctx {
 
 namespace zc {
 
+// shares of device memory that captured launches use (tables, lane arenas)
+typedef std::vector<std::shared_ptr<void>> Holds;
+
 // status helpers
 #define ZC_CUDA_TRY(ctx, call)                                                       \
   do {                                                                               \
@@ -273,8 +277,7 @@ size_t sumcheck_scratch_bytes(const zc_ctx* ctx, const zc_params* p);
 size_t ntt_scratch_bytes(const zc_params* p, int sm_count, bool q_direct);
 // allocation-time set-up of the NTT form for one size (tables, attributes);
 // holds receives a share of the size's tables: they stay until it is dropped
-typedef std::vector<std::shared_ptr<void>> NttHolds;
-zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st, NttHolds* holds);
+zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st, Holds* holds);
 // batch/serving lanes: child contexts with their own stream and scratch
 zc_status make_lanes(zc_ctx* ctx, int K);
 void destroy_lanes(zc_ctx* ctx);

@@ -1307,7 +1307,7 @@ zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uin
   return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
 }
 
-zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st, NttHolds* holds) {
+zc_status ntt_prepare(zc_ctx* ctx, const zc_params* p, cudaStream_t st, Holds* holds) {
   ensure_pass_attributes(ctx->device);
   NttTables* T = nullptr;
   zc_status s0 = ensure_tables(ctx, st, &T);

@@ -144,13 +144,13 @@ zc_status zc_serve(zc_ctx* ctx, const zc_request* reqs, uint32_t count, const zc
   for (int k = 0; k < K; k++) {
     zc_ctx* L = ctx->lanes[k];
     std::memcpy(L->tune, ctx->tune, sizeof(ctx->tune));
-    if (L->arena.base && !L->arena_borrowed) cudaFree(L->arena.base);
+    L->arena_own.reset();
     L->arena.base = nullptr;
     L->arena.cap = 0;
     L->arena_borrowed = true;
   }
   cudaStream_t prep = ctx->lane_streams[0];
-  NttHolds holds;  // no request's tables go to make room for another's
+  Holds holds;  // no request's tables go to make room for another's
   for (uint32_t i = 0; i < count; i++) {
     if (reqs[i].form != ZC_FORM_NTT || fp[i] > budget) continue;
     s = ntt_prepare(ctx, &reqs[i].params, prep, &holds);
