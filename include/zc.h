@@ -448,8 +448,11 @@ zc_status zc_serve(zc_ctx* ctx, const zc_request* reqs, uint32_t count, const zc
  *                        1..24, default 16.
  *   ZC_TUNE_BATCH_LANES  batches: concurrent lanes (streams); set with n = 0
  *                        under either form; 1..64, default 16.
- *   ZC_TUNE_NTT_TILE_LOG NTT: elements per shared-memory pass tile, 2^value;
- *                        10, 11 or 12, default 11.
+ *   ZC_TUNE_NTT_TILE_LOG NTT: elements per shared-memory pass tile, 2^value,
+ *                        at least the sub-transform's; 10, 11 or 12, default
+ *                        10.  With neither this key nor ZC_TUNE_NTT_MINB set,
+ *                        launches of at most 2^19 elements take a kernel of
+ *                        smaller tiles; either key gives it up.
  *   ZC_TUNE_NTT_TWO_LOG  NTT: sizes 2^n with n >= value run each transform as
  *                        two four-step passes (more, smaller CTAs), smaller
  *                        ones as one pass (always two above n = 12); 2..24,

@@ -968,9 +968,12 @@ static void set_dft(NttPassArgs& a, const NttTables* T, bool inverse) {
 // launch one batched pass over `items` columns
 static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int items, uint64_t B, uint32_t slices = 1) {
   const uint32_t logL = a.logL;
-  // few elements: two per thread, tiles of 256 (or one sub-DFT)
-  if (logL >= 1 && logL <= 10 && (uint64_t)items * slices * (B << logL) <= kSmallElems && a.pre != PRE_COSET &&
-      (a.post == POST_NONE || a.post == POST_TAB)) {
+  uint32_t logTile = (uint32_t)ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_TILE_LOG);
+  const int minb = ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_MINB);
+  // few elements, and no tile or residency asked for: two per thread, tiles of
+  // 256 (or one sub-DFT)
+  if (!logTile && !minb && logL >= 1 && logL <= 10 && (uint64_t)items * slices * (B << logL) <= kSmallElems &&
+      a.pre != PRE_COSET && (a.post == POST_NONE || a.post == POST_TAB)) {
     const uint32_t lt = std::max<uint32_t>(logL, 8);
     if ((B << logL) % (1ull << lt) == 0) {
       a.logW = lt - logL;
@@ -982,8 +985,6 @@ static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int item
       return ZC_OK;
     }
   }
-  uint32_t logTile = (uint32_t)ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_TILE_LOG);
-  const int minb = ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_MINB);
   if (logTile < logL) logTile = logL < 10 ? 10 : logL;
   if (logTile > 12) logTile = 12;
   if (logTile < 10) logTile = 10;
