@@ -31,6 +31,7 @@
 #include <cstring>
 
 #include "zc_internal.cuh"
+#include "zc_ntt_index.cuh"
 #include "zc_transcript.cuh"
 
 namespace zc {
@@ -39,6 +40,7 @@ constexpr int kLog30 = 30;
 constexpr uint32_t kLoBits = 15;
 constexpr uint32_t kLoMask = (1u << kLoBits) - 1;
 constexpr int kMaxNttN = 24;
+static_assert((uint64_t)kMaxCols << kMaxNttN < 1ull << 32, "slice strides are 32-bit");
 
 struct NttTables {
   bool ready = false;
@@ -58,15 +60,6 @@ struct NttTables {
 
 static NttTables g_tabs_by_dev[64];
 static std::mutex g_tabs_mu;
-
-// Twiddles of the radix-R stage at stride Ns = 8, 64 or 512: w_{Ns R}^{r k},
-// 1 <= r < R, k < Ns, at stage_tab + (r - 1) Ns + k, so that consecutive k are
-// consecutive entries.
-constexpr uint32_t kStageTab = 11 * (8 + 64 + 512);
-__host__ __device__ __forceinline__ uint32_t stage_tab(uint32_t logNs, uint32_t lr) {
-  const uint32_t Ns = 1u << logNs;
-  return 11 * ((Ns - 8) / 7) + (lr == 3 ? 0 : lr == 2 ? 7 * Ns : 10 * Ns);
-}
 
 struct NttTabArgs {
   FrcTab dft_fwd, dft_inv; fr* wf_lo; fr* wf_hi; fr* wi_lo; fr* wi_hi; fr* s7_lo; fr* s7_hi;
@@ -119,26 +112,6 @@ __device__ __forceinline__ fr root_pow(const fr* lo, const fr* hi, uint32_t e) {
 enum { PRE_NONE = 0, PRE_COSET = 1, PRE_TAB = 2 };
 enum { POST_NONE = 0, POST_TW = 1, POST_OUTER = 2, POST_FINAL = 3, POST_TAB = 4 };
 
-// Index of element t of sub-DFT b in a column or a factor table; every stride
-// is a power of two: ((b >> div) << hs) + ((b & mask) << ls) + (t << ts).
-struct NttMap {
-  uint32_t div, hs, mask, ls, ts;
-  __device__ __forceinline__ uint32_t at(uint32_t b, uint32_t t) const {
-    return ((b >> div) << hs) + ((b & mask) << ls) + (t << ts);
-  }
-};
-constexpr uint32_t kNone = 31;  // a shift that leaves nothing of b < 2^31
-// b << ls, t << ts
-static NttMap map_flat(uint32_t ls, uint32_t ts) { return NttMap{kNone, 0, 0xffffffffu, ls, ts}; }
-// (b >> div) << hs, (b mod 2^div) << ls, t << ts
-static NttMap map_split(uint32_t div, uint32_t hs, uint32_t ls, uint32_t ts) {
-  return NttMap{div, hs, (1u << div) - 1, ls, ts};
-}
-// the low div bits of b only
-static NttMap map_low(uint32_t div, uint32_t ls, uint32_t ts) {
-  return NttMap{kNone, 0, (1u << div) - 1, ls, ts};
-}
-
 struct NttPassArgs {
   const fr* in[kMaxCols];
   fr* out[kMaxCols];
@@ -167,6 +140,7 @@ struct NttPassArgs {
   uint32_t outer_lbdiv;   // POST_OUTER: e = (b >> lbdiv) * ((t << lbdiv) + (b mod 2^lbdiv))
   uint32_t fin_logN;      // POST_FINAL: k = (t << fin_logN) + b
   uint32_t* err;          // if set: the pass reads the proof's input columns, and a value >= r sets bit 0
+  void use(const NttMaps& m) { logL = m.logL; im = m.im; om = m.om; pm = m.pm; qm = m.qm; }
 };
 
 // radix-2/4/8 butterflies on x[0..R) in registers, X[k] = sum_r x[r] w_R^(rk).
@@ -215,8 +189,7 @@ __device__ __forceinline__ void dft8(fr (&x)[8], const NttPassArgs& A) {
 struct SmTile {
   uint4* p;     // plane 0: p[0, T), plane 1: p[T, 2T)
   uint32_t T;
-  __device__ __forceinline__ uint32_t sw(uint32_t i) const { return i ^ ((i >> 3) & 7); }
-  __device__ __forceinline__ fr get(uint32_t i) const { return get_at(sw(i)); }
+  __device__ __forceinline__ fr get(uint32_t i) const { return get_at(tile_slot(i)); }
   __device__ __forceinline__ fr get_at(uint32_t s) const {
     const uint4 a = p[s], b = p[T + s];
     fr x;
@@ -225,7 +198,7 @@ struct SmTile {
     return x;
   }
   __device__ __forceinline__ void put(uint32_t i, const fr& x) const {
-    const uint32_t s = sw(i);
+    const uint32_t s = tile_slot(i);
     p[s] = make_uint4(x.v[0], x.v[1], x.v[2], x.v[3]);
     p[T + s] = make_uint4(x.v[4], x.v[5], x.v[6], x.v[7]);
   }
@@ -263,17 +236,9 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   // items (columns) vary fastest across consecutive CTAs, so the per-element
   // factor tables, shared by every column, are reused from L2
   const uint32_t item = blockIdx.x % A.items;
-  const uint32_t logL = A.logL, logW = A.logW, Wm = (1u << logW) - 1, tq = (1u << logL) >> 3;
+  const uint32_t logL = A.logL, logW = A.logW;
   const uint32_t b0 = (blockIdx.x / A.items) << logW;
-  // the sub-DFT and the element of tile element i
-  auto sub = [&](uint32_t i) { return FAST ? b0 + (i & Wm) : min(b0 + (i & Wm), A.B - 1); };
-  auto elt = [&](uint32_t i) { return i >> logW; };
-  // index of tile element i, and from i0 to i0 + NT p (FAST: p tq elements
-  // further on; otherwise it may go back)
-  auto index = [&](const NttMap& m, uint32_t i) { return m.at(sub(i), elt(i)); };
-  auto step = [&](const NttMap& m, uint32_t i0, int p) -> ptrdiff_t {
-    return FAST ? (ptrdiff_t)(p * (tq << m.ts)) : (ptrdiff_t)index(m, i0 + NT * p) - (ptrdiff_t)index(m, i0);
-  };
+  const NttTile<FAST> X(logL, logW, b0, A.B, NT, tid);
   // The column's elements come through shared memory in 16-byte halves, two
   // lanes to an element; a warp copies its own slots only.
   {
@@ -281,21 +246,19 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
     const char* in = reinterpret_cast<const char*>(A.in[item] + (size_t)A.in_y * blockIdx.y) + 16 * half;
 #pragma unroll
     for (int s = 0; s < 2; s++) {
-      const uint32_t i = (tid & ~31u) + ((tid & 31) >> 1) + 16 * s;
-      const char* g = in + sizeof(fr) * (size_t)index(A.im, i);
+      const uint32_t i = X.copy_elt(s);
+      const char* g = in + sizeof(fr) * (size_t)X.index(A.im, i);
 #pragma unroll
       for (int p = 0; p < 8; p++) {
-        const uint32_t sl = FAST ? sm.sw(i) + NT * p : sm.sw(i + NT * p);
-        const uint32_t d = (uint32_t)__cvta_generic_to_shared(sm.p + sm.T * half + sl);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(g + (ptrdiff_t)sizeof(fr) * step(A.im, i, p))
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(sm.p + sm.T * half + X.slot(i, p));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(g + (ptrdiff_t)sizeof(fr) * X.step(A.im, i, p))
                      : "memory");
       }
     }
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncwarp();
   }
-  // slot p of this thread (NT is a multiple of 64 in the FAST form: the swizzle of slot 0 serves all)
-  auto get = [&](int p) { return FAST ? sm.get_at(sm.sw(tid) + NT * p) : sm.get(tid + NT * p); };
+  auto get = [&](int p) { return sm.get_at(X.slot(tid, p)); };
   fr x[8];
 #pragma unroll
   for (int p = 0; p < 8; p++) x[p] = get(p);
@@ -308,7 +271,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   if (!FAST && A.pre == PRE_COSET) {
 #pragma unroll
     for (int p = 0; p < 8; p++) {
-      const uint32_t k = index(A.pm, tid + NT * p);
+      const uint32_t k = X.index(A.pm, tid + NT * p);
       // one slice per launch: every column uses the same tables
       x[p] = fr_mul(fr_mul(ld_fr(A.pre_hi + (k >> A.pre_shift)), ld_fr(A.pre_lo + (k & ((1u << A.pre_shift) - 1)))),
                     x[p]);
@@ -319,24 +282,18 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   bool fin = false;  // the step after the last stage: the post table
 #pragma unroll 1
   while (true) {
-    const uint32_t lr = min(3u, logL - logNs), lg = 3 - lr;  // radix R, and the 8 / R groups, as logs
+    const uint32_t lr = min(3u, logL - logNs);  // radix R as a log
     // factors: pre or post table, or the twiddles w_{Ns R}^{r k}, r = p >> lg
     // (for r = 0 the previous stage's lazy output is only reduced)
     const bool tw = !fin && logNs > 0, all = fin || (logNs == 0 && A.pre == PRE_TAB);
     if (tw || all) {
       const FrcTab base = tw ? A.dft : fin ? A.post_tab : A.pre_tab;
       const NttMap m = fin ? A.qm : A.pm;
-      // group g's sub-DFT element is j + g tq; only a last stage has several
-      // groups, and there k = j
-      const uint32_t j = elt(tid), km = (1u << logNs) - 1;
-      const FrcTab first = base.at(tw ? (ptrdiff_t)(stage_tab(logNs, lr) + (FAST ? j & km : 0)) - (ptrdiff_t)(km + 1)
-                                     : (ptrdiff_t)index(m, tid) + (fin ? 0 : (ptrdiff_t)A.pre_y * blockIdx.y));
+      const FrcTab first = base.at(tw ? X.tw_first(logNs, lr)
+                                     : (ptrdiff_t)X.index(m, tid) + (fin ? 0 : (ptrdiff_t)A.pre_y * blockIdx.y));
+      // one load for both kinds (a load in each branch: n = 20 7.72 to 7.84 ms, this 7.61)
       auto fac = [&](int p) {
-        if (tw) {
-          const uint32_t g = p & ((1u << lg) - 1), r = (uint32_t)p >> lg;
-          return first.ld((r << logNs) + (FAST ? g * tq : elt(tid + NT * g) & km));
-        }
-        return first.ld(step(m, tid, p));
+        return first.ld(tw ? (ptrdiff_t)X.tw_step(logNs, lr, p) : X.step(m, tid, p));
       };
 #pragma unroll
       for (int p = 7; p >= 4; p--) x[p] = fr_mulc(fac(p), x[p]);
@@ -371,14 +328,9 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
       fin = true;
       continue;
     }
-    // element (j, r) of the stage goes to (j / Ns) Ns R + j mod Ns + r Ns
-    const uint32_t ls = logNs + logW;
     __syncthreads();  // every slot has been read
 #pragma unroll
-    for (int p = 0; p < 8; p++) {
-      const uint32_t ja = tid + NT * (p & ((1u << lg) - 1)), r = (uint32_t)p >> lg;
-      sm.put(((ja >> ls) << (ls + lr)) + (ja & ((1u << ls) - 1)) + (r << ls), x[p]);
-    }
+    for (int p = 0; p < 8; p++) sm.put(X.exchange(logNs, lr, p), x[p]);
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < 8; p++) x[p] = get(p);
@@ -390,13 +342,13 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
   // Without a post table the values are lazy: reduced, or multiplied here.
   const bool odd = tid & 1;
   char* const out = reinterpret_cast<char*>(A.out[item] + (size_t)A.out_y * blockIdx.y) + 16 * odd;
-  char* const oe = out + sizeof(fr) * (size_t)index(A.om, tid & ~1u);  // the even lane's element
-  char* const oo = out + sizeof(fr) * (size_t)index(A.om, tid | 1u);
+  char* const oe = out + sizeof(fr) * (size_t)X.index(A.om, tid & ~1u);  // the even lane's element
+  char* const oo = out + sizeof(fr) * (size_t)X.index(A.om, tid | 1u);
 #pragma unroll
   for (int p = 0; p < 8; p++) {
     fr y = x[p];
     if (!post_tab) {
-      const uint32_t b = sub(tid + NT * p), t = elt(tid + NT * p);
+      const uint32_t b = X.sub(tid + NT * p), t = X.elt(tid + NT * p);
       if (FAST || A.post == POST_NONE) {
         y = fr_reduce1(y);
       } else if (A.post == POST_FINAL) {
@@ -413,12 +365,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_ntt_pass(NttPassArgs A) {
     uint32_t r[4];
 #pragma unroll
     for (int h = 0; h < 4; h++) r[h] = __shfl_xor_sync(0xffffffffu, odd ? y.v[h] : y.v[4 + h], 1);
-    const bool le = FAST || b0 + (((tid & ~1u) + NT * p) & Wm) < A.B, lo = FAST || b0 + (((tid | 1u) + NT * p) & Wm) < A.B;
-    if (le)
-      *reinterpret_cast<uint4*>(oe + (ptrdiff_t)sizeof(fr) * step(A.om, tid & ~1u, p)) =
+    if (X.stored((tid & ~1u) + NT * p))
+      *reinterpret_cast<uint4*>(oe + (ptrdiff_t)sizeof(fr) * X.step(A.om, tid & ~1u, p)) =
           odd ? make_uint4(r[0], r[1], r[2], r[3]) : make_uint4(y.v[0], y.v[1], y.v[2], y.v[3]);
-    if (lo)
-      *reinterpret_cast<uint4*>(oo + (ptrdiff_t)sizeof(fr) * step(A.om, tid | 1u, p)) =
+    if (X.stored((tid | 1u) + NT * p))
+      *reinterpret_cast<uint4*>(oo + (ptrdiff_t)sizeof(fr) * X.step(A.om, tid | 1u, p)) =
           odd ? make_uint4(y.v[4], y.v[5], y.v[6], y.v[7]) : make_uint4(r[0], r[1], r[2], r[3]);
   }
 }
@@ -433,9 +384,9 @@ __global__ void __launch_bounds__(512) k_ntt_pass_small(NttPassArgs A) {
   extern __shared__ __align__(16) uint4 sm_planes[];
   const uint32_t NT = blockDim.x, tid = threadIdx.x;
   const uint32_t item = blockIdx.x % A.items;
-  const uint32_t logL = A.logL, logW = A.logW, Wm = (1u << logW) - 1;
-  const uint32_t b = ((blockIdx.x / A.items) << logW) + (tid & Wm);  // NT is a multiple of W
-  const uint32_t t0 = tid >> logW, t1 = (tid + NT) >> logW;
+  const uint32_t logL = A.logL;
+  const NttSmallTile X{logL, A.logW, (blockIdx.x / A.items) << A.logW, NT, tid};
+  const uint32_t b = X.sub(), t0 = X.elt(0), t1 = X.elt(1);
   const fr* in = A.in[item] + (size_t)A.in_y * blockIdx.y;
   fr x0 = ld_fr(in + A.im.at(b, t0)), x1 = ld_fr(in + A.im.at(b, t1));
   if (A.err && !(fr_is_canonical(x0) && fr_is_canonical(x1))) atomicOr(A.err, 1u);
@@ -446,10 +397,8 @@ __global__ void __launch_bounds__(512) k_ntt_pass_small(NttPassArgs A) {
   }
   for (uint32_t logNs = 0; logNs < logL; logNs++) {
     if (logNs > 0) {
-      // w_{2 Ns}^k = w_4096^(4 k'), k' = k 512 / Ns: the radix-8 table at stride 512, r = 4
-      const uint32_t k = t0 & ((1u << logNs) - 1);
       x0 = fr_reduce1(x0);
-      x1 = fr_mulc(A.dft.ld(stage_tab(9, 3) + 3 * 512 + (k << (9 - logNs))), x1);
+      x1 = fr_mulc(A.dft.ld(X.twiddle(logNs)), x1);
     }
     const fr y0 = fr_add_lazy(x0, x1), y1 = fr_sub_lazy(x0, x1);
     if (logNs + 1 == logL) {
@@ -458,9 +407,8 @@ __global__ void __launch_bounds__(512) k_ntt_pass_small(NttPassArgs A) {
       break;
     }
     const SmTile sm{sm_planes + (logNs & 1) * 4 * NT, 2 * NT};
-    const uint32_t ls = logNs + logW, q = ((tid >> ls) << (ls + 1)) + (tid & ((1u << ls) - 1));
-    sm.put(q, y0);
-    sm.put(q + (1u << ls), y1);
+    sm.put(X.exchange(logNs, 0), y0);
+    sm.put(X.exchange(logNs, 1), y1);
     __syncthreads();
     x0 = sm.get(tid);
     x1 = sm.get(tid + NT);
@@ -522,11 +470,6 @@ struct NttSizeArgs {
   const NttTables* T;
   const DevConst* C;
 };
-
-// coefficient k = L2 t + b at entry L1 b + t: the passes over t read consecutive entries
-__host__ __device__ __forceinline__ uint64_t tab_pos(uint64_t k, uint32_t l1, uint32_t l2) {
-  return ((k & ((1ull << l2) - 1)) << l1) + (k >> l2);
-}
 
 __global__ void k_ntt_size_tables(NttSizeArgs A, NttTables T) {
   const uint64_t N = 1ull << A.n, M = N << A.lb;
@@ -922,12 +865,11 @@ static zc_status ensure_tables(zc_ctx* ctx, cudaStream_t st, NttTables** out) {
 // resident CTAs per SM (caps registers).  The context's tuning picks the tile
 // and residency.
 template <int MAXT, int MINB>
-static void launch_pass_variant(const NttPassArgs& a, dim3 grid, uint32_t tile, cudaStream_t st) {
-  if (a.logL >= 3 && tile >= 512 && !(a.B & ((1u << a.logW) - 1)) && a.pre != PRE_COSET &&
-      (a.post == POST_NONE || a.post == POST_TAB))
-    k_ntt_pass<MAXT, MINB, true><<<grid, tile / 8, tile * sizeof(fr), st>>>(a);
+static void launch_pass_variant(const NttPassArgs& a, dim3 grid, const NttPlan& P, cudaStream_t st) {
+  if (ntt_fast(P, a.logL, a.B) && a.pre != PRE_COSET && (a.post == POST_NONE || a.post == POST_TAB))
+    k_ntt_pass<MAXT, MINB, true><<<grid, P.tile / 8, P.tile * sizeof(fr), st>>>(a);
   else
-    k_ntt_pass<MAXT, MINB, false><<<grid, tile / 8, tile * sizeof(fr), st>>>(a);
+    k_ntt_pass<MAXT, MINB, false><<<grid, P.tile / 8, P.tile * sizeof(fr), st>>>(a);
 }
 
 static void set_pass_attributes() {
@@ -968,39 +910,22 @@ static void set_dft(NttPassArgs& a, const NttTables* T, bool inverse) {
 // launch one batched pass over `items` columns
 static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int items, uint64_t B, uint32_t slices = 1) {
   const uint32_t logL = a.logL;
-  uint32_t logTile = (uint32_t)ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_TILE_LOG);
+  const uint32_t tile = (uint32_t)ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_TILE_LOG);
   const int minb = ctx->tuned(ZC_FORM_NTT, ctx->cur_n, ZC_TUNE_NTT_MINB);
-  // few elements, and no tile or residency asked for: two per thread, tiles of
-  // 256 (or one sub-DFT)
-  if (!logTile && !minb && logL >= 1 && logL <= 10 && (uint64_t)items * slices * (B << logL) <= kSmallElems &&
-      a.pre != PRE_COSET && (a.post == POST_NONE || a.post == POST_TAB)) {
-    const uint32_t lt = std::max<uint32_t>(logL, 8);
-    if ((B << logL) % (1ull << lt) == 0) {
-      a.logW = lt - logL;
-      a.items = (uint32_t)items;
-      a.B = (uint32_t)B;
-      const dim3 grid((uint32_t)((B >> a.logW) * (uint64_t)items), slices);
-      k_ntt_pass_small<<<grid, 1u << (lt - 1), 2 * sizeof(fr) << lt, st>>>(a);
-      ctx->launches++;
-      return ZC_OK;
-    }
-  }
-  if (logTile < logL) logTile = logL < 10 ? 10 : logL;
-  if (logTile > 12) logTile = 12;
-  if (logTile < 10) logTile = 10;
-  // a tile holds at least one warp's elements, sub-DFTs past the last included
-  a.logW = logTile - logL;
-  while (a.logW > 0 && a.logW + logL > 8 && (1ull << a.logW) > B) a.logW--;
-  const uint64_t W = 1ull << a.logW;
-  const uint64_t blocks = (B + W - 1) / W;
-  const uint32_t tile = 1u << (a.logW + logL);
+  NttPlan P;
+  // few elements, and no tile or residency asked for: two per thread
+  const bool small = !tile && !minb && (uint64_t)items * slices * (B << logL) <= kSmallElems && a.pre != PRE_COSET &&
+                     (a.post == POST_NONE || a.post == POST_TAB) && ntt_plan_small(logL, B, &P);
+  if (!small) P = ntt_plan(logL, B, tile);
+  a.logW = P.logW;
   a.items = (uint32_t)items;
   a.B = (uint32_t)B;
-  const dim3 grid((uint32_t)(blocks * (uint64_t)items), slices);
-  if (logTile == 12) launch_pass_variant<512, 1>(a, grid, tile, st);
-  else if (logTile == 11 && minb != 1) launch_pass_variant<256, 2>(a, grid, tile, st);
-  else if (logTile == 11) launch_pass_variant<256, 1>(a, grid, tile, st);
-  else launch_pass_variant<128, 4>(a, grid, tile, st);
+  const dim3 grid((uint32_t)(P.blocks * (uint64_t)items), slices);
+  if (small) k_ntt_pass_small<<<grid, P.tile / 2, 2 * P.tile * sizeof(fr), st>>>(a);
+  else if (P.logTile == 12) launch_pass_variant<512, 1>(a, grid, P, st);
+  else if (P.logTile == 11 && minb != 1) launch_pass_variant<256, 2>(a, grid, P, st);
+  else if (P.logTile == 11) launch_pass_variant<256, 1>(a, grid, P, st);
+  else launch_pass_variant<128, 4>(a, grid, P, st);
   ctx->launches++;
   return ZC_OK;
 }
@@ -1296,13 +1221,11 @@ zc_status pcs_encode(zc_ctx* ctx, const fr* const* cols, int c, uint32_t nr, uin
       a.in[j] = cols[j];
       a.out[j] = enc[j] + sl * m;     // position k = sl + 4 k'
     }
-    a.logL = nc;
-    a.im = map_flat(nc, 0);           // row b, coefficient t
-    a.om = map_flat(0, nr + 2);       // position 4 t
+    const NttMaps mp = maps_pcs(nr, nc);
+    a.use(mp);
     set_dft(a, T, false);
     a.pre = PRE_TAB; a.pre_tab = tab.at(sl * w);
-    a.pm = map_low(0, 0, 0);
-    zc_status rs = run_pass(ctx, st, a, c, m);
+    zc_status rs = run_pass(ctx, st, a, c, mp.B);
     if (rs != ZC_OK) return rs;
   }
   return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
@@ -1410,7 +1333,6 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
   const bool two = ntt_two_pass(ctx, n);
   const uint32_t l1 = two ? (n + 1) / 2 : n;   // first digit
   const uint32_t l2 = two ? n / 2 : 0;         // second digit
-  const uint64_t L1 = 1ull << l1, L2 = 1ull << l2;
   zc_status rs;
   zc_ctx::NttSizeTables* ST = size_tables(ctx, T, n, lb, l1, l2, D.step, st);
   if (D.step && (!ST || !step_tables(ctx, ST, T, st))) {
@@ -1427,18 +1349,16 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.in[j - j0] = in[j];
       a.out[j - j0] = coef[j];
     }
-    a.logL = l2;                       // rows of length L2 over i2
-    a.im = map_flat(0, l1);            // element (i1, i2) read from e[i1 + L1 i2]
-    a.om = map_flat(l2, 0);
+    const NttMaps mp = maps_n1_rows(l1, l2);
+    a.use(mp);
     set_dft(a, T, true);
     a.err = &dstate->err;              // every input element passes through here once
     a.post = POST_TW; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
     a.tw_lbmod = l1; a.tw_shift = kLog30 - n;
-    if (ST) {  // w_N^-(i1 k2) = tw_inv[i1 L2 + k2]
+    if (ST) {
       a.post = POST_TAB; a.post_tab = ST->tw_inv;
-      a.qm = map_flat(l2, 0);
     }
-    return run_pass(ctx, st, a, j1 - j0, L1);
+    return run_pass(ctx, st, a, j1 - j0, mp.B);
   };
   // N1's second pass (columns of length L1, in place) for the columns [j0, j1)
   auto n1_second = [&](int j0, int j1) -> zc_status {
@@ -1448,10 +1368,10 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.in[j - j0] = coef[j];
       a.out[j - j0] = coef[j];
     }
-    a.logL = l1;
-    a.im = a.om = map_flat(0, l2);
+    const NttMaps mp = maps_n1_cols(l1, l2);
+    a.use(mp);
     set_dft(a, T, true);
-    return run_pass(ctx, st, a, j1 - j0, L2);
+    return run_pass(ctx, st, a, j1 - j0, mp.B);
   };
 
   k_ntt_state_init<<<1, 32, 0, st>>>(dstate);
@@ -1527,8 +1447,7 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       a.in[j] = src[j];
       a.out[j] = coef[j];
     }
-    a.logL = n;
-    a.im = a.om = map_flat(0, 0);
+    a.use(maps_one(n));
     set_dft(a, T, true);
     a.err = &dstate->err;
     if ((rs = run_pass(ctx, st, a, c, 1)) != ZC_OK) return rs;
@@ -1555,30 +1474,29 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     a.pre_y = (uint32_t)N;
     set_dft(a, T, false);
     if (two) {
-      a.logL = l1;                     // columns over k1: k = L2 k1 + k2
-      a.im = a.om = a.pm = map_flat(0, l2);
+      const NttMaps mc = maps_n2_cols(l1, l2), mr = maps_n2_rows(l1, l2);
+      a.use(mc);
       a.post = POST_TW; a.tw_lo = T->wf_lo; a.tw_hi = T->wf_hi;
       a.tw_lbmod = l2; a.tw_shift = kLog30 - n;
-      if (ST) {  // coset factor of k = L2 k1 + k2 at L1 k2 + k1; twiddle w_N^(k2 i1) = tw_fwd[k2 L1 + i1]
-        a.pre = PRE_TAB; a.pre_tab = *pre; a.pm = map_flat(l1, 0);
+      if (ST) {
+        a.pre = PRE_TAB; a.pre_tab = *pre;
         a.post = POST_TAB; a.post_tab = ST->tw_fwd;
-        a.qm = map_flat(l1, 0);
+      } else {
+        a.pm = mc.km;
       }
-      if ((rs = run_pass(ctx, st, a, items, L2, sb)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, items, mc.B, sb)) != ZC_OK) return rs;
       if (mark) ZC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev[7], st));
       pass_defaults(a);
       for (int i = 0; i < items; i++) {
         a.in[i] = out[i];
         a.out[i] = out[i];
       }
-      a.logL = l2;                     // rows over k2
-      a.im = a.om = map_flat(l2, 0);
+      a.use(mr);
       a.in_y = a.out_y = (uint32_t)(c * Na);
       set_dft(a, T, false);
-      if ((rs = run_pass(ctx, st, a, items, L1, sb)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, items, mr.B, sb)) != ZC_OK) return rs;
     } else {
-      a.logL = n;
-      a.im = a.om = a.pm = map_flat(0, 0);
+      a.use(maps_one(n));
       if (ST) {
         a.pre = PRE_TAB; a.pre_tab = *pre;
       }
@@ -1619,49 +1537,45 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
     if (two) {
       pass_defaults(a);
       a.in[0] = qin; a.out[0] = qin;
-      a.logL = l2;                     // rows (j, i2) over i3
-      a.im = a.om = map_flat(l2, 0);
+      const NttMaps mr = maps_n3_rows(l1, l2, s), mc = maps_n3_cols(l1, l2, s);
+      a.use(mr);
       set_dft(a, T, true);
       a.post = POST_TW; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.tw_lbmod = l1; a.tw_shift = kLog30 - n;
-      if (ST) {  // w_N^-(i2 k3) = tw_inv[(b mod L1) L2 + k3]
+      if (ST) {
         a.post = POST_TAB; a.post_tab = ST->tw_inv;
-        a.qm = map_low(l1, l2, 0);
       }
-      if ((rs = run_pass(ctx, st, a, 1, s * L1)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, 1, mr.B)) != ZC_OK) return rs;
       pass_defaults(a);
       a.in[0] = qin; a.out[0] = qin;
-      a.logL = l1;                     // columns (j, k3) over i2 within a slice
-      a.im = a.om = map_split(l2, n, 0, l2);
+      a.use(mc);
       set_dft(a, T, true);
       a.post = POST_OUTER; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.outer_lbdiv = l2; a.tw_shift = kLog30 - logm;
-      if (ST) {  // w_M^-(j k') 7^-k', k' = L2 k2 + k3: outer[j N + L1 k3 + k2]
+      if (ST) {
         if (s == 1) a.out[0] = qout;  // no cross-slice stage
         a.post = POST_TAB; a.post_tab = ST->outer;
-        a.qm = map_split(l2, n, l1, 0);
       }
-      if ((rs = run_pass(ctx, st, a, 1, s * L2)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, 1, mc.B)) != ZC_OK) return rs;
     } else {
       pass_defaults(a);
       a.in[0] = qin; a.out[0] = qin;
-      a.logL = n;                      // one row per slice
-      a.im = a.om = map_flat(n, 0);
+      const NttMaps mp = maps_n3_one(n, s);
+      a.use(mp);
       set_dft(a, T, true);
       a.post = POST_OUTER; a.tw_lo = T->wi_lo; a.tw_hi = T->wi_hi;
       a.outer_lbdiv = 0; a.tw_shift = kLog30 - logm;
       if (ST) {
         if (s == 1) a.out[0] = qout;
         a.post = POST_TAB; a.post_tab = ST->outer;
-        a.qm = map_flat(n, 0);
       }
-      if ((rs = run_pass(ctx, st, a, 1, s)) != ZC_OK) return rs;
+      if ((rs = run_pass(ctx, st, a, 1, mp.B)) != ZC_OK) return rs;
     }
     if (ST && s == 1) return ZC_OK;
     pass_defaults(a);
     a.in[0] = qin; a.out[0] = qout;
-    a.logL = lb;                       // across slices
-    a.im = a.om = map_flat(0, n);
+    const NttMaps ms = maps_n3_slices(n, lb);
+    a.use(ms);
     set_dft(a, T, true);
     a.post = POST_FINAL; a.tw_lo = T->s7_lo; a.tw_hi = T->s7_hi;
     a.fin_logN = n;
@@ -1675,11 +1589,10 @@ zc_status ntt_prove(zc_ctx* ctx, const zc_params* p, const void* const* cols, in
       ctx->launches++;
       return ZC_OK;
     }
-    if (ST) {  // 7^-(N t)
+    if (ST) {
       a.post = POST_TAB; a.post_tab = ST->fin;
-      a.qm = map_low(0, 0, 0);
     }
-    if ((rs = run_pass(ctx, st, a, 1, N)) != ZC_OK) return rs;
+    if ((rs = run_pass(ctx, st, a, 1, ms.B)) != ZC_OK) return rs;
   }
     return ZC_OK;
   };
