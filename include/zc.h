@@ -367,7 +367,10 @@ zc_status zc_sumcheck_point(const zc_params* params, zc_form form, const uint8_t
  * zc_prove_sumcheck / zc_prove_ntt returns for the same request.
  *
  * Scratch bytes one proof takes (device columns, roots computed on the
- * device; q_on_device: the NTT quotient goes to a caller buffer). */
+ * device; q_on_device: the NTT quotient goes to a caller buffer).  A context
+ * that allocates its scratch for a small NTT proof takes up to about 40 MB more
+ * where mem_budget_bytes allows it, and several slices then share a launch;
+ * with the reported bytes alone the proof is the same and slower. */
 zc_status zc_scratch_bytes(zc_ctx* ctx, const zc_params* params, zc_form form, int q_on_device,
                            size_t* bytes);
 

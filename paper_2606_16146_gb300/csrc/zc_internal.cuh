@@ -46,7 +46,7 @@ struct ScState {        // SumCheck per-proof device state
   fr r1inv[kMaxN];       // 1/(1 - r_i) (level 1), or 0
   uint32_t p0[kMaxN];    // the finite point computed besides 2..d-1: 0 or 1
   fr alpha[kMaxN];       // challenges, level 1
-  frc alphac[kMaxN];     // ... as constant multipliers (not kept inside the persistent and tail rounds)
+  frc alphac[kMaxN];     // ... as constant multipliers (not in the tail; of the cooperative kernels only the product rounds read it)
   fr claim;              // H_{i-1}(alpha_{i-1}), level 0
   fr ci;                 // prod_{j<i} eq(alpha_j, r_j), level 1
   uint32_t counter[kMaxN];  // CTAs that finished round i (last one runs the challenge)

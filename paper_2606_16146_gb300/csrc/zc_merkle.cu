@@ -6,9 +6,10 @@
 // leaf t = SHA-256 of the canonical bytes of v[64 t .. min(64 t + 63, L-1)]
 // (the last leaf is shorter when 64 does not divide L), node =
 // SHA-256(left | right), and at a level with an odd count the last node
-// moves up unchanged; root = SHA-256(le64(len) | top).  One thread hashes
-// one 2 KB leaf; a CTA reduces its 128 (or 32) leaves to one node in shared
-// memory; a second kernel reduces the CTA nodes of each column.  The CTAs' leaf
+// moves up unchanged; root = SHA-256(le64(len) | top).  A 2 KB leaf is hashed by
+// one lane of two warps (see k_root_leaves); a CTA reduces its 128 (or 32)
+// leaves to one node in shared memory; a second kernel reduces the CTA nodes of
+// each column.  The CTAs' leaf
 // ranges start at multiples of 128 (32), so their subtrees are the global
 // tree's first seven (five) levels (a ragged last CTA's node arrives at that
 // level unchanged, as the odd last node of every level above it).

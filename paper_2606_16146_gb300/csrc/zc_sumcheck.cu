@@ -1586,8 +1586,9 @@ static zc_status sc_enqueue(const zc_params* p, const ScPlan& P, const fr* const
   const uint32_t inv_cta = need_inv ? 1u : 0u;
   for (; i < n; i++) {
     const uint64_t h = N >> (i + 1);
-    // the Plonk tail starts at round 2 at the earliest: round 1 always runs the
-    // pair kernel, so the tail carries no round-1 code (fewer registers)
+    // the Plonk tail starts at round 2 at the earliest: round 1 runs in the pair
+    // kernel or the cooperative one, so the tail carries no round-1 code (fewer
+    // registers)
     if (h <= tail_pairs && !(plonk && i == 0)) break;
     R.round = (int)i;
     R.h = h;
