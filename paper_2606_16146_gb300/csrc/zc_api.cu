@@ -82,7 +82,6 @@ zc_status ensure_arena(zc_ctx* ctx, size_t bytes) {
     return ZC_ERR_OOM;
   }
   if (ctx->arena.base) {
-    cudaDeviceSynchronize();
     ctx->arena_own.reset();
     ctx->arena.base = nullptr;
     ctx->arena.cap = 0;
@@ -95,7 +94,7 @@ zc_status ensure_arena(zc_ctx* ctx, size_t bytes) {
     ctx->err = std::string("cudaMalloc scratch: ") + cudaGetErrorString(e);
     return ZC_ERR_OOM;
   }
-  ctx->arena_own = std::shared_ptr<void>(p, [](void* q) { cudaFree(q); });
+  ctx->arena_own = std::shared_ptr<void>(p, device_free);
   ctx->arena.base = static_cast<char*>(p);
   ctx->arena.cap = want;
   ctx->arena.used = 0;

@@ -106,6 +106,13 @@ struct Arena {
   }
 };
 
+// Frees memory that launches of any stream (lanes, batch graphs) may still use.
+inline void device_free(void* p) {
+  if (!p) return;
+  cudaDeviceSynchronize();
+  cudaFree(p);
+}
+
 }  // namespace zc
 
 struct zc_ctx {
@@ -149,8 +156,8 @@ struct zc_ctx {
     NttTableMem(const NttTableMem&) = delete;
     NttTableMem& operator=(const NttTableMem&) = delete;
     ~NttTableMem() {
-      if (mem) cudaFree(mem);
-      if (step_mem) cudaFree(step_mem);
+      zc::device_free(mem);
+      zc::device_free(step_mem);
     }
   };
   struct NttSizeTables {

@@ -934,7 +934,7 @@ static zc_status run_pass(zc_ctx* ctx, cudaStream_t st, NttPassArgs& a, int item
 // recently used sizes go, but never one that a captured batch graph or a set
 // being prepared holds.  False when that leaves too little (must: what can go
 // goes, and the budget is passed by the rest).
-static bool table_room(zc_ctx* ctx, size_t bytes, bool must, cudaStream_t st) {
+static bool table_room(zc_ctx* ctx, size_t bytes, bool must) {
   size_t used = 0, held = 0;
   for (auto& e : ctx->ntt_cache) {
     used += e.bytes + e.step_bytes;
@@ -948,7 +948,6 @@ static bool table_room(zc_ctx* ctx, size_t bytes, bool must, cudaStream_t st) {
           (old == SIZE_MAX || ctx->ntt_cache[i].stamp < ctx->ntt_cache[old].stamp))
         old = i;
     if (old == SIZE_MAX) break;
-    cudaStreamSynchronize(st);
     used -= ctx->ntt_cache[old].bytes + ctx->ntt_cache[old].step_bytes;
     ctx->ntt_cache.erase(ctx->ntt_cache.begin() + old);
   }
@@ -970,7 +969,7 @@ static zc_ctx::NttSizeTables* size_tables(zc_ctx* user, const NttTables* T, uint
   const uint64_t s = 1ull << lb;
   const size_t bytes = sizeof(frc) * (2 * N + 2 * M + 2 * s);
   if (ctx->ntt_cache_frozen || bytes > ctx->ntt_cache_budget) return nullptr;
-  if (!table_room(ctx, bytes, step, st)) return nullptr;  // a step-radix domain has no other route
+  if (!table_room(ctx, bytes, step)) return nullptr;  // a step-radix domain has no other route
   zc_ctx::NttSizeTables e;
   e.own = std::make_shared<zc_ctx::NttTableMem>();
   if (cudaMalloc(&e.own->mem, bytes) != cudaSuccess) {
@@ -1108,7 +1107,7 @@ static bool step_tables(zc_ctx* user, zc_ctx::NttSizeTables*& e, const NttTables
   if (ctx->ntt_cache_frozen) return false;
   // room for them too, with this entry held; e moves as others go
   const std::shared_ptr<zc_ctx::NttTableMem> own = e->own;
-  table_room(ctx, step_table_bytes(e->n, e->lb), true, st);
+  table_room(ctx, step_table_bytes(e->n, e->lb), true);
   for (auto& t : ctx->ntt_cache)
     if (t.own == own) e = &t;
   const uint32_t n = e->n, lb = e->lb;
