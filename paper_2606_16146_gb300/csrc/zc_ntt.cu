@@ -214,11 +214,11 @@ struct SmTile {
 // table before the store) go through one copy of the code.
 //
 // What bounds it: the wide multiply-adds of the ~6 products per element (the
-// multiplier pipe is 77 % busy in the first N2 pass at n = 20, 699 us; reading
+// multiplier pipe is 79 % busy in the first N2 pass at n = 20, 670 us; reading
 // elements and factors one per lane it was 67 %, 769 us), then the latency of
 // 16 warps per SM.  Why the pass looks as it does: 32- and 64-byte elements
 // read one per lane made every request touch 16 to 32 lines (L1 75 % busy, now
-// 22 %), so columns move in 16-byte halves, two lanes to an element, and
+// 21 %), so columns move in 16-byte halves, two lanes to an element, and
 // factors lie in 16-byte planes in the order the lanes read them; products
 // inlined at each use were 75 KB of instructions, more than the instruction
 // cache keeps, hence the shared step; address arithmetic competes for the
